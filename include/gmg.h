@@ -93,7 +93,7 @@ typedef struct {
     int coarse_sweeps; /* red-black sweeps from zero on a coarsest grid with more than
                           one unknown (truncated hierarchy); unused otherwise */
     int transfer;      /* gmg_transfer.  GMG_MCGS and GMG_TRANSFER_PAPER run in the plain
-                          FP64 form (V-cycles or FMG), every level on grid kernels */
+                          FP64 form (V-cycles or FMG) */
 } gmg_config;
 
 typedef struct gmg_handle_s* gmg_handle;

@@ -483,7 +483,6 @@ template <typename T>
 int tail_level(gmg_handle h, const std::vector<Level<T>>& lv) {
     const gmg_config& c = h->cfg;
     const int L = (int)lv.size();
-    if (c.smoother == GMG_MCGS || c.transfer == GMG_TRANSFER_PAPER) return L;  // grid kernels
     const int nmax = h->tail_max > 0 ? h->tail_max : c.d != 3 ? 32 : 8;
     int lo = 0;
     if (c.smoother == GMG_LEARNED)
@@ -578,7 +577,8 @@ gmg_status enqueue_vcycle(gmg_handle h, std::vector<Level<T>>& lv, bool first_re
         cudaError_t e = cudaSuccess;
         timed(h, K_TAIL, 0, p, lv[0].n, false, [&] {
             e = tail::launch<T>(d, lv[0].lay, L, lv[0].u[0], lv[0].q, c.smoother, c.omega, c.nu1,
-                                c.nu2, c.coarse_sweeps, h->stream, true);
+                                c.nu2, c.coarse_sweeps, h->stream, true,
+                                c.transfer == GMG_TRANSFER_PAPER);
         });
         GMG_CUDA_TRY(e);
     } else if (L == 1) {
@@ -650,7 +650,8 @@ gmg_status enqueue_vcycle(gmg_handle h, std::vector<Level<T>>& lv, bool first_re
             cudaError_t e = cudaSuccess;
             timed(h, K_TAIL, lt, p, lv[lt].n, false, [&] {
                 e = tail::launch<T>(d, lv[lt].lay, L - lt, lv[lt].u[0], lv[lt].q, c.smoother,
-                                    c.omega, c.nu1, c.nu2, c.coarse_sweeps, h->stream);
+                                    c.omega, c.nu1, c.nu2, c.coarse_sweeps, h->stream, false,
+                                    c.transfer == GMG_TRANSFER_PAPER);
             });
             GMG_CUDA_TRY(e);
         } else {

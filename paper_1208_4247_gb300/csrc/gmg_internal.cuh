@@ -228,10 +228,11 @@ size_t smem_bytes(int d, int n_top, int levels, int smoother, size_t elem);
 // exact_top: the top level is level 0 of a plain FP64 3D hierarchy, whose
 // last pre-smoothing half sweep and residual use the unbiased value
 // (level_kernels.cuh, gs_value), as the grid kernels there do
+// paper: the paper's transfers (FP64); the paper's smoother runs too (FP64)
 template <typename T>
 cudaError_t launch(int d, const Lay& top, int levels, T* u_top, const T* q_top, int smoother,
                    double omega, int nu1, int nu2, int coarse_sweeps, cudaStream_t s,
-                   bool exact_top = false);
+                   bool exact_top = false, bool paper = false);
 // The same on the levels' own dense arrays (n[l], u[l], q[l], r[l] for the
 // `levels` levels from the first one down), one cooperative launch of
 // `blocks` CTAs (grid_blocks: one wave; 0 when the device cannot) with grid
