@@ -294,21 +294,22 @@ gmg_status gmg_learned_train(int d, int n, int steps, int batch, int pair_cycles
 
 /* ------------------------------------------------------------ FFT solve
  * The paper's comparison method (section 2.3): a direct solve of the same FD
- * system A'u = h^2 f by sine transforms, u = S^-1 diag(1/lambda) S h^2 f with
- * S the DST-I along every axis and lambda_k = sum_m 4 sin^2(pi k_m / (2n))
- * the discrete eigenvalues (the paper writes the continuous symbol), each
- * DST-I done by a length-2n cuFFT D2Z of the odd extension. */
+ * system A'u = h^2 f by sine transforms (DST-I) with the discrete eigenvalues
+ * 4 sin^2(pi k_m / (2n)) (the paper writes the continuous symbol).  The
+ * first d-1 axes are transformed, the tridiagonal systems this leaves along
+ * the last one eliminated, and the transforms applied back: the solution of
+ * the system to rounding, as with a transform of every axis. */
 typedef struct gmg_fft_s* gmg_fft;
 
 /* d = 2 or 3, n a power of two (2D up to 8192, 3D up to 1024); allocates
- * about 3 (n+1)^d doubles of work space and two cuFFT plans. */
+ * about 1.5 n^d doubles: work space and the eliminations' coefficients. */
 gmg_status gmg_fft_create(int d, int n, void* cuda_stream, gmg_fft* out);
 /* Section 2.3: u = A'^-1 h^2 f on the interior, 0 on the boundary (f, u
  * device pointers, layout above).  Synchronises the handle's stream.
  * Errors: GMG_ERR_ARG for NULL arguments, GMG_ERR_CUDA for a failed
  * transform or launch. */
 gmg_status gmg_fft_solve(gmg_fft h, const double* f, double* u);
-/* Release the plans and work space of h.  NULL is a no-op. */
+/* Release the tables and work space of h.  NULL is a no-op. */
 gmg_status gmg_fft_destroy(gmg_fft h);
 
 /* ---------------------------------------------------------------- batches

@@ -68,7 +68,7 @@ def build(force: bool = False, verbose: bool = False, extra=()) -> str:
             if lg.strip():
                 print(os.path.basename(s), lg)
     tmp = LIB + f".tmp{os.getpid()}"
-    cmd = [nvcc(), "-shared", *ARCH, "-o", tmp, *objs, "-lcufft", "-lcudart"]
+    cmd = [nvcc(), "-shared", *ARCH, "-o", tmp, *objs, "-lcudart"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")

@@ -1,18 +1,32 @@
-// Direct FFT Poisson solve (the paper's comparison method, section 2.3):
-// the FD system A'u = h^2 f is diagonal in the sine basis, so
-//     u = S^-1 diag(1 / lambda) S (h^2 f),   S = DST-I along every axis,
-//     lambda_k = sum_m 4 sin^2(pi k_m / (2n)),  S^-1 = (2/n)^d S.
+// Direct solve of the FD system by sine transforms (the paper's comparison
+// method, section 2.3).  A'u = h^2 f is diagonal in the sine basis along
+// every axis; here the first d-1 axes are transformed (DST-I), which leaves
+// one tridiagonal system per line of the last axis,
+//     -v_{k-1} + (2 + lambda) v_k - v_{k+1} = h^2 fhat_k,
+//     lambda = sum over the transformed axes of 4 sin^2(pi k_m / (2n)),
+// solved by elimination, and the same transforms back: S^-1 = (2/n) S.
 // (The paper divides by the continuous symbol k_x^2 + k_y^2; the discrete
 // eigenvalues make the result the exact solution of the same FD system the
-// multigrid solves.)  Each DST-I of length n-1 is a length-2n real-to-complex
-// cuFFT of the odd extension [0, x, 0, -reverse(x)]: its k-th coefficient is
-// -2i y_k.  Lines along x use a line-major extension; lines along y and z an
-// element-major one (cuFFT strided layout), so every gather and scatter
-// kernel reads and writes contiguous x.
-#include <cufft.h>
-
+// multigrid solves.)  The work array holds nodes 0..n-1 of each transformed
+// axis, row pitch n, so that a tile of 16 columns is one 128-byte segment.
+//
+// What bounds the solve on GB300 is the FP64 pipe (0.505 T adds/s measured,
+// against 6.8 TB/s of HBM: at 16 bytes a node and pass, 6 instructions cost as
+// much as the traffic).  So the transforms are built for few FP64 operations:
+// two real lines share one complex line, and a DST-I of length n - 1 is folded
+// into DST-IIIs of sizes n/2, n/4, .., 1, each a complex FFT of its own size
+// (about 14 instructions per value at n = 256; a complex FFT of the odd
+// extension, length 2n, takes about 35, the real one of length 2n that a
+// library offers the same again in gathers and scatters).  The elimination
+// along the last axis takes 3 where the two transforms and the division by
+// the eigenvalues would take about 30.
+// 3D 257^3: 14.94 ms with length-2n library transforms of the odd extension
+// on all three axes, 2.16 ms with these kernels (0.50 ms a
+// transform of one axis at 84% of the FP64 pipe, 0.13 ms the eliminations).
+#include <algorithm>
 #include <cmath>
 #include <string>
+#include <vector>
 
 #include "gmg_internal.cuh"
 
@@ -20,95 +34,504 @@ namespace gmg {
 namespace fft {
 namespace {
 
-// axis 0 (x): ext[line][j], line = (k-1)(n-1) + (j'-1);
-// axes 1, 2: ext[j][line], line = (other-1)(n-1) + (i-1)
-__device__ inline int64_t node(int d, int n, int axis, int64_t line, int j) {
-    const int64_t m = n + 1;
-    const int a = (int)(line % (n - 1)) + 1;
-    const int b = d == 3 ? (int)(line / (n - 1)) + 1 : 0;
-    if (axis == 0) return ((int64_t)b * m + a) * m + j;    // a = y, b = z
-    if (axis == 1) return ((int64_t)b * m + j) * m + a;    // a = x, b = z
-    return ((int64_t)j * m + b) * m + a;                    // axis 2: a = x, b = y
-}
-
-__global__ void k_extend(const double* __restrict__ x, double* __restrict__ ext, int d, int n,
-                         int axis, int64_t lines) {
-    const int L = 2 * n;
-    const int64_t total = lines * L;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        int64_t line;
-        int j;
-        if (axis == 0) {
-            line = t / L;
-            j = (int)(t % L);
-        } else {
-            j = (int)(t / lines);
-            line = t % lines;
-        }
-        double v = 0.0;
-        if (j > 0 && j < n)
-            v = x[node(d, n, axis, line, j)];
-        else if (j > n)
-            v = -x[node(d, n, axis, line, L - j)];
-        ext[t] = v;
+// ------------------------------------------------------------ DST-I of lines
+//
+// Positions 1..n-1 of a line hold x_1..x_{n-1} (complex: two real lines).
+// Folding x_j, x_{r-j} (r = n, n/2, .., 4) into the difference at j and the sum
+// at r - j leaves at positions M .. 2M-1 (M = r/2) the input c_0 .. c_{M-1} of
+// a DCT-III of size M whose values are, up to the sign (-1)^k, the
+// coefficients y_{(n/2M)(2k+1)} (sin(pi (M-j)(2k+1)/2M) = (-1)^k cos(pi j
+// (2k+1)/2M)).  The DCT-III by one complex FFT of size M (Makhoul 1980, "A
+// fast cosine transform in one and two dimensions"):
+//     V_j = e^{i pi j/2M} (c_j - i c_{M-j}) / 2,  V_0 = c_0,
+//     v = sum_j V_j e^{2 pi i jm/M},  C_{2m} = v_m, C_{2m+1} = v_{M-1-m}.
+// The kernels form 2 V_j, hence twice the DST: the powers of two go into the
+// scale of the line solves, exactly.
+// Everything stays in place in shared memory: the FFTs are
+// decimation-in-frequency radix-8 stages (the last one 8, 4 or 2) that leave
+// their output digit-reversed, which the final gather undoes.
+//
+// A CTA takes a tile of 2^lgP pairs of lines with n/8 threads per pair (one
+// radix-8 butterfly each and stage; 32 to 512 threads in all).  The tasks of a
+// step are numbered with the pair fastest and dealt to the threads one loop
+// after the other, so that the small folds and blocks, which would leave most
+// of a warp idle if every pair kept its own warp, fill warps across pairs: an
+// FP64 instruction costs its 64 cycles of a sub-core whatever lanes are on
+// (257^3, one pass over an axis: 697 -> 500 us).
+// Position p of a line sits at entry p + p/8 and a line's entries are an odd
+// number apart: neither butterflies whose legs are 8, 4 or 2 apart nor the
+// pairs of a tile meet in a bank.
+struct Plan {
+    int lg, lgP, threads;
+    __host__ __device__ int n() const { return 1 << lg; }
+    __host__ __device__ int pairs() const { return 1 << lgP; }
+    __host__ __device__ int stride() const { return ((1 << lg) + ((1 << lg) >> 3)) | 1; }
+    size_t smem() const { return sizeof(double2) * (size_t)pairs() * stride(); }
+};
+// total: pairs of lines of a transform.  Tiles of 256 threads (512 from n =
+// 512 up: 8 pairs of columns there are 128-byte segments along x) where there
+// are enough of them for two per SM, smaller ones (one warp at least) else.
+Plan plan_of(int n, int64_t total) {
+    Plan p;
+    p.lg = 0;
+    while ((1 << p.lg) < n) ++p.lg;
+    const int lgG = std::min(9, std::max(1, p.lg - 3));  // log2 threads per pair
+    p.lgP = (n >= 512 ? 9 : 8) - lgG;
+    p.threads = 1 << (lgG + p.lgP);
+    while (p.lgP > 0 && lgG + p.lgP > 5 && total >> p.lgP < 2 * 152) {
+        --p.lgP;
+        p.threads = std::max(p.threads / 2, 128);
     }
+    return p;
 }
 
-// y_k = -Im(X_k) / 2 for k = 1..n-1, times scale (and, with eig, divided by
-// lambda at the node: the diagonal solve fused into the last forward pass)
-__global__ void k_extract(const cufftDoubleComplex* __restrict__ X, double* __restrict__ y, int d,
-                          int n, int axis, int64_t lines, double scale, int eig) {
-    const int C = n + 1;
-    const int64_t total = lines * (n - 1);
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        int64_t line;
-        int k;
-        int64_t src;
-        if (axis == 0) {
-            line = t / (n - 1);
-            k = (int)(t % (n - 1)) + 1;
-            src = line * C + k;
-        } else {
-            k = (int)(t / lines) + 1;
-            line = t % lines;
-            src = (int64_t)k * lines + line;
-        }
-        const int64_t p = node(d, n, axis, line, k);
-        double v = -0.5 * X[src].y * scale;
-        if (eig) {
-            const int64_t m = n + 1;
-            const int i = (int)(p % m), jj = (int)((p / m) % m), kk = (int)(p / (m * m));
-            double lam = 0.0;
-            const double w = M_PI / (2.0 * n);
-            double s = sin(w * i);
-            lam += 4.0 * s * s;
-            s = sin(w * jj);
-            lam += 4.0 * s * s;
-            if (d == 3) {
-                s = sin(w * kk);
-                lam += 4.0 * s * s;
+__device__ inline double2 operator+(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ inline double2 operator-(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ inline double2 times_i(double2 a) { return make_double2(-a.y, a.x); }
+__device__ inline double2 cmul(double2 a, double2 w) {
+    return make_double2(fma(a.x, w.x, -(a.y * w.y)), fma(a.x, w.y, a.y * w.x));
+}
+// r + s * v
+__device__ inline double2 axpy(double s, double2 v, double2 r) {
+    return make_double2(fma(s, v.x, r.x), fma(s, v.y, r.y));
+}
+__device__ inline int at(int p) { return p + (p >> 3); }
+
+__device__ inline void dft4(double2& a, double2& b, double2& c, double2& d) {
+    const double2 s = a + c, t = a - c, u = b + d, v = times_i(b - d);
+    a = s + u;
+    b = t + v;
+    c = s - u;
+    d = t - v;
+}
+// x[p] <- sum_q x[q] e^{2 pi i p q / 8}: 52 instructions (the rotations by pi/4
+// are scaled in the last sums)
+__device__ inline void dft8(double2 (&x)[8]) {
+    const double h = 0.70710678118654752440;  // sqrt(1/2)
+    double2 e0 = x[0] + x[4], e1 = x[1] + x[5], e2 = x[2] + x[6], e3 = x[3] + x[7];
+    const double2 o0 = x[0] - x[4], o1 = x[1] - x[5], o2 = times_i(x[2] - x[6]), o3 = x[3] - x[7];
+    dft4(e0, e1, e2, e3);
+    // o1 e^{i pi/4} = h r1, o3 e^{3 i pi/4} = h r3
+    const double2 r1 = make_double2(o1.x - o1.y, o1.x + o1.y);
+    const double2 r3 = make_double2(-o3.x - o3.y, o3.x - o3.y);
+    const double2 s = o0 + o2, t = o0 - o2, u = r1 + r3, v = times_i(r1 - r3);
+    x[0] = e0;
+    x[2] = e1;
+    x[4] = e2;
+    x[6] = e3;
+    x[1] = axpy(h, u, s);
+    x[3] = axpy(h, v, t);
+    x[5] = axpy(-h, u, s);
+    x[7] = axpy(-h, v, t);
+}
+
+// The transform of the tile's pairs of lines (positions 1..n-1 of pair v at
+// entries at(p) of sm + v * stride, the first fold done and visible) by the
+// whole CTA; ends with a barrier.  T[k] = e^{i pi k/n}, k < 2n.
+__device__ void dst_tile(double2* __restrict__ sm, const Plan& P, const double2* __restrict__ T) {
+    const int lg = P.lg, n = 1 << lg, nt = blockDim.x, stride = P.stride();
+    int cursor = 0;  // the thread that takes the next loop's first task
+    auto tasks = [&](int w0, int w1, auto&& f) {
+        const int total = (w1 - w0) << P.lgP;
+        for (int id = ((int)threadIdx.x - cursor) & (nt - 1); id < total; id += nt)
+            f(sm + (id & (P.pairs() - 1)) * stride, w0 + (id >> P.lgP));
+        cursor = (cursor + ((total + 31) & ~31)) & (nt - 1);
+    };
+    // folds r = n/2, n/4, .., 4, two at a time: the orbit of j under both
+    for (int r = n / 2; r >= 4; r /= 4) {
+        const int h = r / 2;
+        tasks(1, r / 4 + 1, [&](double2* s, int j) {
+            const double2 a = s[at(j)], b = s[at(r - j)];
+            if (j == r / 4) {  // h - j = j: the inner fold leaves its middle
+                s[at(j)] = a - b;
+                s[at(r - j)] = a + b;
+            } else {
+                const double2 c = s[at(h - j)], d = s[at(h + j)];
+                const double2 e = a - b, f = c - d;
+                s[at(r - j)] = a + b;
+                s[at(h + j)] = c + d;
+                s[at(j)] = e - f;
+                s[at(h - j)] = e + f;
             }
-            v /= lam;
+        });
+        __syncthreads();
+    }
+    // 2 V_j, 2 V_{M-j} in each block M = 2 .. n/2; the pair index w = M/2 + j runs
+    // over all blocks (j = 0 of block M: V_0 and the middle element, M/2)
+    tasks(0, 1, [&](double2* s, int) {  // the block of size 1
+        s[at(1)].x *= 2.0;
+        s[at(1)].y *= 2.0;
+    });
+    tasks(1, n / 2, [&](double2* s, int w) {
+        const int l2 = 31 - __clz(w), m2 = 1 << l2;  // M/2
+        const int j = w - m2, M = 2 * m2;
+        if (j == 0) {
+            const int p = at(M + m2), p0 = at(M);
+            s[p].x *= 1.41421356237309504880;
+            s[p].y *= 1.41421356237309504880;
+            s[p0].x *= 2.0;
+            s[p0].y *= 2.0;
+        } else {
+            const int p = at(M + j), q = at(2 * M - j);
+            const double2 a = s[p], b = times_i(s[q]);
+            const double2 t = T[j << (lg - 2 - l2)];
+            s[p] = cmul(a - b, t);
+            s[q] = cmul(a + b, make_double2(t.x, -t.y));
         }
-        y[p] = v;
+    });
+    __syncthreads();
+    // radix-8 stages: sub-block length L = M, M/8, ..; butterfly index w over
+    // all blocks with L >= 8 (block M holds w = M/8 .. M/4 - 1)
+    for (int sh = 0; (n / 2 >> sh) >= 2; sh += 3) {  // L = M >> sh
+        if (1 << sh < n / 8)
+            tasks(1 << sh, n / 8, [&](double2* s, int w) {
+                const int lm = 31 - __clz(w);
+                const int M = 8 << lm, t = w - (1 << lm);
+                const int L = M >> sh, sub = L >> 3;
+                const int k = t & (sub - 1);
+                const int p0 = M + (t - k) * 8 + k;
+                double2 x[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) x[q] = s[at(p0 + q * sub)];
+                dft8(x);
+                if (sub > 1) {
+                    const int st = (2 * n / L) * k;  // e^{2 pi i k/L} = T[st]
+#pragma unroll
+                    for (int q = 1; q < 8; ++q) x[q] = cmul(x[q], T[st * q]);
+                }
+#pragma unroll
+                for (int q = 0; q < 8; ++q) s[at(p0 + q * sub)] = x[q];
+            });
+        // the blocks whose sub-block length is now 4 or 2
+        const int M4 = 4 << sh, M2 = 2 << sh;
+        if (M4 <= n / 2)
+            tasks(0, M4 / 4, [&](double2* s, int t) {
+                double2* x = s + at(M4 + 4 * t);  // four entries of one group of 8
+                double2 a = x[0], b = x[1], c = x[2], d = x[3];
+                dft4(a, b, c, d);
+                x[0] = a;
+                x[1] = b;
+                x[2] = c;
+                x[3] = d;
+            });
+        if (M2 <= n / 2)
+            tasks(0, M2 / 2, [&](double2* s, int t) {
+                double2* x = s + at(M2 + 2 * t);
+                const double2 a = x[0], b = x[1];
+                x[0] = a + b;
+                x[1] = a - b;
+            });
+        __syncthreads();
     }
 }
 
-__global__ void k_scale_rhs(const double* __restrict__ f, double* __restrict__ b, int d, int n) {
-    const int64_t m = n + 1;
-    const int64_t total = d == 3 ? m * m * m : m * m;
-    const double h2 = 1.0 / ((double)n * n);
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < total;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(p % m), j = (int)((p / m) % m), k = d == 3 ? (int)(p / (m * m)) : 1;
-        const bool in = i > 0 && i < n && j > 0 && j < n && k > 0 && k < (d == 3 ? n : 2);
-        b[p] = in ? h2 * f[p] : 0.0;
+// Entry of coefficient K (1..n-1) of a transformed line, and its sign.
+__device__ inline int coeff_at(int K, int lg, bool& minus) {
+    const int r = __ffs(K) - 1;
+    const int lm = lg - 1 - r;  // log2 M
+    const int k = K >> (r + 1);
+    minus = k & 1;
+    int m = minus ? (1 << lm) - 1 - (k >> 1) : k >> 1;
+    int pos = 0, left = lm;
+    while (left > 0) {  // digits from the first stage on
+        const int b = left >= 3 ? 3 : left;
+        left -= b;
+        pos += (m & ((1 << b) - 1)) << left;
+        m >>= b;
+    }
+    return at((1 << lm) + pos);
+}
+
+// DST-I along x of every interior row of src into dst (element (i, j, k) at
+// k*sz + j*sy + i).  whole_u: dst is u, whose boundary nodes are set to 0 too
+// (the rows' ends here, the boundary rows dealt over the CTAs).
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_dst_x(const double* __restrict__ src, int64_t ssy,
+                                                   int64_t ssz, double* __restrict__ dst,
+                                                   int64_t dsy, int64_t dsz, int64_t lines, int d,
+                                                   Plan P, int whole_u,
+                                                   const double2* __restrict__ T) {
+    extern __shared__ double2 sm[];
+    const int lg = P.lg, n = P.n();
+    // loading and storing: the threads of a pair along x
+    const int lgG = 31 - __clz(blockDim.x) - P.lgP, G = 1 << lgG;
+    const int g = threadIdx.x & (G - 1), pair = threadIdx.x >> lgG;
+    double2* s = sm + pair * P.stride();
+    const int64_t la = 2 * ((int64_t)blockIdx.x * P.pairs() + pair), lb = la + 1;
+    auto row = [&](int64_t l, int64_t sy, int64_t sz) {
+        const int64_t k = l / (n - 1);
+        return (l - k * (n - 1) + 1) * sy + (k + 1) * sz;  // sz = 0 in 2D
+    };
+    const bool ina = la < lines, inb = lb < lines;
+    const double* pa = src + (ina ? row(la, ssy, ssz) : 0);
+    const double* pb = src + (inb ? row(lb, ssy, ssz) : 0);
+#pragma unroll 4
+    for (int j = 1 + g; j < n / 2; j += G) {
+        const double2 a = make_double2(ina ? pa[j] : 0.0, inb ? pb[j] : 0.0);
+        const double2 b = make_double2(ina ? pa[n - j] : 0.0, inb ? pb[n - j] : 0.0);
+        s[at(j)] = a - b;
+        s[at(n - j)] = a + b;
+    }
+    if (g == 0) s[at(n / 2)] = make_double2(ina ? pa[n / 2] : 0.0, inb ? pb[n / 2] : 0.0);
+    __syncthreads();
+    dst_tile(sm, P, T);
+    double* qa = dst + (ina ? row(la, dsy, dsz) : 0);
+    double* qb = dst + (inb ? row(lb, dsy, dsz) : 0);
+    for (int K = 1 + g; K < n; K += G) {
+        bool minus;
+        const double2 v = s[coeff_at(K, lg, minus)];
+        if (ina) qa[K] = minus ? -v.x : v.x;
+        if (inb) qb[K] = minus ? -v.y : v.y;
+    }
+    if (!whole_u) return;
+    if (g == 0) {
+        if (ina) qa[0] = qa[n] = 0.0;
+        if (inb) qb[0] = qb[n] = 0.0;
+    }
+    const int m = n + 1;
+    for (int r = blockIdx.x; r < (d == 3 ? 4 * m : 2); r += gridDim.x) {
+        // 2D: j = 0, n; 3D: (j = 0, n; every k), then (every j; k = 0, n)
+        const int side = d == 3 ? r / m : r, t = d == 3 ? r % m : 0;
+        const int j = side == 0 ? 0 : side == 1 ? n : t;
+        const int k = side == 2 ? 0 : side == 3 ? n : t;
+        double* p = dst + k * dsz + j * dsy;
+        for (int i = threadIdx.x; i < m; i += blockDim.x) p[i] = 0.0;
     }
 }
 
-int flat_blocks(int64_t total) { return (int)std::min<int64_t>((total + 255) / 256, 152 * 16); }
+// DST-I along y of the work array, in place (row pitch n, plane n*n, planes
+// 1..n-1): a CTA takes the tile's pairs of neighbouring columns, loaded and
+// stored row by row.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_dst_y(double* __restrict__ w, int64_t pairs, Plan P,
+                                                   const double2* __restrict__ T) {
+    extern __shared__ double2 sm[];
+    const int lg = P.lg, n = P.n();
+    const int cols = 2 * P.pairs();
+    const int col = threadIdx.x & (cols - 1), lp = col >> 1;
+    const int j0 = threadIdx.x / cols, dj = blockDim.x / cols;
+    const int64_t q = (int64_t)blockIdx.x * P.pairs() + lp;
+    const int64_t plane = q >> (lg - 1);
+    const int64_t x = 2 * (q & (n / 2 - 1)) + (col & 1);
+    // column 0 is no line: its partner's rounding errors must not stay in it
+    const bool in = q < pairs && x > 0;
+    double* base = w + (in ? ((plane + 1) << (2 * lg)) + x : 0);
+    double* sl = reinterpret_cast<double*>(sm + lp * P.stride()) + (col & 1);
+#pragma unroll 4
+    for (int j = 1 + j0; j < n / 2; j += dj) {
+        const double a = in ? base[(int64_t)j << lg] : 0.0;
+        const double b = in ? base[(int64_t)(n - j) << lg] : 0.0;
+        sl[2 * at(j)] = a - b;
+        sl[2 * at(n - j)] = a + b;
+    }
+    if (j0 == 0) sl[2 * at(n / 2)] = in ? base[(int64_t)(n / 2) << lg] : 0.0;
+    __syncthreads();
+    dst_tile(sm, P, T);
+    if (!in) return;
+    for (int K = 1 + j0; K < n; K += dj) {
+        bool minus;
+        const double v = sl[2 * coeff_at(K, lg, minus)];
+        base[(int64_t)K << lg] = minus ? -v : v;
+    }
+}
+
+// -------------------------------------------------- lines of the last axis
+//
+// Elimination from both ends to the middle k = n/2 (half the chain, half the
+// coefficients): c_1 = 1/(2+lambda), c_k = 1/(2+lambda - c_{k-1}) serve both
+// halves, v'_k = (s d_k + v'_{k-1}) c_k, the middle value takes 1/(2+lambda -
+// 2 c_{n/2-1}), and each half substitutes back v_k = v'_k + c_k v_{k+1}.
+// The coefficients are a table of the plan (one row per k = 1..n/2, the last
+// one the middle's), in closed form: with r + 1/r = 2 + lambda, r < 1,
+//     c_k = 1 - e_k,  e_k = (1-r)(1 + r^{2k+1}) / (1 - r^{2k+2}),
+//     1 - r = sqrt(lambda + lambda^2/4) - lambda/2.
+// r and its powers are double-double.  An error that all c_k of a line share
+// enters the solution 1/(1-r) times over, so they have to be as good as
+// correctly rounded: the recurrence in double (c_k = 1/(2 + lambda - c_{k-1}),
+// or e_k = t/(1+t), t = lambda + e_{k-1}, free of cancellation) cost 2D 4097^2
+// a relative 1e-14, these 5e-15 like the transforms.
+struct DD {
+    double h, l;
+};
+__device__ inline DD dd_sum(double a, double b) {  // a + b, exactly
+    const double s = a + b, t = s - a;
+    return {s, (a - (s - t)) + (b - t)};
+}
+__device__ inline DD dd_add(DD a, DD b) {
+    const DD s = dd_sum(a.h, b.h);
+    return dd_sum(s.h, s.l + (a.l + b.l));
+}
+__device__ inline DD dd_mul(DD a, DD b) {
+    const double p = a.h * b.h;
+    return dd_sum(p, fma(a.h, b.h, -p) + fma(a.h, b.l, a.l * b.h));
+}
+// One thread per line and kSeg coefficients.
+constexpr int kSeg = 16;
+__global__ void __launch_bounds__(128) k_coeffs(double* __restrict__ c, int d, int n) {
+    const int64_t lines = d == 3 ? (int64_t)n * n : n;
+    const int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (l >= lines) return;
+    const int x = (int)(l % n), y = (int)(l / n);  // y = 0 in 2D
+    const double sx = sinpi(x / (2.0 * n)), sy = sinpi(y / (2.0 * n));
+    const double lambda = 4.0 * fma(sx, sx, sy * sy);
+    const int k0 = 1 + kSeg * (int)blockIdx.y, k1 = min(k0 + kSeg, n / 2);
+    if (lambda == 0.0) {  // row and column 0 of the transformed axes: no line
+        for (int k = k0; k < k1; ++k) c[(int64_t)k * lines + l] = 0.0;
+        if (k1 == n / 2) c[(int64_t)k1 * lines + l] = 0.0;
+        return;
+    }
+    const DD w = dd_mul({lambda, 0.0}, dd_sum(1.0, 0.25 * lambda));
+    const double q = sqrt(w.h);
+    const DD e1 = dd_add(dd_sum(q, (fma(-q, q, w.h) + w.l) / (2.0 * q)), {-0.5 * lambda, 0.0});
+    const DD r = dd_add({1.0, 0.0}, {-e1.h, -e1.l});
+    // power = r^(2 k0 - 1); 0 where it is far below the last bit (r <= exp(-e1))
+    DD power{0.0, 0.0};
+    if ((2.0 * k0 - 1.0) * e1.h < 45.0) {
+        DD base = r;
+        power = {1.0, 0.0};
+        for (int m = 2 * k0 - 1; m > 0; m >>= 1) {
+            if (m & 1) power = dd_mul(power, base);
+            base = dd_mul(base, base);
+        }
+    }
+    const DD r2 = dd_mul(r, r);
+    // e_k from r^(2k+1)
+    auto e_of = [&](DD pw) {
+        const DD rp = dd_mul(pw, r);
+        const DD den = dd_add({1.0, 0.0}, {-rp.h, -rp.l}), num = dd_add({1.0, 0.0}, pw);
+        return e1.h * num.h / den.h;
+    };
+    if (power.h == 0.0) {
+        const double ck = r.h;
+        for (int k = k0; k < k1; ++k) c[(int64_t)k * lines + l] = ck;
+    } else {
+        for (int k = k0; k < k1; ++k) {
+            power = dd_mul(power, r2);  // r^(2k+1)
+            c[(int64_t)k * lines + l] = 1.0 - e_of(power);
+        }
+    }
+    // the middle: 2 + lambda - 2 c = lambda + 2 e, k = n/2 - 1
+    if (k1 == n / 2) c[(int64_t)k1 * lines + l] = 1.0 / (lambda + 2.0 * e_of(power));
+}
+
+// `count` steps v[k dv] -> f(v[k dv], c[k dc]), k = 0.. ; the operands of kB
+// steps are loaded together.  STORE: f's value replaces v[k dv].
+constexpr int kB = 8;
+template <bool STORE, class F>
+__device__ inline void chain(double* __restrict__ v, int64_t dv, const double* __restrict__ c,
+                             int64_t dc, int count, F&& f) {
+    for (int k0 = 0; k0 < count; k0 += kB) {
+        double a[kB], b[kB];
+#pragma unroll
+        for (int t = 0; t < kB; ++t)
+            if (k0 + t < count) {
+                a[t] = v[(k0 + t) * dv];
+                b[t] = c[(k0 + t) * dc];
+            }
+#pragma unroll
+        for (int t = 0; t < kB; ++t)
+            if (k0 + t < count) {
+                const double w = f(a[t], b[t]);
+                if (STORE) v[(k0 + t) * dv] = w;
+            }
+    }
+}
+
+// 3D: one thread per half line; x along the lanes, threadIdx.y the half (0:
+// from k = 1 up, 1: from k = n-1 down), threadIdx.z one of the CTA's rows.
+// 3 FP64 instructions and (with the coefficients, read twice) 40 bytes per
+// node: 126 us at 257^3, 76% of the FP64 pipe.
+__global__ void __launch_bounds__(256) k_lines(double* __restrict__ w, const double* __restrict__ c,
+                                               int n, int64_t step, double scale) {
+    __shared__ double tip[4][2][32];
+    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 4 + threadIdx.z;
+    const int half = threadIdx.y;
+    // column 0 and row 0 of the transformed axes hold no coefficient
+    const bool in = x > 0 && x < n && y > 0 && y < n;
+    const int m = n / 2;
+    const int64_t l = (int64_t)y * n + x;
+    double* v = w + l + (half ? (int64_t)n * step : 0);
+    const int64_t dir = half ? -step : step;
+    const double* cl = c + l;
+    double prev = 0.0, dm = 0.0;
+    if (in) {
+        chain<true>(v + dir, dir, cl + step, step, m - 1,
+                    [&](double d, double ck) { return prev = fma(scale, d, prev) * ck; });
+        tip[threadIdx.z][half][threadIdx.x] = prev;
+        dm = v[m * dir];  // the same entry for both halves, read before it is replaced
+    }
+    __syncthreads();
+    if (!in) return;
+    prev = (fma(scale, dm, tip[threadIdx.z][0][threadIdx.x]) +
+            tip[threadIdx.z][1][threadIdx.x]) *
+           cl[m * step];
+    if (half == 0) v[m * dir] = prev;
+    chain<true>(v + (m - 1) * dir, -dir, cl + (m - 1) * step, -step, m - 1,
+                [&](double d, double ck) { return prev = fma(ck, prev, d); });
+}
+
+// 2D has only n - 1 lines, too few for their chains (192 cycles of dependent
+// FP64 a node) to be hidden: each half line is cut into kC pieces with a
+// thread each.  Both recurrences are linear in what flows into a piece, so a
+// first pass over the piece with inflow 0 gives its outflow t and the factor
+// p = prod c_k of its inflow, the inflows follow from those, and a second
+// pass stores the values.  7 instructions per node instead of 3, a chain 1/16
+// as long: 4097^2 578 -> 318 us, 257^2 33 -> 12 us.
+// X columns to a CTA: 16 (128-byte rows) where that makes enough CTAs, else 8.
+constexpr int kC = 16;
+template <int X>
+__global__ void __launch_bounds__(2 * X * kC) k_lines_2d(double* __restrict__ w,
+                                                      const double* __restrict__ c, int n,
+                                                      double scale) {
+    __shared__ double out[2][kC][X], fac[2][kC][X];
+    const int tx = threadIdx.x, half = threadIdx.y & 1, piece = threadIdx.y >> 1;
+    const int x = blockIdx.x * X + tx;
+    const bool in = x > 0 && x < n;
+    const int m = n / 2, len = (m - 1 + kC - 1) / kC;
+    const int k0 = 1 + piece * len, count = max(0, min(len, m - k0));  // k = k0 ..
+    const int64_t step = n;
+    double* v = w + x + (half ? (int64_t)n * step : 0);
+    const int64_t dir = half ? -step : step;
+    const double* cl = c + x;
+    double t = 0.0, p = 1.0, dm = 0.0;
+    if (in) {
+        chain<false>(v + k0 * dir, dir, cl + k0 * step, step, count, [&](double d, double ck) {
+            p *= ck;
+            return t = fma(scale, d, t) * ck;
+        });
+        dm = v[m * dir];  // read before it is replaced
+    }
+    out[half][piece][tx] = t;
+    fac[half][piece][tx] = p;
+    __syncthreads();
+    // flow[h]: what flows into this piece (own half) and into the middle
+    double prev = 0.0, tip[2] = {0.0, 0.0};
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        for (int i = 0; i < kC; ++i) {
+            if (h == half && i == piece) prev = tip[h];
+            tip[h] = fma(fac[h][i][tx], tip[h], out[h][i][tx]);
+        }
+    double mid = 0.0;
+    if (in) {
+        mid = (fma(scale, dm, tip[0]) + tip[1]) * cl[m * step];
+        chain<true>(v + k0 * dir, dir, cl + k0 * step, step, count,
+                    [&](double d, double ck) { return prev = fma(scale, d, prev) * ck; });
+        // back substitution from the piece's far end
+        t = 0.0;
+        chain<false>(v + (k0 + count - 1) * dir, -dir, cl + (k0 + count - 1) * step, -step, count,
+                     [&](double d, double ck) { return t = fma(ck, t, d); });
+    }
+    __syncthreads();
+    out[half][piece][tx] = t;
+    __syncthreads();
+    if (!in) return;
+    prev = mid;
+    for (int i = kC - 1; i > piece; --i) prev = fma(fac[half][i][tx], prev, out[half][i][tx]);
+    if (half == 0 && piece == 0) v[m * dir] = mid;
+    chain<true>(v + (k0 + count - 1) * dir, -dir, cl + (k0 + count - 1) * step, -step, count,
+                [&](double d, double ck) { return prev = fma(ck, prev, d); });
+}
 
 }  // namespace
 }  // namespace fft
@@ -119,25 +542,53 @@ using namespace gmg::fft;
 
 struct gmg_fft_s {
     int d = 3, n = 0, device = 0;
-    int64_t lines = 0;
     cudaStream_t user_stream = nullptr, stream = nullptr;
     cudaEvent_t ev = nullptr;
-    cufftHandle plan_x = 0, plan_yz = 0;
-    bool have_x = false, have_yz = false;
-    double* ext = nullptr;
-    cufftDoubleComplex* spec = nullptr;
-    double* work = nullptr;
+    Plan plan;
+    double2* twiddles = nullptr;  // e^{i pi k/n}, k < 2n
+    double* coeffs = nullptr;     // the eliminations' coefficients, n/2 + 1 rows
+    double* work = nullptr;       // n^d
 };
+
+namespace {
+
+template <int THREADS>
+cudaError_t allow_smem(size_t bytes) {
+    cudaError_t e = cudaFuncSetAttribute(k_dst_x<THREADS>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_dst_y<THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)bytes);
+    return e;
+}
+
+void dst_x(gmg_fft h, const double* src, int64_t ssy, int64_t ssz, double* dst, int64_t dsy,
+           int64_t dsz, int whole_u) {
+    const int64_t m = h->n - 1, lines = h->d == 3 ? m * m : m;
+    const unsigned blocks = (unsigned)(((lines + 1) / 2 + h->plan.pairs() - 1) / h->plan.pairs());
+    auto kern = h->plan.threads > 256 ? k_dst_x<512> : k_dst_x<256>;
+    kern<<<blocks, h->plan.threads, h->plan.smem(), h->stream>>>(src, ssy, ssz, dst, dsy, dsz,
+                                                                   lines, h->d, h->plan, whole_u,
+                                                                   h->twiddles);
+}
+
+void dst_y(gmg_fft h) {
+    const int64_t pairs = (int64_t)(h->n - 1) * (h->n / 2);
+    const unsigned blocks = (unsigned)((pairs + h->plan.pairs() - 1) / h->plan.pairs());
+    auto kern = h->plan.threads > 256 ? k_dst_y<512> : k_dst_y<256>;
+    kern<<<blocks, h->plan.threads, h->plan.smem(), h->stream>>>(h->work, pairs, h->plan,
+                                                                   h->twiddles);
+}
+
+}  // namespace
 
 extern "C" {
 
 gmg_status gmg_fft_destroy(gmg_fft h) {
     if (!h) return GMG_OK;
     if (h->stream) cudaStreamSynchronize(h->stream);
-    if (h->have_x) cufftDestroy(h->plan_x);
-    if (h->have_yz) cufftDestroy(h->plan_yz);
-    cudaFree(h->ext);
-    cudaFree(h->spec);
+    cudaFree(h->twiddles);
+    cudaFree(h->coeffs);
     cudaFree(h->work);
     if (h->ev) cudaEventDestroy(h->ev);
     if (h->stream) cudaStreamDestroy(h->stream);
@@ -160,7 +611,7 @@ gmg_status gmg_fft_create(int d, int n, void* cuda_stream, gmg_fft* out) {
     h->d = d;
     h->n = n;
     h->user_stream = (cudaStream_t)cuda_stream;
-    h->lines = d == 3 ? (int64_t)(n - 1) * (n - 1) : (n - 1);
+    h->plan = plan_of(n, d == 3 ? (int64_t)(n - 1) * (n - 1) / 2 : n / 2);
     auto fail = [&](gmg_status s, const std::string& m) {
         set_error("gmg_fft_create: " + m);
         gmg_fft_destroy(h);
@@ -170,27 +621,45 @@ gmg_status gmg_fft_create(int d, int n, void* cuda_stream, gmg_fft* out) {
     if (cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev, cudaEventDisableTiming) != cudaSuccess)
         return fail(GMG_ERR_CUDA, "stream/event creation failed");
-    const int64_t m = n + 1;
-    const int64_t nodes = d == 3 ? m * m * m : m * m;
-    if (cudaMalloc(&h->ext, sizeof(double) * h->lines * 2 * n) != cudaSuccess ||
-        cudaMalloc(&h->spec, sizeof(cufftDoubleComplex) * h->lines * (n + 1)) != cudaSuccess ||
-        cudaMalloc(&h->work, sizeof(double) * nodes) != cudaSuccess)
+    const int64_t lines = d == 3 ? (int64_t)n * n : n;
+    if (cudaMalloc(&h->twiddles, sizeof(double2) * 2 * n) != cudaSuccess ||
+        cudaMalloc(&h->coeffs, sizeof(double) * lines * (n / 2 + 1)) != cudaSuccess ||
+        cudaMalloc(&h->work, sizeof(double) * lines * n) != cudaSuccess)
         return fail(GMG_ERR_ALLOC, "cudaMalloc failed");
-    int len = 2 * n;
-    int batch = (int)h->lines;
-    // lines along x: contiguous extensions
-    if (cufftPlanMany(&h->plan_x, 1, &len, nullptr, 1, len, nullptr, 1, n + 1, CUFFT_D2Z, batch) !=
-        CUFFT_SUCCESS)
-        return fail(GMG_ERR_CUDA, "cufftPlanMany (x) failed");
-    h->have_x = true;
-    // lines along y / z: element-major extensions (stride = lines)
-    int inembed = len, onembed = n + 1;
-    if (cufftPlanMany(&h->plan_yz, 1, &len, &inembed, batch, 1, &onembed, batch, 1, CUFFT_D2Z,
-                      batch) != CUFFT_SUCCESS)
-        return fail(GMG_ERR_CUDA, "cufftPlanMany (y/z) failed");
-    h->have_yz = true;
-    cufftSetStream(h->plan_x, h->stream);
-    cufftSetStream(h->plan_yz, h->stream);
+    const size_t smem = h->plan.smem();
+    if ((h->plan.threads > 256 ? allow_smem<512>(smem) : allow_smem<256>(smem)) != cudaSuccess)
+        return fail(GMG_ERR_CUDA, "cudaFuncSetAttribute failed");
+    std::vector<double> t(4 * (size_t)n);
+    for (int k = 0; k < 2 * n; ++k) {
+        // from the first octant, so that every entry is correctly rounded up to
+        // the rounding of a small argument
+        const int oct = (int)((int64_t)4 * k / n), r = k - (int)((int64_t)oct * n / 4);
+        double c, s;
+        if (n < 4) {  // k multiples of pi/2
+            const double cs[4] = {1, 0, -1, 0}, sn[4] = {0, 1, 0, -1};
+            c = cs[(k * (2 / n)) & 3];
+            s = sn[(k * (2 / n)) & 3];
+        } else {
+            const bool odd = oct & 1;  // measured back from the octant's end
+            const long double a = 3.14159265358979323846264338327950288L * (odd ? n / 4 - r : r) / n;
+            const double ca = (double)cosl(a), sa = (double)sinl(a);
+            const int quad = ((oct + 1) / 2) & 3;  // nearest multiple of pi/2, angle = quad pi/2 +- a
+            const double sg = odd ? -1.0 : 1.0;
+            const double cc[4] = {ca, -sg * sa, -ca, sg * sa}, ss[4] = {sg * sa, ca, -sg * sa, -ca};
+            c = cc[quad];
+            s = ss[quad];
+        }
+        t[2 * k] = c;
+        t[2 * k + 1] = s;
+    }
+    if (cudaMemcpyAsync(h->twiddles, t.data(), sizeof(double) * t.size(), cudaMemcpyHostToDevice,
+                        h->stream) != cudaSuccess ||
+        cudaMemsetAsync(h->work, 0, sizeof(double) * lines * n, h->stream) != cudaSuccess)
+        return fail(GMG_ERR_CUDA, "initialisation failed");
+    const unsigned segs = (unsigned)std::max(1, (n / 2 - 1 + kSeg - 1) / kSeg);
+    k_coeffs<<<dim3((unsigned)((lines + 127) / 128), segs), 128, 0, h->stream>>>(h->coeffs, d, n);
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(h->stream) != cudaSuccess)
+        return fail(GMG_ERR_CUDA, "initialisation failed");
     *out = h;
     return GMG_OK;
 }
@@ -204,31 +673,22 @@ gmg_status gmg_fft_solve(gmg_fft h, const double* f, double* u) {
     cudaStream_t s = h->stream;
     GMG_CUDA_TRY(cudaEventRecord(h->ev, h->user_stream));
     GMG_CUDA_TRY(cudaStreamWaitEvent(s, h->ev, 0));
-    const int64_t m = n + 1;
-    const int64_t nodes = d == 3 ? m * m * m : m * m;
-    // b = h^2 f (interior), u = 0 on the boundary; work holds the transforms
-    k_scale_rhs<<<flat_blocks(nodes), 256, 0, s>>>(f, h->work, d, n);
-    GMG_CUDA_TRY(cudaMemsetAsync(u, 0, sizeof(double) * nodes, s));
-    const int64_t ext_total = h->lines * 2 * n, out_total = h->lines * (n - 1);
-    auto pass = [&](const double* src, double* dst, int axis, double scale, int eig) -> gmg_status {
-        k_extend<<<flat_blocks(ext_total), 256, 0, s>>>(src, h->ext, d, n, axis, h->lines);
-        if (cufftExecD2Z(axis == 0 ? h->plan_x : h->plan_yz, h->ext, h->spec) != CUFFT_SUCCESS) {
-            set_error("cufftExecD2Z failed");
-            return GMG_ERR_CUDA;
-        }
-        k_extract<<<flat_blocks(out_total), 256, 0, s>>>(h->spec, dst, d, n, axis, h->lines,
-                                                        scale, eig);
-        return GMG_OK;
-    };
-    gmg_status st;
-    // forward DST on every axis, the last pass divided by lambda
-    for (int a = 0; a < d; ++a)
-        if ((st = pass(h->work, h->work, a, 1.0, a == d - 1)) != GMG_OK) return st;
-    // inverse: the same transforms scaled by (2/n)^d, the last pass into u
-    for (int a = 0; a < d; ++a) {
-        const double sc = a == 0 ? std::pow(2.0 / n, d) : 1.0;
-        if ((st = pass(h->work, a == d - 1 ? u : h->work, a, sc, 0)) != GMG_OK) return st;
-    }
+    const int64_t m = n + 1, mz = d == 3 ? m * m : 0;
+    const int64_t wy = n, wz = d == 3 ? (int64_t)n * n : 0;
+    dst_x(h, f, m, mz, h->work, wy, wz, 0);
+    if (d == 3) dst_y(h);
+    // h^2, the inverse transforms' (2/n)^(d-1) and a half per transform: a power
+    // of two, exact
+    const double scale = std::pow(0.5 / n, d - 1) / ((double)n * n);
+    if (d == 3)
+        k_lines<<<dim3((n + 31) / 32, (n + 3) / 4), dim3(32, 2, 4), 0, s>>>(h->work, h->coeffs, n,
+                                                                            wz, scale);
+    else if (n >= 2048)
+        k_lines_2d<16><<<n / 16, dim3(16, 2 * kC), 0, s>>>(h->work, h->coeffs, n, scale);
+    else
+        k_lines_2d<8><<<(n + 7) / 8, dim3(8, 2 * kC), 0, s>>>(h->work, h->coeffs, n, scale);
+    if (d == 3) dst_y(h);
+    dst_x(h, h->work, wy, wz, u, m, mz, 1);
     GMG_CUDA_TRY(cudaGetLastError());
     GMG_CUDA_TRY(cudaStreamSynchronize(s));
     return GMG_OK;

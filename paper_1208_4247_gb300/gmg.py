@@ -484,7 +484,7 @@ def measure_fp64_rate(kind: int = 0, stream=None) -> float:
 
 
 class FFTSolver:
-    """Direct sine-transform (cuFFT DST-I) solve of the same FD system."""
+    """Direct sine-transform (DST-I) solve of the same FD system."""
 
     def __init__(self, d: int, n: int, stream=None):
         self.d, self.n = d, n
