@@ -479,6 +479,14 @@ bool leg_level(gmg_handle h, const std::vector<Level<T>>& lv, int l) {
 // level with n <= 8 (3D) / 32 (2D) (GMG_TAIL_N overrides) whose tail arrays
 // fit in 200 KB of shared memory, below every learned level, leaving at
 // least two tail levels.
+// Red-black 3D handles start it at 33^3 or 17^3 (as the cluster of
+// slab_tail.cu) where the hierarchy has such a level and no threshold is given.
+template <typename T>
+bool slab_level(gmg_handle h, const std::vector<Level<T>>& lv, int l) {
+    const gmg_config& c = h->cfg;
+    return h->tail_max == 0 && tail::slab_applies(c.d, lv[l].n, (int)lv.size() - l, c.smoother,
+                                                  c.transfer == GMG_TRANSFER_PAPER);
+}
 template <typename T>
 int tail_level(gmg_handle h, const std::vector<Level<T>>& lv) {
     const gmg_config& c = h->cfg;
@@ -488,6 +496,8 @@ int tail_level(gmg_handle h, const std::vector<Level<T>>& lv) {
     if (c.smoother == GMG_LEARNED)
         for (int l = 0; l < L && l < (int)h->lw.size(); ++l)
             if (h->lw[l]) lo = l + 1;
+    for (int l = lo; l < L; ++l)
+        if (slab_level<T>(h, lv, l)) return l;
     for (int l = lo; l + 1 < L; ++l) {
         const int n = lv[l].n;
         if (n <= nmax && tail::smem_bytes(c.d, n, L - l, c.smoother, sizeof(T)) <= 200 * 1024)
@@ -557,6 +567,19 @@ cudaError_t launch_grid_tail(gmg_handle h, std::vector<Level<T>>& lv, int lg) {
                                 h->stream, h->gtail_cluster);
 }
 
+// The tail from level l on (tail_level); top: level l is level 0.
+template <typename T>
+cudaError_t launch_tail(gmg_handle h, std::vector<Level<T>>& lv, int l, bool top) {
+    const gmg_config& c = h->cfg;
+    Level<T>& v = lv[l];
+    const int levels = (int)lv.size() - l;
+    if (slab_level<T>(h, lv, l))
+        return tail::launch_slab<T>(v.lay, levels, v.u[0], v.q, c.smoother, c.nu1, c.nu2,
+                                    c.coarse_sweeps, h->stream, top, false);
+    return tail::launch<T>(c.d, v.lay, levels, v.u[0], v.q, c.smoother, c.omega, c.nu1, c.nu2,
+                           c.coarse_sweeps, h->stream, top, c.transfer == GMG_TRANSFER_PAPER);
+}
+
 // One cycle of Algorithm 1 on the hierarchy lv (level-0 iterate lv[0].u[0]
 // in and out), in stream order.  first_red_done: the cycle's first level-0
 // red half sweep already ran (fp64::red_ahead); it starts with the black one.
@@ -576,9 +599,7 @@ gmg_status enqueue_vcycle(gmg_handle h, std::vector<Level<T>>& lv, bool first_re
         // the whole hierarchy is small: one persistent launch
         cudaError_t e = cudaSuccess;
         timed(h, K_TAIL, 0, p, lv[0].n, false, [&] {
-            e = tail::launch<T>(d, lv[0].lay, L, lv[0].u[0], lv[0].q, c.smoother, c.omega, c.nu1,
-                                c.nu2, c.coarse_sweeps, h->stream, true,
-                                c.transfer == GMG_TRANSFER_PAPER);
+            e = launch_tail<T>(h, lv, 0, true);
         });
         GMG_CUDA_TRY(e);
     } else if (L == 1) {
@@ -649,9 +670,7 @@ gmg_status enqueue_vcycle(gmg_handle h, std::vector<Level<T>>& lv, bool first_re
         } else if (lt < L) {
             cudaError_t e = cudaSuccess;
             timed(h, K_TAIL, lt, p, lv[lt].n, false, [&] {
-                e = tail::launch<T>(d, lv[lt].lay, L - lt, lv[lt].u[0], lv[lt].q, c.smoother,
-                                    c.omega, c.nu1, c.nu2, c.coarse_sweeps, h->stream, false,
-                                    c.transfer == GMG_TRANSFER_PAPER);
+                e = launch_tail<T>(h, lv, lt, false);
             });
             GMG_CUDA_TRY(e);
         } else {

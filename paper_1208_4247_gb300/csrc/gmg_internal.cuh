@@ -233,6 +233,14 @@ template <typename T>
 cudaError_t launch(int d, const Lay& top, int levels, T* u_top, const T* q_top, int smoother,
                    double omega, int nu1, int nu2, int coarse_sweeps, cudaStream_t s,
                    bool exact_top = false, bool paper = false);
+// The tail from a 33^3 or 17^3 level down as one cluster of 16 CTAs
+// (slab_tail.cu): red-black smoothing, full weighting, a hierarchy that
+// reaches 9^3.  first_done: the top level's first red half sweep ran already.
+bool slab_applies(int d, int n, int levels, int smoother, bool paper);
+template <typename T>
+cudaError_t launch_slab(const Lay& top, int levels, T* u_top, const T* q_top, int smoother,
+                        int nu1, int nu2, int coarse_sweeps, cudaStream_t s, bool exact_top,
+                        bool first_done);
 // The same on the levels' own dense arrays (n[l], u[l], q[l], r[l] for the
 // `levels` levels from the first one down), one cooperative launch of
 // `blocks` CTAs (grid_blocks: one wave; 0 when the device cannot) with grid

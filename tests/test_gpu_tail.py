@@ -52,3 +52,28 @@ def test_tail_equals_grid_kernels(monkeypatch, d, n, kw):
         u, rel = cycles(monkeypatch, tail_n, d, n, kw)
         assert np.array_equal(u, ref), (tail_n, np.max(np.abs(u - ref)))
         assert rel == rel_ref
+
+
+SLAB = [(n, prec, dict(nu1=nu1, nu2=nu2, **kw))
+        for prec in ("fp64", "df", "fp32", "bf16")
+        for n, nu1, nu2, kw in ((64, 2, 2, {}), (32, 1, 3, {}), (16, 2, 1, {}), (32, 2, 2, {"levels": 4}),
+                                (16, 1, 1, {"levels": 3}), (64, 1, 2, {"levels": 5, "coarse_sweeps": 3}))]
+SLAB += [(32, "fp64", dict(nu1=0, nu2=2)), (16, "fp64", dict(nu1=2, nu2=0)),
+         (32, "fp64", dict(nu1=1, nu2=2, cycle="fmg")), (16, "fp64", dict(nu1=2, nu2=2, cycle="fmg")),
+         (32, "df", dict(nu1=0, nu2=1)), (64, "fp32", dict(nu1=2, nu2=0))]
+
+
+@pytest.mark.parametrize("n,prec,kw", SLAB)
+def test_slab_tail_equals_grid_kernels(monkeypatch, n, prec, kw):
+    """The cluster of 16 CTAs (levels 33^3 and 17^3 in distributed shared
+    memory) against the grid kernels, bit for bit: as the tail of a larger
+    hierarchy and as the whole of a small one, hierarchies cut below 9^3,
+    no pre- or post-smoothing (full residual, full prolongation), FMG."""
+    pytest.importorskip("torch")
+    kw = dict(kw, precision=prec)
+    if prec != "fp64":
+        kw["inner_cycles"] = 2 if prec == "fp32" else 1
+    ref, rel_ref = cycles(monkeypatch, 1, 3, n, kw)
+    u, rel = cycles(monkeypatch, 0, 3, n, kw)
+    assert np.array_equal(u, ref), np.max(np.abs(u - ref))
+    assert rel == rel_ref
