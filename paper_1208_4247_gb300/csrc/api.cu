@@ -89,6 +89,7 @@ struct gmg_handle_s {
     cudaGraphExec_t loop_graph = nullptr;
     cudaGraphConditionalHandle loop_cond = 0;
     int loop_kernels = 0;         // kernel launches per loop iteration
+    int loop_partials = 0;        // the norm's partial sums that the loop's test adds up (0: none)
     int loop_cap = 0;             // history capacity of d_loop
     LoopState* d_loop = nullptr;
     LoopState* h_loop = nullptr;  // pinned
@@ -377,15 +378,15 @@ bool learned_level(gmg_handle h, int l) {
 }
 
 // One learned smoothing sweep on FP64 level l: sigma = (b - A'u)/(2d),
-// u += conv2(relu(conv1(sigma))).  sigma_ready: L.r already holds sigma of
-// the current u (level 0 after the stopping-test norm).
-void learned_sweep(gmg_handle h, Level<double>& L, int l, bool sigma_ready) {
+// u += conv2(relu(conv1(sigma))).  ready (may be NULL): sigma of the current u
+// (level 0 after the stopping-test norm: L.r; a coarse level's u = 0: L.q).
+void learned_sweep(gmg_handle h, Level<double>& L, int l, const double* ready) {
     const int d = h->cfg.d;
-    if (!sigma_ready)
+    if (!ready)
         timed(h, K_RESIDUAL, l, 0, L.n, false,
               [&] { lk::residual<double>(d, L.n, L.u[0], L.q, L.r, false, h->stream); });
     timed(h, K_CONV2, l, 0, L.n, false,
-          [&] { learned::conv_tc(d, L.n, L.r, L.u[0], 1, h->lw[l], h->stream); });
+          [&] { learned::conv_tc(d, L.n, ready ? ready : L.r, L.u[0], 1, h->lw[l], h->stream); });
 }
 
 // Enqueue `sweeps` smoothing sweeps on level l; cur tracks which u buffer
@@ -398,8 +399,9 @@ bool sigma_carried(gmg_handle h) {
 
 // backward: post-smoothing (Relax_backward), which takes the colours of the
 // multi-colour smoother in decreasing order.
-// first_red_done: the first red half sweep already ran (fused with the
-// previous step's stopping-test norm).
+// first_done: the first step (red half sweep, colour 0, Jacobi sweep) already
+// ran: fused with the previous step's stopping-test norm, or done by the
+// restriction to a coarse level (CoarseInit).
 // exact_last: the last half sweep (a black one) uses the unbiased FP64 3D
 // Gauss-Seidel value (lk::gs_value), as the level-0 pre-smoothing before the
 // unbiased red-only residual must (the black residual then stays exactly 0).
@@ -407,16 +409,17 @@ bool sigma_carried(gmg_handle h) {
 // (mixed::outer_red_update forms it in triple-float).
 template <typename T>
 void relax(gmg_handle h, std::vector<Level<T>>& lv, int l, int sweeps, int& cur,
-           bool sigma_ready = false, bool backward = false, bool first_red_done = false,
+           const double* sigma_ready = nullptr, bool backward = false, bool first_done = false,
            bool exact_last = false, bool skip_last_black = false) {
     Level<T>& L = lv[l];
     const int d = h->cfg.d;
     const int p = prec_of<T>();
     for (int s = 0; s < sweeps; ++s) {
+        const bool first = first_done && s == 0;
         if constexpr (std::is_same<T, double>::value) {
             if (h->cfg.smoother == GMG_MCGS) {
                 const int ncol = d == 3 ? 8 : 4;
-                for (int t = 0; t < ncol; ++t) {
+                for (int t = first ? 1 : 0; t < ncol; ++t) {
                     const int color = backward ? ncol - 1 - t : t;
                     timed(h, K_MC_SWEEP, l, p, L.n, false,
                           [&] { lk::mc_sweep<T>(d, L.lay, L.u[cur], L.q, color, h->stream); });
@@ -426,7 +429,7 @@ void relax(gmg_handle h, std::vector<Level<T>>& lv, int l, int sweeps, int& cur,
         }
         if constexpr (std::is_same<T, double>::value) {
             if (learned_level(h, l)) {
-                learned_sweep(h, L, l, sigma_ready && s == 0);
+                learned_sweep(h, L, l, s == 0 ? sigma_ready : nullptr);
                 continue;
             }
         }
@@ -440,13 +443,13 @@ void relax(gmg_handle h, std::vector<Level<T>>& lv, int l, int sweeps, int& cur,
             }
         }
         if (h->cfg.smoother == GMG_RBGS || h->cfg.smoother == GMG_LEARNED) {
-            for (int color = first_red_done && s == 0 ? 1 : 0; color < 2; ++color) {
+            for (int color = first ? 1 : 0; color < 2; ++color) {
                 if (skip_last_black && s == sweeps - 1 && color == 1) break;
                 const bool ex = exact_last && s == sweeps - 1 && color == 1;
                 timed(h, K_RB_HALF, l, p, L.n, false,
                       [&] { lk::rb_half<T>(d, L.lay, L.u[cur], L.q, color, h->stream, ex); });
             }
-        } else {
+        } else if (!first) {
             timed(h, K_WJ, l, p, L.n, false, [&] {
                 lk::wj_sweep<T>(d, L.lay, L.u[cur], L.u[cur ^ 1], L.q, h->cfg.omega, h->stream);
             });
@@ -485,7 +488,8 @@ template <typename T>
 bool slab_level(gmg_handle h, const std::vector<Level<T>>& lv, int l) {
     const gmg_config& c = h->cfg;
     return h->tail_max == 0 && tail::slab_applies(c.d, lv[l].n, (int)lv.size() - l, c.smoother,
-                                                  c.transfer == GMG_TRANSFER_PAPER);
+                                                  c.transfer == GMG_TRANSFER_PAPER,
+                                                  std::is_same<T, double>::value);
 }
 template <typename T>
 int tail_level(gmg_handle h, const std::vector<Level<T>>& lv) {
@@ -567,17 +571,32 @@ cudaError_t launch_grid_tail(gmg_handle h, std::vector<Level<T>>& lv, int lg) {
                                 h->stream, h->gtail_cluster);
 }
 
+// What the restriction to level l of the V-cycle leaves in its iterate: the
+// result of its first smoothing step, except on the coarsest level and on
+// levels whose smoothing does not take it (the grid tail's, the fused FP32
+// sweep's, a learned level's, whose first sigma is q then).
+template <typename T>
+int level_init(gmg_handle h, const std::vector<Level<T>>& lv, int l) {
+    const gmg_config& c = h->cfg;
+    if (l + 1 == (int)lv.size()) return lv[l].n == 2 ? INIT_EXACT : INIT_ZERO;
+    if (c.nu1 == 0 || l >= grid_tail_level<T>(h, lv) || use_fused_rb<T>(h) || learned_level(h, l))
+        return INIT_ZERO;
+    if (c.nu1 == 1 && leg_level<T>(h, lv, l)) return INIT_ZERO;  // a down leg takes two half sweeps or more
+    return c.smoother == GMG_WJACOBI ? INIT_WJ : c.smoother == GMG_MCGS ? INIT_COLOR0 : INIT_RED;
+}
+
 // The tail from level l on (tail_level); top: level l is level 0.
 template <typename T>
-cudaError_t launch_tail(gmg_handle h, std::vector<Level<T>>& lv, int l, bool top) {
+cudaError_t launch_tail(gmg_handle h, std::vector<Level<T>>& lv, int l, bool top, bool first_done) {
     const gmg_config& c = h->cfg;
     Level<T>& v = lv[l];
     const int levels = (int)lv.size() - l;
     if (slab_level<T>(h, lv, l))
         return tail::launch_slab<T>(v.lay, levels, v.u[0], v.q, c.smoother, c.nu1, c.nu2,
-                                    c.coarse_sweeps, h->stream, top, false);
+                                    c.coarse_sweeps, h->stream, top, first_done);
     return tail::launch<T>(c.d, v.lay, levels, v.u[0], v.q, c.smoother, c.omega, c.nu1, c.nu2,
-                           c.coarse_sweeps, h->stream, top, c.transfer == GMG_TRANSFER_PAPER);
+                           c.coarse_sweeps, h->stream, top, c.transfer == GMG_TRANSFER_PAPER,
+                           first_done);
 }
 
 // One cycle of Algorithm 1 on the hierarchy lv (level-0 iterate lv[0].u[0]
@@ -593,24 +612,27 @@ gmg_status enqueue_vcycle(gmg_handle h, std::vector<Level<T>>& lv, bool first_re
     const int L = (int)lv.size();
     const int p = prec_of<T>();
     std::vector<int> cur(L, 0);
+    // the level's first smoothing step ran already (level_init, or level 0's)
+    std::vector<char> done(L, 0);
+    done[0] = first_red_done;
     const int lt = tail_level<T>(h, lv);
     const int lg = lt == 0 ? L : grid_tail_level<T>(h, lv);
     if (lt == 0) {
         // the whole hierarchy is small: one persistent launch
         cudaError_t e = cudaSuccess;
         timed(h, K_TAIL, 0, p, lv[0].n, false, [&] {
-            e = launch_tail<T>(h, lv, 0, true);
+            e = launch_tail<T>(h, lv, 0, true, false);
         });
         GMG_CUDA_TRY(e);
     } else if (L == 1) {
-        relax(h, lv, 0, c.nu1, cur[0], false, false, first_red_done);
+        relax(h, lv, 0, c.nu1, cur[0], nullptr, false, first_red_done);
     } else {
         // levels smoothed by grid kernels going down
         const int Ldown = lg < L ? lg : lt < L ? lt : L - 1;
         for (int l = 0; l < Ldown; ++l) {
             // fused down leg: the pre-smoothing half sweeps, the red residual
             // and the restriction in one pass (u ping-pongs)
-            const int s_down = 2 * c.nu1 - (l == 0 && first_red_done ? 1 : 0);
+            const int s_down = 2 * c.nu1 - (done[l] ? 1 : 0);
             if (leg_level<T>(h, lv, l) && s_down >= 2 && s_down <= 4) {
                 Level<T>& F = lv[l];
                 Level<T>& C = lv[l + 1];
@@ -631,9 +653,12 @@ gmg_status enqueue_vcycle(gmg_handle h, std::vector<Level<T>>& lv, bool first_re
             // level 0 of the plain FP64 form: the residual of the full
             // iterate, unbiased in 3D (lk::gs_value)
             const bool unbiased = l == 0 && std::is_same<T, double>::value && d == 3;
-            relax(h, lv, l, c.nu1, cur[l],
-                  l == 0 && std::is_same<T, double>::value && sigma_carried(h), false,
-                  l == 0 && first_red_done, unbiased);
+            const double* sigma = nullptr;
+            if constexpr (std::is_same<T, double>::value) {
+                if (l == 0 && sigma_carried(h)) sigma = lv[l].r;
+                if (l > 0 && learned_level(h, l)) sigma = lv[l].q;
+            }
+            relax(h, lv, l, c.nu1, cur[l], sigma, false, done[l], unbiased);
             Level<T>& F = lv[l];
             Level<T>& C = lv[l + 1];
             // After a black half sweep the black residual vanishes identically.
@@ -644,21 +669,22 @@ gmg_status enqueue_vcycle(gmg_handle h, std::vector<Level<T>>& lv, bool first_re
             timed(h, K_RESIDUAL, l, p, F.n, red_only, [&] {
                 lk::residual<T>(d, F.lay, F.u[cur[l]], F.q, F.r, red_only, h->stream, unbiased);
             });
-            const bool exact = C.n == 2;
-            bool done = false;
+            const int init = level_init<T>(h, lv, l + 1);
+            done[l + 1] = init > INIT_EXACT;
+            bool restricted = false;
             if constexpr (std::is_same<T, double>::value) {
                 if (paper) {
                     timed(h, K_RESTRICT_PAPER, l, p, F.n, false, [&] {
-                        lk::restrict_paper<T>(d, F.lay, C.lay, F.r, C.q, C.u[0], exact,
-                                              h->stream);
+                        lk::restrict_paper<T>(d, F.lay, C.lay, F.r, C.q, C.u[0], init,
+                                              h->stream, c.omega);
                     });
-                    done = true;
+                    restricted = true;
                 }
             }
-            if (!done)
+            if (!restricted)
                 timed(h, K_RESTRICT, l, p, F.n, red_only, [&] {
-                    lk::restrict_fw<T>(d, F.lay, C.lay, F.r, C.q, C.u[0], red_only, exact,
-                                       h->stream);
+                    lk::restrict_fw<T>(d, F.lay, C.lay, F.r, C.q, C.u[0], red_only, init,
+                                       h->stream, c.omega);
                 });
             cur[l + 1] = 0;
         }
@@ -670,7 +696,7 @@ gmg_status enqueue_vcycle(gmg_handle h, std::vector<Level<T>>& lv, bool first_re
         } else if (lt < L) {
             cudaError_t e = cudaSuccess;
             timed(h, K_TAIL, lt, p, lv[lt].n, false, [&] {
-                e = launch_tail<T>(h, lv, lt, false);
+                e = launch_tail<T>(h, lv, lt, false, done[lt]);
             });
             GMG_CUDA_TRY(e);
         } else {
@@ -719,7 +745,7 @@ gmg_status enqueue_vcycle(gmg_handle h, std::vector<Level<T>>& lv, bool first_re
                                        black);
                 });
             }
-            relax(h, lv, l, c.nu2, cur[l], false, true, false, false, skip_last_black0 && l == 0);
+            relax(h, lv, l, c.nu2, cur[l], nullptr, true, false, false, skip_last_black0 && l == 0);
         }
     }
     if (cur[0] != 0) {
@@ -770,8 +796,9 @@ bool outer_red_only(gmg_handle h) {
 }
 
 // Refinement step: e = 0, k inner cycles on A'e = sigma, u += e, new sigma.
+// in_loop: the norm's partials are left to the loop's test (loop_partials).
 template <typename T>
-gmg_status enqueue_refinement(gmg_handle h, std::vector<Level<T>>& in) {
+gmg_status enqueue_refinement(gmg_handle h, std::vector<Level<T>>& in, bool in_loop) {
     const gmg_config& c = h->cfg;
     const int p = prec_of<T>();
     const bool ahead = inner_red_ahead<T>(h);
@@ -797,6 +824,7 @@ gmg_status enqueue_refinement(gmg_handle h, std::vector<Level<T>>& in) {
                                            h->resid_b, h->resid_flag);
             },
             3);
+        h->loop_partials = 0;  // summed already
         return GMG_OK;
     }
     timed(h, K_UPDATE, 0, p, c.n, false,
@@ -804,10 +832,11 @@ gmg_status enqueue_refinement(gmg_handle h, std::vector<Level<T>>& in) {
     timed(
         h, K_OUTER_RES, 0, p, c.n, ahead,
         [&] {
-            mixed::outer_residual<T>(c.d, in[0].lay, h->lv[0].u[0], h->lv[0].q, in[0].q, h->partial,
-                                     h->d_res2, h->stream, ahead ? in[0].u[0] : nullptr);
+            h->loop_partials = mixed::outer_residual<T>(
+                c.d, in[0].lay, h->lv[0].u[0], h->lv[0].q, in[0].q, h->partial,
+                in_loop ? nullptr : h->d_res2, h->stream, ahead ? in[0].u[0] : nullptr);
         },
-        2);
+        in_loop ? 1 : 2);
     return GMG_OK;
 }
 
@@ -835,15 +864,16 @@ bool norm_ahead_ok(gmg_handle h) {
 
 // The fused norm of the step's (or FMG pass's) result plus the next red half
 // sweep; the squared scaled norm lands in h->d_res2.
-void enqueue_norm_ahead(gmg_handle h) {
+void enqueue_norm_ahead(gmg_handle h, bool in_loop = false) {
     const gmg_config& c = h->cfg;
     Level<double>& L0 = h->lv[0];
     timed(
         h, K_NORM_AHEAD, 0, 0, c.n, true,
         [&] {
-            fp64::red_ahead(c.n, L0.u[0], L0.q, L0.r, h->partial, h->d_res2, true, h->stream);
+            h->loop_partials = fp64::red_ahead(c.n, L0.u[0], L0.q, L0.r, h->partial,
+                                               in_loop ? nullptr : h->d_res2, true, h->stream);
         },
-        2);
+        in_loop ? 1 : 2);
 }
 
 // Double-float refinement in steps of several cycles.  Each cycle of the
@@ -993,7 +1023,7 @@ gmg_status enqueue_step_kernels(gmg_handle h, bool in_loop = false) {
     } else if (c.precision == GMG_FP64 && h->ahead) {
         st = enqueue_vcycle<double>(h, h->lv, true);
         if (st != GMG_OK) return st;
-        enqueue_norm_ahead(h);
+        enqueue_norm_ahead(h, in_loop);
     } else if (c.precision == GMG_FP64) {
         st = enqueue_vcycle<double>(h, h->lv);
         if (st != GMG_OK) return st;
@@ -1001,16 +1031,17 @@ gmg_status enqueue_step_kernels(gmg_handle h, bool in_loop = false) {
         timed(
             h, K_RESNORM, 0, 0, c.n, norm_red_only(h),
             [&] {
-                fp64::resnorm(c.d, c.n, h->lv[0].u[0], h->lv[0].q, h->partial, h->d_res2,
-                              h->stream, keep, norm_red_only(h));
+                h->loop_partials =
+                    fp64::resnorm(c.d, c.n, h->lv[0].u[0], h->lv[0].q, h->partial,
+                                  in_loop ? nullptr : h->d_res2, h->stream, keep, norm_red_only(h));
             },
-            2);
+            in_loop ? 1 : 2);
     } else if (c.precision == GMG_FP32_IR) {
-        st = enqueue_refinement<float>(h, h->lvf);
+        st = enqueue_refinement<float>(h, h->lvf, in_loop);
     } else if (c.precision == GMG_DF_IR) {
-        st = enqueue_refinement<df32>(h, h->lvd);
+        st = enqueue_refinement<df32>(h, h->lvd, in_loop);
     } else {
-        st = enqueue_refinement<bf16>(h, h->lvb);
+        st = enqueue_refinement<bf16>(h, h->lvb, in_loop);
     }
     if (st != GMG_OK) return st;
     GMG_CUDA_TRY(cudaGetLastError());
@@ -1040,11 +1071,17 @@ gmg_status enqueue_step(gmg_handle h) {
 // (the host loop's test, in the same FP64 operations).
 }  // namespace
 namespace gmg {
-__global__ void k_loop_test(const double* __restrict__ res2, LoopState* __restrict__ st,
-                            cudaGraphConditionalHandle cond) {
+// count > 0: sums the norm's partials itself (fp64::k_sum_partials' order; one
+// launch less per cycle), else takes *res2.
+__global__ void __launch_bounds__(1024) k_loop_test(const double* __restrict__ partial, int count,
+                                                    const double* __restrict__ res2,
+                                                    LoopState* __restrict__ st,
+                                                    cudaGraphConditionalHandle cond) {
+    const double sum = count > 0 ? fp64::block_sum(partial, count) : res2[0];
+    if (threadIdx.x != 0) return;
     const int it = st->it + 1;
     st->it = it;
-    const double res = sqrt(res2[0]);
+    const double res = sqrt(sum);
     st->res = res;
     st->hist[it - 1] = st->res0 > 0.0 ? res / st->res0 : 0.0;
     const bool more = it < st->cap && isfinite(res) && (!st->stop || res > st->rtol * st->res0);
@@ -1090,7 +1127,8 @@ void build_loop_graph(gmg_handle h) {
     if (chain_on(h)) {  // the chain's test kernels set the condition
         h->loop_kernels = h->timer.graph_kernels;
     } else {
-        k_loop_test<<<1, 1, 0, h->stream>>>(h->d_res2, h->d_loop, h->loop_cond);
+        k_loop_test<<<1, 1024, 0, h->stream>>>(h->partial, h->loop_partials, h->d_res2, h->d_loop,
+                                               h->loop_cond);
         h->loop_kernels = h->timer.graph_kernels + 1;
     }
     h->timer.graph_kernels = step_kernels;
@@ -1114,12 +1152,13 @@ gmg_status enqueue_fmg(gmg_handle h) {
         Level<double>& C = lv[l + 1];
         if (c.transfer == GMG_TRANSFER_PAPER)
             timed(h, K_RESTRICT_PAPER, l, 0, F.n, false, [&] {
-                lk::restrict_paper<double>(d, F.lay, C.lay, F.q, C.q, C.u[0], C.n == 2,
-                                           h->stream);
+                lk::restrict_paper<double>(d, F.lay, C.lay, F.q, C.q, C.u[0],
+                                           C.n == 2 ? INIT_EXACT : INIT_ZERO, h->stream);
             });
         else
             timed(h, K_RESTRICT, l, 0, F.n, false, [&] {
-                lk::restrict_fw<double>(d, F.n, F.q, C.q, C.u[0], false, C.n == 2, h->stream);
+                lk::restrict_fw<double>(d, F.n, F.q, C.q, C.u[0], false,
+                                        C.n == 2 ? INIT_EXACT : INIT_ZERO, h->stream);
             });
     }
     if (L > 1 && lv[L - 1].n > 2) {

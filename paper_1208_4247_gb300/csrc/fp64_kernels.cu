@@ -23,12 +23,12 @@ template void wj_sweep<double>(int, const Lay&, const double*, double*, const do
 template void residual<double>(int, const Lay&, const double*, const double*, double*, bool,
                                cudaStream_t, bool);
 template void restrict_fw<double>(int, const Lay&, const Lay&, const double*, double*, double*,
-                                  bool, bool, cudaStream_t);
+                                  bool, int, cudaStream_t, double);
 template void prolong_add<double>(int, const Lay&, const Lay&, const double*, double*,
                                   cudaStream_t, bool);
 template void mc_sweep<double>(int, const Lay&, double*, const double*, int, cudaStream_t);
 template void restrict_paper<double>(int, const Lay&, const Lay&, const double*, double*,
-                                     double*, bool, cudaStream_t);
+                                     double*, int, cudaStream_t, double);
 template void prolong_paper<double>(int, const Lay&, const Lay&, const double*, double*,
                                     cudaStream_t);
 }  // namespace lk
@@ -287,17 +287,8 @@ NormLaunch norm_launch(int d, int n, bool red_only = false) {
 
 __global__ void __launch_bounds__(1024) k_sum_partials(const double* __restrict__ partial,
                                                        int count, double* __restrict__ out) {
-    __shared__ double warp_sums[32];
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < count; i += blockDim.x) acc += partial[i];
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-    if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x / 32); ++w) s += warp_sums[w];
-        out[0] = s;
-    }
+    const double s = block_sum(partial, count);
+    if (threadIdx.x == 0) out[0] = s;
 }
 
 void prepare(int d, int n, const double* f, double* q, double* u, cudaStream_t s,
@@ -355,8 +346,8 @@ bool red_ahead_applies(int d, int n) {
     return on && lk::walk_applies(d, n, sizeof(double));
 }
 
-void red_ahead(int n, double* u, const double* q, double* save, double* partial, double* out,
-               bool norm, cudaStream_t s, const double* plus) {
+int red_ahead(int n, double* u, const double* q, double* save, double* partial, double* out,
+              bool norm, cudaStream_t s, const double* plus) {
     // two waves of 3 resident CTAs per SM stride over the walkers; the
     // partial sums (one per CTA) fit the resnorm buffer (resnorm_partials)
     const lk::WalkLaunch W = lk::walk_launch(n);
@@ -374,7 +365,8 @@ void red_ahead(int n, double* u, const double* q, double* save, double* partial,
         launch(std::integral_constant<int, 256>{});
     else
         launch(std::integral_constant<int, 512>{});
-    if (norm) k_sum_partials_plus<<<1, 1024, 0, s>>>(partial, (int)blocks, plus, out);
+    if (norm && out) k_sum_partials_plus<<<1, 1024, 0, s>>>(partial, (int)blocks, plus, out);
+    return (int)blocks;
 }
 
 void resnorm_black(int n, const double* u, const double* q, double* partial, double* out,
@@ -391,14 +383,14 @@ void red_restore(int n, double* u, const double* save, cudaStream_t s) {
     k_red_restore3<<<blocks, 256, 0, s>>>(u, save, n);
 }
 
-void resnorm(int d, int n, const double* u, const double* q, double* partial, double* out,
-             cudaStream_t s, double* sigma_out, bool red_only) {
+int resnorm(int d, int n, const double* u, const double* q, double* partial, double* out,
+            cudaStream_t s, double* sigma_out, bool red_only) {
     if (red_only && !sigma_out && lk::walk_applies(d, n, sizeof(double))) {
         const lk::WalkLaunch W = lk::walk_launch(n);
         const unsigned blocks = std::min<unsigned>(W.blocks, (unsigned)resnorm_partials(d, n));
         k_resnorm3_walk<<<blocks, W.block, 0, s>>>(u, q, partial, n, W.segs, 0);
-        k_sum_partials<<<1, 1024, 0, s>>>(partial, (int)blocks, out);
-        return;
+        if (out) k_sum_partials<<<1, 1024, 0, s>>>(partial, (int)blocks, out);
+        return (int)blocks;
     }
     NormLaunch L = norm_launch(d, n, red_only && !sigma_out);
     if (sigma_out) {
@@ -417,7 +409,8 @@ void resnorm(int d, int n, const double* u, const double* q, double* partial, do
         else
             k_resnorm<2, false, false><<<L.grid, L.block, 0, s>>>(u, q, partial, n, nullptr);
     }
-    k_sum_partials<<<1, 1024, 0, s>>>(partial, (int)L.grid.x, out);
+    if (out) k_sum_partials<<<1, 1024, 0, s>>>(partial, (int)L.grid.x, out);
+    return (int)L.grid.x;
 }
 
 }  // namespace fp64

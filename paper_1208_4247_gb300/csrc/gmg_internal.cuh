@@ -69,6 +69,14 @@ struct Level {
     Lay lay;              // addressing of u, q, r
 };
 
+// What a restriction leaves in the coarse iterate, which starts from zero: 0;
+// the coarse values themselves (the grid of one unknown, solved exactly);
+// or the result of the level's first smoothing step from zero, which needs no
+// neighbour -- the red half sweep (u = q on red nodes), colour 0 of the
+// paper's Gauss-Seidel, or a weighted-Jacobi sweep (u = omega q) -- so that the
+// step needs no launch of its own.
+enum CoarseInit { INIT_ZERO = 0, INIT_EXACT = 1, INIT_RED = 2, INIT_COLOR0 = 3, INIT_WJ = 4 };
+
 // Level kernels, explicitly instantiated for double (fp64_kernels.cu) and
 // float / __nv_bfloat16 (mixed_kernels.cu); definitions in level_kernels.cuh.
 namespace lk {
@@ -90,7 +98,7 @@ void residual(int d, const Lay& L, const T* u, const T* q, T* r, bool red_only, 
               bool exact = false);
 template <typename T>
 void restrict_fw(int d, const Lay& F, const Lay& C, const T* r, T* qc, T* uc, bool red_only,
-                 bool exact_coarsest, cudaStream_t s);
+                 int init, cudaStream_t s, double omega = 0.0);
 // black_only: correct the black fine nodes only (valid when a red half sweep
 // follows, which overwrites every red node without reading it)
 template <typename T>
@@ -102,8 +110,8 @@ void prolong_add(int d, const Lay& C, const Lay& F, const T* uc, T* u, cudaStrea
 template <typename T>
 void mc_sweep(int d, const Lay& L, T* u, const T* q, int color, cudaStream_t s);
 template <typename T>
-void restrict_paper(int d, const Lay& F, const Lay& C, const T* r, T* qc, T* uc,
-                    bool exact_coarsest, cudaStream_t s);
+void restrict_paper(int d, const Lay& F, const Lay& C, const T* r, T* qc, T* uc, int init,
+                    cudaStream_t s, double omega = 0.0);
 template <typename T>
 void prolong_paper(int d, const Lay& C, const Lay& F, const T* uc, T* u, cudaStream_t s);
 
@@ -119,10 +127,9 @@ inline void residual(int d, int n, const T* u, const T* q, T* r, bool red_only, 
     residual<T>(d, dense_lay(d, n), u, q, r, red_only, s, exact);
 }
 template <typename T>
-inline void restrict_fw(int d, int n, const T* r, T* qc, T* uc, bool red_only,
-                        bool exact_coarsest, cudaStream_t s) {
-    restrict_fw<T>(d, dense_lay(d, n), dense_lay(d, n / 2), r, qc, uc, red_only, exact_coarsest,
-                   s);
+inline void restrict_fw(int d, int n, const T* r, T* qc, T* uc, bool red_only, int init,
+                        cudaStream_t s) {
+    restrict_fw<T>(d, dense_lay(d, n), dense_lay(d, n / 2), r, qc, uc, red_only, init, s);
 }
 template <typename T>
 inline void prolong_add(int d, int nc, const T* uc, T* u, cudaStream_t s,
@@ -144,10 +151,26 @@ void copy_strided(int d, int n, const double* src, int64_t ssy, int64_t ssz, dou
                   int64_t dsy, int64_t dsz, cudaStream_t s);
 // sum of sigma^2 into *out; sigma_out (may be NULL) also receives sigma;
 // red_only (ignored with sigma_out) sums red nodes only, valid right after a
-// black half sweep of level 0 (black sigma is then exactly zero)
-void resnorm(int d, int n, const double* u, const double* q, double* partial, double* out,
+// black half sweep of level 0 (black sigma is then exactly zero).  Returns
+// the number of partial sums; out = NULL leaves their sum to the caller
+// (block_sum).
+int resnorm(int d, int n, const double* u, const double* q, double* partial, double* out,
              cudaStream_t s, double* sigma_out = nullptr, bool red_only = false);
 __global__ void k_sum_partials(const double* partial, int count, double* out);
+// The sum of count partials by one CTA of 1024 threads in a fixed order (the
+// result in thread 0).
+__device__ inline double block_sum(const double* __restrict__ partial, int count) {
+    __shared__ double warp_sums[32];
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < count; i += blockDim.x) acc += partial[i];
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+    if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < (int)(blockDim.x / 32); ++w) s += warp_sums[w];
+    return s;
+}
 // The stopping-test norm of a red-black cycle fused with the next cycle's
 // first red half sweep (3D FP64 levels the diagonal walkers take, unless
 // GMG_NORM_AHEAD=0): the red-only norm of u into *out (norm = true; plus
@@ -156,8 +179,8 @@ __global__ void k_sum_partials(const double* partial, int count, double* out);
 // red interior nodes).  resnorm_black: the black nodes' sigma^2 sum (the
 // other half of a first norm whose red half red_ahead sums).
 bool red_ahead_applies(int d, int n);
-void red_ahead(int n, double* u, const double* q, double* save, double* partial, double* out,
-               bool norm, cudaStream_t s, const double* plus = nullptr);
+int red_ahead(int n, double* u, const double* q, double* save, double* partial, double* out,
+              bool norm, cudaStream_t s, const double* plus = nullptr);
 void resnorm_black(int n, const double* u, const double* q, double* partial, double* out,
                    cudaStream_t s);
 void red_restore(int n, double* u, const double* save, cudaStream_t s);
@@ -177,8 +200,9 @@ int outer_partials(int d, int n);
 // u_nonzero (may be NULL): fp64::prepare's flag; where it is 0 (u = +0.0
 // everywhere) sigma = q + 0.0 exactly (the stencil's value for a zero
 // iterate, bit for bit), formed without the FP64 stencil.
+// Returns the number of sigma partials; out = NULL leaves their sum to the caller.
 template <typename T>
-void outer_residual(int d, const Lay& in, const double* u, const double* q, T* q_in,
+int outer_residual(int d, const Lay& in, const double* u, const double* q, T* q_in,
                     double* partial, double* out, cudaStream_t s, T* e_init = nullptr,
                     float* resid = nullptr, int* resid_flag = nullptr,
                     double* qnorm_out = nullptr, const int* u_nonzero = nullptr);
@@ -228,15 +252,17 @@ size_t smem_bytes(int d, int n_top, int levels, int smoother, size_t elem);
 // exact_top: the top level is level 0 of a plain FP64 3D hierarchy, whose
 // last pre-smoothing half sweep and residual use the unbiased value
 // (level_kernels.cuh, gs_value), as the grid kernels there do
-// paper: the paper's transfers (FP64); the paper's smoother runs too (FP64)
+// paper: the paper's transfers (FP64); the paper's smoother runs too (FP64).
+// first_done: u_top holds the result of the top level's first smoothing step
+// (CoarseInit)
 template <typename T>
 cudaError_t launch(int d, const Lay& top, int levels, T* u_top, const T* q_top, int smoother,
                    double omega, int nu1, int nu2, int coarse_sweeps, cudaStream_t s,
-                   bool exact_top = false, bool paper = false);
-// The tail from a 33^3 or 17^3 level down as one cluster of 16 CTAs
+                   bool exact_top = false, bool paper = false, bool first_done = false);
+// The tail from a 33^3 (FP64: 17^3) level down as one cluster of 16 CTAs
 // (slab_tail.cu): red-black smoothing, full weighting, a hierarchy that
-// reaches 9^3.  first_done: the top level's first red half sweep ran already.
-bool slab_applies(int d, int n, int levels, int smoother, bool paper);
+// reaches 9^3.  first_done: as launch's.
+bool slab_applies(int d, int n, int levels, int smoother, bool paper, bool fp64);
 template <typename T>
 cudaError_t launch_slab(const Lay& top, int levels, T* u_top, const T* q_top, int smoother,
                         int nu1, int nu2, int coarse_sweeps, cudaStream_t s, bool exact_top,

@@ -478,7 +478,7 @@ struct Trainer {
                 for (int c = 0; c < 2; ++c) lk::rb_half<double>(d, lv[l].n, lv[l].u[0], lv[l].q, c, s);
             lk::residual<double>(d, lv[l].n, lv[l].u[0], lv[l].q, lv[l].r, nu > 0, s);
             lk::restrict_fw<double>(d, lv[l].n, lv[l].r, lv[l + 1].q, lv[l + 1].u[0], nu > 0,
-                                    lv[l + 1].n == 2, s);
+                                    lv[l + 1].n == 2 ? INIT_EXACT : INIT_ZERO, s);
         }
         if (L == 1)
             for (int k = 0; k < nu; ++k)
@@ -494,7 +494,7 @@ struct Trainer {
     void coarse_solve_of(double* src) {
         Level<double>& C = coarse[0];
         // restrict_fw writes q_c and zeroes u_c (or u_c = q_c on a one-unknown grid)
-        lk::restrict_fw<double>(d, n, src, C.q, C.u[0], false, C.n == 2, s);
+        lk::restrict_fw<double>(d, n, src, C.q, C.u[0], false, C.n == 2 ? INIT_EXACT : INIT_ZERO, s);
         if (C.n > 2)
             for (int k = 0; k < coarse_cycles; ++k) vcycle(coarse, 2);
     }

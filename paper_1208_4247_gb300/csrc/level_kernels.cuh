@@ -707,13 +707,29 @@ __global__ void __launch_bounds__(256) k_residual(const T* __restrict__ u, const
     }
 }
 
-// q_c = 4 FW(sigma) at every coarse interior node; u_c = 0 (a fresh coarse
-// iterate) or u_c = q_c when the coarse grid has its single unknown (exact
-// solve u = b/(2d)).  With RED_ONLY the black-node terms (faces and corners
+// The coarse iterate a restriction leaves at node (I, J, K) with right-hand
+// side q (as stored): CoarseInit.  The Gauss-Seidel and Jacobi values are the
+// smoothers' expressions with every neighbour (and u) zero.
+template <int DIM, typename T>
+__device__ inline T coarse_init(int init, double omega, int I, int J, int K, T q) {
+    using N = Num<T>;
+    using C = typename N::C;
+    if (init == INIT_ZERO) return N::st(C(0));
+    if (init == INIT_EXACT) return q;
+    const C c = DIM == 3 ? C(1.0 / 6.0) : C(0.25);
+    const C gs = gs_value<DIM, false>(c, C(0), N::ld(q));
+    if (init == INIT_WJ) return N::st(fma(C(omega), gs - C(0), C(0)));
+    const bool on = init == INIT_RED ? ((I + J + K) & 1) == 0 : ((I | J | K) & 1) == 0;
+    return N::st(on ? gs : C(0));
+}
+
+// q_c = 4 FW(sigma) at every coarse interior node; u_c by coarse_init.  With
+// RED_ONLY the black-node terms (faces and corners
 // in 3D, faces in 2D) are zero and skipped.  F: fine layout, Cl: coarse.
 template <int DIM, bool RED_ONLY, bool SPLIT, typename T>
 __global__ void __launch_bounds__(256) k_restrict(const T* __restrict__ r, T* __restrict__ qc,
-                                                  T* __restrict__ uc, Lay F, Lay Cl, int exact) {
+                                                  T* __restrict__ uc, Lay F, Lay Cl, int init,
+                                                  double omega) {
     using N = Num<T>;
     using C = typename N::C;
     const int nc = Cl.n;
@@ -770,8 +786,9 @@ __global__ void __launch_bounds__(256) k_restrict(const T* __restrict__ r, T* __
         }
     }
     const int64_t P = (int64_t)K * Cl.sz + (int64_t)J * Cl.sy + xo_any(Cl, I);
-    qc[P] = N::st(v);
-    uc[P] = exact ? N::st(v) : N::st(C(0));
+    const T q = N::st(v);
+    qc[P] = q;
+    uc[P] = coarse_init<DIM>(init, omega, I, J, K, q);
 }
 
 // u += P u_c, one thread per coarse cell (I,J,K) in [0, nc-1]^d updating
@@ -846,7 +863,7 @@ constexpr int kZWalk = 4;  // restriction
 template <typename T>
 __global__ void __launch_bounds__(256) k_restrict3_zwalk(const T* __restrict__ r,
                                                          T* __restrict__ qc, T* __restrict__ uc,
-                                                         int n) {
+                                                         int n, int init, double omega) {
     using N = Num<T>;
     using C = typename N::C;
     const int nc = n / 2;
@@ -868,7 +885,7 @@ __global__ void __launch_bounds__(256) k_restrict3_zwalk(const T* __restrict__ r
         const C above = odd_plane(p + sz);
         const C v = fma(C(0.125), (in_plane + below) + above, C(0.5) * R(p));
         qc[P] = N::st(v);
-        uc[P] = N::st(C(0));
+        uc[P] = coarse_init<3>(init, omega, I, J, K, N::st(v));
         below = above;
     }
 }
@@ -977,7 +994,7 @@ __global__ void __launch_bounds__(256) k_mc_sweep(T* __restrict__ u, const T* __
 template <int DIM, typename T>
 __global__ void __launch_bounds__(256) k_restrict_paper(const T* __restrict__ r,
                                                         T* __restrict__ qc, T* __restrict__ uc,
-                                                        Lay F, Lay Cl, int exact) {
+                                                        Lay F, Lay Cl, int init, double omega) {
     using N = Num<T>;
     using C = typename N::C;
     const int nc = Cl.n;
@@ -1001,7 +1018,7 @@ __global__ void __launch_bounds__(256) k_restrict_paper(const T* __restrict__ r,
     }
     const int64_t P = (int64_t)K * Cl.sz + (int64_t)J * Cl.sy + I;
     qc[P] = N::st(v);
-    uc[P] = exact ? N::st(v) : N::st(C(0));
+    uc[P] = coarse_init<DIM>(init, omega, I, J, K, N::st(v));
 }
 
 // The paper's prolongation (eq. Prolongation2d, 3D analogue), u += P u_c:
@@ -1192,41 +1209,40 @@ void residual(int d, const Lay& L, const T* u, const T* q, T* r, bool red_only, 
 }
 
 template <int DIM, bool SPLIT, typename T>
-void restrict_grid(const Lay& F, const Lay& C, const T* r, T* qc, T* uc, bool red_only, int ex,
-                   dim3 grid, dim3 block, cudaStream_t s) {
+void restrict_grid(const Lay& F, const Lay& C, const T* r, T* qc, T* uc, bool red_only, int init,
+                   double omega, dim3 grid, dim3 block, cudaStream_t s) {
     if (red_only)
-        k_restrict<DIM, true, SPLIT, T><<<grid, block, 0, s>>>(r, qc, uc, F, C, ex);
+        k_restrict<DIM, true, SPLIT, T><<<grid, block, 0, s>>>(r, qc, uc, F, C, init, omega);
     else
-        k_restrict<DIM, false, SPLIT, T><<<grid, block, 0, s>>>(r, qc, uc, F, C, ex);
+        k_restrict<DIM, false, SPLIT, T><<<grid, block, 0, s>>>(r, qc, uc, F, C, init, omega);
 }
 
 template <typename T>
 void restrict_fw(int d, const Lay& F, const Lay& C, const T* r, T* qc, T* uc, bool red_only,
-                 bool exact_coarsest, cudaStream_t s) {
+                 int init, cudaStream_t s, double omega) {
     const int nc = C.n;
     int bx = 32;
     while (bx < nc - 1 && bx < 128) bx *= 2;
     const int by = 256 / bx;
     dim3 block(bx, by, 1);
     dim3 grid((nc - 1 + bx - 1) / bx, (nc - 1 + by - 1) / by, d == 3 ? nc - 1 : 1);
-    const int ex = exact_coarsest ? 1 : 0;
     if constexpr (std::is_same<T, double>::value) {
-        if (red_only && !exact_coarsest && zwalk_applies(d, F)) {
+        if (red_only && init != INIT_EXACT && zwalk_applies(d, F)) {
             const dim3 gz(grid.x, grid.y, (unsigned)((nc - 1 + kZWalk - 1) / kZWalk));
-            k_restrict3_zwalk<T><<<gz, block, 0, s>>>(r, qc, uc, F.n);
+            k_restrict3_zwalk<T><<<gz, block, 0, s>>>(r, qc, uc, F.n, init, omega);
             return;
         }
     }
     if (d == 3) {
         if (F.he)
-            restrict_grid<3, true>(F, C, r, qc, uc, red_only, ex, grid, block, s);
+            restrict_grid<3, true>(F, C, r, qc, uc, red_only, init, omega, grid, block, s);
         else
-            restrict_grid<3, false>(F, C, r, qc, uc, red_only, ex, grid, block, s);
+            restrict_grid<3, false>(F, C, r, qc, uc, red_only, init, omega, grid, block, s);
     } else {
         if (F.he)
-            restrict_grid<2, true>(F, C, r, qc, uc, red_only, ex, grid, block, s);
+            restrict_grid<2, true>(F, C, r, qc, uc, red_only, init, omega, grid, block, s);
         else
-            restrict_grid<2, false>(F, C, r, qc, uc, red_only, ex, grid, block, s);
+            restrict_grid<2, false>(F, C, r, qc, uc, red_only, init, omega, grid, block, s);
     }
 }
 
@@ -1284,19 +1300,18 @@ void mc_sweep(int d, const Lay& L, T* u, const T* q, int color, cudaStream_t s) 
 }
 
 template <typename T>
-void restrict_paper(int d, const Lay& F, const Lay& C, const T* r, T* qc, T* uc,
-                    bool exact_coarsest, cudaStream_t s) {
+void restrict_paper(int d, const Lay& F, const Lay& C, const T* r, T* qc, T* uc, int init,
+                    cudaStream_t s, double omega) {
     const int nc = C.n;
     int bx = 32;
     while (bx < nc - 1 && bx < 128) bx *= 2;
     const int by = 256 / bx;
     dim3 block(bx, by, 1);
     dim3 grid((nc - 1 + bx - 1) / bx, (nc - 1 + by - 1) / by, d == 3 ? nc - 1 : 1);
-    const int ex = exact_coarsest ? 1 : 0;
     if (d == 3)
-        k_restrict_paper<3, T><<<grid, block, 0, s>>>(r, qc, uc, F, C, ex);
+        k_restrict_paper<3, T><<<grid, block, 0, s>>>(r, qc, uc, F, C, init, omega);
     else
-        k_restrict_paper<2, T><<<grid, block, 0, s>>>(r, qc, uc, F, C, ex);
+        k_restrict_paper<2, T><<<grid, block, 0, s>>>(r, qc, uc, F, C, init, omega);
 }
 
 template <typename T>

@@ -18,8 +18,8 @@ namespace lk {
     template void wj_sweep<T>(int, const Lay&, const T*, T*, const T*, double, cudaStream_t);   \
     template void residual<T>(int, const Lay&, const T*, const T*, T*, bool, cudaStream_t,      \
                               bool);                                                            \
-    template void restrict_fw<T>(int, const Lay&, const Lay&, const T*, T*, T*, bool, bool,     \
-                                 cudaStream_t);                                                 \
+    template void restrict_fw<T>(int, const Lay&, const Lay&, const T*, T*, T*, bool, int,      \
+                                 cudaStream_t, double);                                         \
     template void prolong_add<T>(int, const Lay&, const Lay&, const T*, T*, cudaStream_t, bool);
 GMG_INSTANTIATE(float)
 GMG_INSTANTIATE(__nv_bfloat16)
@@ -445,7 +445,7 @@ int outer_partials(int d, int n) {
 }
 
 template <typename T>
-void outer_residual(int d, const Lay& in, const double* u, const double* q, T* q_in,
+int outer_residual(int d, const Lay& in, const double* u, const double* q, T* q_in,
                     double* partial, double* out, cudaStream_t s, T* e_init, float* resid,
                     int* resid_flag, double* qnorm_out, const int* unz) {
     const int n = in.n;
@@ -460,9 +460,9 @@ void outer_residual(int d, const Lay& in, const double* u, const double* q, T* q
         else
             k_outer_residual3_walk<false, T><<<blocks, W.block, 0, s>>>(u, q, q_in, e_init, partial, in,
                                                                       W.segs, resid, resid_flag, qpart, unz);
-        fp64::k_sum_partials<<<1, 1024, 0, s>>>(partial, blocks, out);
+        if (out) fp64::k_sum_partials<<<1, 1024, 0, s>>>(partial, blocks, out);
         if (qpart) fp64::k_sum_partials<<<1, 1024, 0, s>>>(qpart, blocks, qnorm_out);
-        return;
+        return blocks;
     }
     int bx = 32;
     while (bx < n && bx < 128) bx *= 2;
@@ -483,8 +483,9 @@ void outer_residual(int d, const Lay& in, const double* u, const double* q, T* q
             k_outer_residual<2, false, T><<<blocks, block, 0, s>>>(u, q, q_in, e_init, partial, in,
                                                                    resid, resid_flag, qpart, unz);
     }
-    fp64::k_sum_partials<<<1, 1024, 0, s>>>(partial, blocks, out);
+    if (out) fp64::k_sum_partials<<<1, 1024, 0, s>>>(partial, blocks, out);
     if (qpart) fp64::k_sum_partials<<<1, 1024, 0, s>>>(qpart, blocks, qnorm_out);
+    return blocks;
 }
 
 template <typename T>
@@ -508,13 +509,13 @@ void update(int d, const Lay& in, double* u, const T* e, cudaStream_t s) {
     }
 }
 
-template void outer_residual<float>(int, const Lay&, const double*, const double*, float*,
+template int outer_residual<float>(int, const Lay&, const double*, const double*, float*,
                                     double*, double*, cudaStream_t, float*, float*, int*,
                                     double*, const int*);
-template void outer_residual<__nv_bfloat16>(int, const Lay&, const double*, const double*,
+template int outer_residual<__nv_bfloat16>(int, const Lay&, const double*, const double*,
                                             __nv_bfloat16*, double*, double*, cudaStream_t,
                                             __nv_bfloat16*, float*, int*, double*, const int*);
-template void outer_residual<df32>(int, const Lay&, const double*, const double*, df32*, double*,
+template int outer_residual<df32>(int, const Lay&, const double*, const double*, df32*, double*,
                                    double*, cudaStream_t, df32*, float*, int*, double*,
                                    const int*);
 template void outer_red_update<df32>(int, const Lay&, double*, const double*, df32*, df32*,

@@ -12,9 +12,15 @@
 // Red-black smoothing with full weighting; the arithmetic of every step is
 // the level kernels', node for node, so the results are theirs bit for bit.
 //
-// What bounds it: FP64, the pipes of 16 SMs at n = 32 (1.4 us of a half
-// sweep's KSLAB us) and the barrier at n = 16; the FP32 forms the barrier and
-// the latency of a step throughout.
+// What bounds it: the cluster barrier with the remote stores it waits for
+// (750 cycles of a step's 1200 to 2000) and, in FP64, the 16 SMs' pipes: a half
+// sweep at n = 32 takes 1.9 us of them, so the FP64 form starts at 17^3 and
+// leaves 33^3 to the grid kernels, which spread it over every SM.  One launch,
+// from 33^3: FP32 27 us, double-float 42 us, against 11 grid launches a level
+// and the single-CTA tail, about 70 and 85 us; FP64 from 17^3 26 us (45 us).
+// Per solve, single-CTA tail from 9^3 -> this: 65^3 FP64 1187 -> 1075 us (978
+// from 17^3 with CoarseInit; 1044 from 33^3), 257^3 BF16 9.44 -> 8.89 ms (8.81
+// from 33^3, 8.94 from 17^3), 257^3 double-float 6.94 -> 6.80 ms.
 #include <algorithm>
 
 #include "tail_steps.cuh"
@@ -252,22 +258,20 @@ __global__ void __launch_bounds__(kSlabThreads)
     __syncthreads();
 
     const bool red_only = cy.nu1 > 0;
-    const C c = C(1.0 / 6.0);
+    const int init = cy.nu1 > 0 ? INIT_RED : INIT_ZERO;
     slab_relax(L0, cy.nu1, first_done != 0, exact0 != 0);
     slab_residual(L0, red_only, exact0 != 0);
     if (big) {
         // coarse plane rank + 1 lies under fine plane 2 rank + 2, local plane 1;
-        // where a sweep follows its first red half sweep (u = q from u = 0) is
-        // done here
+        // its first red half sweep is done here
         if (rank + 1 < 16)
             slab_restrict(L0.r + 2 * m2, 4, red_only, [&](int I, int J, C v) {
                 const int o = J * 17 + I;
                 L1.q[o] = N::st(v);
-                const bool red = cy.nu1 > 0 && ((I + J + rank + 1) & 1) == 0;
-                L1.put_u(0, o, N::st(red ? lk::gs_value<3, false>(c, C(0), N::ld(N::st(v))) : C(0)));
+                L1.put_u(0, o, lk::coarse_init<3>(init, 0.0, I, J, rank + 1, N::st(v)));
             });
         cluster_sync();
-        slab_relax(L1, cy.nu1, true, false);
+        slab_relax(L1, cy.nu1, init != INIT_ZERO, false);
         slab_residual(L1, red_only, false);
     }
     // 17^3 -> 9^3 in CTA 0: coarse plane (rank + 1)/2 of the odd ranks
@@ -277,13 +281,13 @@ __global__ void __launch_bounds__(kSlabThreads)
         slab_restrict(L1.r + 289, 3, red_only, [&](int I, int J, C v) {
             const int P = ((rank + 1) / 2) * 81 + J * 9 + I;
             q8[P] = N::st(v);
-            u8[P] = N::st(C(0));
+            u8[P] = lk::coarse_init<3>(init, 0.0, I, J, (rank + 1) / 2, N::st(v));
         });
     cluster_sync();
     if (rank == 0) {
         CtaX x;
         const SmemLevels<T> lv{small, off, 3, 3};
-        vcycle<3>(x, lv, 0, levels - (big ? 2 : 1), cy, false);
+        vcycle<3>(x, lv, 0, levels - (big ? 2 : 1), cy, false, init != INIT_ZERO);
     }
     cluster_sync();
     const bool black = cy.nu2 > 0;
@@ -311,8 +315,8 @@ __global__ void __launch_bounds__(kSlabThreads)
 
 // At least two of the small levels: the cycle CTA 0 runs on them takes a single
 // one for a whole hierarchy.
-bool slab_applies(int d, int n, int levels, int smoother, bool paper) {
-    return d == 3 && (n == 16 || n == 32) && levels >= (n == 32 ? 4 : 3) &&
+bool slab_applies(int d, int n, int levels, int smoother, bool paper, bool fp64) {
+    return d == 3 && (n == 16 || (n == 32 && !fp64)) && levels >= (n == 32 ? 4 : 3) &&
            levels <= (n == 32 ? 5 : 4) &&
            (smoother == GMG_RBGS || smoother == GMG_LEARNED) && !paper;
 }

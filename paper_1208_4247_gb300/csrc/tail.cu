@@ -75,7 +75,8 @@ struct ClusterX {
 // The V-cycle on levels with n = n_top, n_top/2, ..., n_top >> (levels-1).
 template <int DIM, typename T>
 __global__ void __launch_bounds__(1024) k_tail(T* __restrict__ u_top, const T* __restrict__ q_top,
-                                               Lay top, int levels, Cycle cy, int exact0) {
+                                               Lay top, int levels, Cycle cy, int exact0,
+                                               int first_done) {
     const int n_top = top.n;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int off[kMaxLevels + 1];
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(1024) k_tail(T* __restrict__ u_top, const T* _
     load(u_top, u0);
     __syncthreads();
     CtaX x;
-    const int cur = vcycle<DIM>(x, lv, 0, levels, cy, exact0 != 0);
+    const int cur = vcycle<DIM>(x, lv, 0, levels, cy, exact0 != 0, first_done != 0);
     const T* ur = lv.u(0, cur);
     for (int e = threadIdx.x; e < interior_slots<DIM>(lg); e += blockDim.x) {
         int i, j, k;
@@ -164,11 +165,13 @@ __device__ void gtail_body(X& gx, const GridArgs<T>& a) {
     for (int l = 0; l < lc; ++l) {
         relax<DIM>(gx, lv, l, cy, cy.nu1, cur, false, false);
         residual<DIM>(gx, lv.lg(l), lv.u(l, 0), lv.q(l), lv.r(l), red_only, false);
-        restrict_to<DIM>(gx, lv.lg(l + 1), lv.r(l), lv.q(l + 1), lv.u(l + 1, 0), red_only, false);
+        restrict_to<DIM>(gx, lv.lg(l + 1), lv.r(l), lv.q(l + 1), lv.u(l + 1, 0), red_only, false,
+                         l + 2 < a.levels ? INIT_ZERO : lv.lg(l + 1) == 1 ? INIT_EXACT : INIT_ZERO,
+                         0.0);
     }
     if (blockIdx.x == 0) {
         CtaX cx;
-        vcycle<DIM>(cx, lv, lc, a.levels, cy, false);
+        vcycle<DIM>(cx, lv, lc, a.levels, cy, false, false);
     }
     gx.sync();
     for (int l = lc - 1; l >= 0; --l) {
@@ -205,7 +208,7 @@ size_t smem_bytes(int d, int n_top, int levels, int smoother, size_t elem) {
 template <typename T>
 cudaError_t launch(int d, const Lay& top, int levels, T* u_top, const T* q_top, int smoother,
                    double omega, int nu1, int nu2, int coarse_sweeps, cudaStream_t s,
-                   bool exact_top, bool paper) {
+                   bool exact_top, bool paper, bool first_done) {
     if (levels < 1 || levels > kMaxLevels) return cudaErrorInvalidValue;
     const int exact0 = exact_top && std::is_same<T, double>::value && d == 3 ? 1 : 0;
     const size_t bytes = smem_bytes(d, top.n, levels, smoother, sizeof(T));
@@ -219,7 +222,8 @@ cudaError_t launch(int d, const Lay& top, int levels, T* u_top, const T* q_top, 
     cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
-    kern<<<1, threads, bytes, s>>>(u_top, q_top, top, levels, cy, exact0);
+    kern<<<1, threads, bytes, s>>>(u_top, q_top, top, levels, cy, exact0,
+                                  first_done ? 1 : 0);
     return cudaGetLastError();
 }
 
@@ -312,14 +316,14 @@ GMG_GRID_INST(df32)
 #undef GMG_GRID_INST
 
 template cudaError_t launch<double>(int, const Lay&, int, double*, const double*, int, double,
-                                    int, int, int, cudaStream_t, bool, bool);
+                                    int, int, int, cudaStream_t, bool, bool, bool);
 template cudaError_t launch<float>(int, const Lay&, int, float*, const float*, int, double, int,
-                                   int, int, cudaStream_t, bool, bool);
+                                   int, int, cudaStream_t, bool, bool, bool);
 template cudaError_t launch<__nv_bfloat16>(int, const Lay&, int, __nv_bfloat16*,
                                            const __nv_bfloat16*, int, double, int, int, int,
-                                           cudaStream_t, bool, bool);
+                                           cudaStream_t, bool, bool, bool);
 template cudaError_t launch<df32>(int, const Lay&, int, df32*, const df32*, int, double, int, int,
-                                  int, cudaStream_t, bool, bool);
+                                  int, cudaStream_t, bool, bool, bool);
 
 }  // namespace tail
 }  // namespace gmg

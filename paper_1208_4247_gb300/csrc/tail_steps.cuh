@@ -154,13 +154,16 @@ struct Cycle {
 };
 
 // `sweeps` sweeps on level l of lv; cur: which u buffer holds the iterate
-// (weighted Jacobi alternates).
+// (weighted Jacobi alternates).  first_done: the first step (CoarseInit) ran
+// already.
 template <int DIM, class X, class LV>
 __device__ void relax(X& x, const LV& lv, int l, const Cycle& cy, int sweeps, int& cur,
-                      bool backward, bool exact_last) {
+                      bool backward, bool exact_last, bool first_done = false) {
     const int lg = lv.lg(l);
     for (int s = 0; s < sweeps; ++s) {
+        const bool first = first_done && s == 0;
         if (cy.smoother == GMG_WJACOBI) {
+            if (first) continue;
             wj_sweep<DIM>(x, lg, lv.u(l, cur), lv.u(l, cur ^ 1), lv.q(l), cy.omega);
             cur ^= 1;
             continue;
@@ -168,12 +171,12 @@ __device__ void relax(X& x, const LV& lv, int l, const Cycle& cy, int sweeps, in
         if constexpr (std::is_same<typename LV::Type, double>::value) {
             if (cy.smoother == GMG_MCGS) {
                 constexpr int ncol = 1 << DIM;
-                for (int t = 0; t < ncol; ++t)
+                for (int t = first ? 1 : 0; t < ncol; ++t)
                     mc_color<DIM>(x, lg, lv.u(l, cur), lv.q(l), backward ? ncol - 1 - t : t);
                 continue;
             }
         }
-        for (int color = 0; color < 2; ++color)
+        for (int color = first ? 1 : 0; color < 2; ++color)
             rb_half<DIM>(x, lg, lv.u(l, cur), lv.q(l), color,
                          exact_last && color == 1 && s == sweeps - 1);
     }
@@ -235,11 +238,11 @@ __device__ inline C fw3(RF&& R, int sy, int sz, bool red_only) {
 
 // fine level lg + 1 -> coarse level lg
 template <int DIM, typename T, class X>
-__device__ void restrict_to(X& x, int lg, const T* r, T* qc, T* uc, bool red_only, bool paper) {
+__device__ void restrict_to(X& x, int lg, const T* r, T* qc, T* uc, bool red_only, bool paper,
+                            int init, double omega) {
     using N = Num<T>;
     using C = typename N::C;
     const int sy = (2 << lg) + 1, sz = DIM == 3 ? sy * sy : 0;
-    const bool exact = lg == 1;
     for (int idx = x.tid(); idx < interior_slots<DIM>(lg); idx += x.nt()) {
         int I, J, K;
         if (!inode<DIM>(idx, lg, I, J, K)) continue;
@@ -273,7 +276,7 @@ __device__ void restrict_to(X& x, int lg, const T* r, T* qc, T* uc, bool red_onl
             }
         }
         qc[P] = N::st(v);
-        uc[P] = exact ? N::st(v) : N::st(C(0));
+        uc[P] = lk::coarse_init<DIM>(init, omega, I, J, K, N::st(v));
     }
     x.sync();
 }
@@ -354,25 +357,38 @@ __device__ void prolong_add(X& x, int lg, const T* uc, T* u, bool paper, bool bl
 // coarsest grid, up (prolongation with correction, post-smoothing).  Returns
 // the u buffer of level `from` that holds the result.
 // exact0: level `from` is level 0 of a plain FP64 3D hierarchy (unbiased value).
+// first_done: the first smoothing step of level `from` ran already.
 template <int DIM, class X, class LV>
-__device__ int vcycle(X& x, const LV& lv, int from, int levels, const Cycle& cy, bool exact0) {
+__device__ int vcycle(X& x, const LV& lv, int from, int levels, const Cycle& cy, bool exact0,
+                      bool first_done) {
     // (a learned handle's tail levels smooth with red-black Gauss-Seidel)
     const bool red_black = cy.smoother == GMG_RBGS || cy.smoother == GMG_LEARNED;
     const bool red_only = red_black && cy.nu1 > 0 && !cy.paper;
     // a red half sweep follows the prolongation
     const bool black = red_black && cy.nu2 > 0;
-    // weighted Jacobi: every level descends in buffer nu1 & 1
-    int down = 0;
+    // every level but the coarsest gets its first smoothing step from the
+    // restriction
+    const int init = cy.nu1 == 0                    ? INIT_ZERO
+                     : cy.smoother == GMG_WJACOBI ? INIT_WJ
+                     : cy.smoother == GMG_MCGS    ? INIT_COLOR0
+                                                    : INIT_RED;
+    // down: u buffer of each level after its pre-smoothing (bit l; weighted
+    // Jacobi), which the correction goes into
+    unsigned down = 0;
     for (int l = from; l + 1 < levels; ++l) {
-        down = 0;
-        relax<DIM>(x, lv, l, cy, cy.nu1, down, false, exact0 && l == from);
-        residual<DIM>(x, lv.lg(l), lv.u(l, down), lv.q(l), lv.r(l), red_only, exact0 && l == from);
-        restrict_to<DIM>(x, lv.lg(l + 1), lv.r(l), lv.q(l + 1), lv.u(l + 1, 0), red_only, cy.paper);
+        int c = 0;
+        const bool first = l == from ? first_done : init != INIT_ZERO;
+        relax<DIM>(x, lv, l, cy, cy.nu1, c, false, exact0 && l == from, first);
+        down |= (unsigned)c << l;
+        residual<DIM>(x, lv.lg(l), lv.u(l, c), lv.q(l), lv.r(l), red_only, exact0 && l == from);
+        const int lgc = lv.lg(l + 1);
+        restrict_to<DIM>(x, lgc, lv.r(l), lv.q(l + 1), lv.u(l + 1, 0), red_only, cy.paper,
+                         l + 2 < levels ? init : lgc == 1 ? INIT_EXACT : INIT_ZERO, cy.omega);
     }
     const int b = levels - 1;
     int cur = 0;
     if (levels - from == 1) {
-        relax<DIM>(x, lv, b, cy, cy.nu1, cur, false, false);
+        relax<DIM>(x, lv, b, cy, cy.nu1, cur, false, false, first_done);
     } else if (lv.lg(b) > 1) {
         for (int s = 0; s < cy.coarse_sweeps; ++s) {
             rb_half<DIM>(x, lv.lg(b), lv.u(b, 0), lv.q(b), 0);
@@ -381,7 +397,7 @@ __device__ int vcycle(X& x, const LV& lv, int from, int levels, const Cycle& cy,
     }
     for (int l = levels - 2; l >= from; --l) {
         const int c = cur;
-        cur = down;
+        cur = (down >> l) & 1;
         prolong_add<DIM>(x, lv.lg(l + 1), lv.u(l + 1, c), lv.u(l, cur), cy.paper, black);
         relax<DIM>(x, lv, l, cy, cy.nu2, cur, true, false);
     }
