@@ -327,8 +327,10 @@ std::pair<double, double> model(int kind, int d, int n, bool red_only, double w,
         case K_CONV2: return {N * 16 * (t ? 27 : 9), N * 3 * w};  // both convs, u read+write
         case K_TAIL: return {N * (t ? 40 : 30) * 8.0 / 7.0, N * 2 * w};
         case K_RB_FUSED: return {N * (t ? 6 : 4), N * 3 * w};  // read u, q; write u
-        case K_MC_SWEEP:  // one of 2^d colours: the colour's nodes updated
-            return {N / (t ? 8 : 4) * (t ? 6 : 4), N / (t ? 8 : 4) * (t ? 8 : 6) * w};
+        case K_MC_SWEEP: {  // 1 of 2^d colours, or (red_only) 2 of 4 / 3 of 8: their nodes updated
+            const double part = N / (t ? 8 : 4) * (red_only ? (t ? 3 : 2) : 1);
+            return {part * (t ? 6 : 4), part * (t ? 8 : 6) * w};
+        }
         case K_RESTRICT_PAPER: return {Nc * (t ? 16 : 8), N * w + Nc * 2 * w};
         case K_PROLONG_PAPER: return {cells * (t ? 14 : 6), Nc * w + N * 2 * w};
         case K_NORM_AHEAD:  // red nodes: sigma^2 and the update; read u, q (red); write u, save
@@ -418,11 +420,10 @@ void relax(gmg_handle h, std::vector<Level<T>>& lv, int l, int sweeps, int& cur,
         const bool first = first_done && s == 0;
         if constexpr (std::is_same<T, double>::value) {
             if (h->cfg.smoother == GMG_MCGS) {
-                const int ncol = d == 3 ? 8 : 4;
-                for (int t = first ? 1 : 0; t < ncol; ++t) {
-                    const int color = backward ? ncol - 1 - t : t;
-                    timed(h, K_MC_SWEEP, l, p, L.n, false,
-                          [&] { lk::mc_sweep<T>(d, L.lay, L.u[cur], L.q, color, h->stream); });
+                for (int t = first ? 1 : 0; t <= d; ++t) {
+                    const int bits = backward ? d - t : t;
+                    timed(h, K_MC_SWEEP, l, p, L.n, 2 * bits == d || (d == 3 && (bits == 1 || bits == 2)),
+                          [&] { lk::mc_sweep<T>(d, L.lay, L.u[cur], L.q, bits, h->stream); });
                 }
                 continue;
             }
@@ -478,8 +479,21 @@ bool leg_level(gmg_handle h, const std::vector<Level<T>>& lv, int l) {
     return l + 1 < (int)lv.size() && leg_possible<T>(h, lv[l].n) && lv[l].u[1] != nullptr;
 }
 
+// The 2D leg kernels (legs2d.cu) run an FP64 level of n intervals.
+template <typename T>
+bool leg2d_possible(gmg_handle h, int n) {
+    const gmg_config& c = h->cfg;
+    return std::is_same<T, double>::value && c.d == 2 && h->legs_mode > 0 &&
+           legs2d::applies(n, h->leg_nmax, c.smoother, c.nu1, c.nu2);
+}
+template <typename T>
+bool leg2d_level(gmg_handle h, const std::vector<Level<T>>& lv, int l) {
+    return l + 1 < (int)lv.size() && leg2d_possible<T>(h, lv[l].n) && lv[l].u[1] != nullptr;
+}
+
 // First level handled by the persistent tail kernel (L = none): the first
-// level with n <= 8 (3D) / 32 (2D) (GMG_TAIL_N overrides) whose tail arrays
+// level with n <= 8 (3D) / 32 (2D; 16 under levels with leg kernels)
+// (GMG_TAIL_N overrides) whose tail arrays
 // fit in 200 KB of shared memory, below every learned level, leaving at
 // least two tail levels.
 // Red-black 3D handles start it at 33^3 or 17^3 (as the cluster of
@@ -495,7 +509,10 @@ template <typename T>
 int tail_level(gmg_handle h, const std::vector<Level<T>>& lv) {
     const gmg_config& c = h->cfg;
     const int L = (int)lv.size();
-    const int nmax = h->tail_max > 0 ? h->tail_max : c.d != 3 ? 32 : 8;
+    const int nmax = h->tail_max > 0             ? h->tail_max
+                     : c.d == 3                  ? 8
+                     : leg2d_possible<T>(h, 32) ? 16
+                                                 : 32;
     int lo = 0;
     if (c.smoother == GMG_LEARNED)
         for (int l = 0; l < L && l < (int)h->lw.size(); ++l)
@@ -650,6 +667,28 @@ gmg_status enqueue_vcycle(gmg_handle h, std::vector<Level<T>>& lv, bool first_re
                 cur[l + 1] = 0;
                 continue;
             }
+            if constexpr (std::is_same<T, double>::value) {
+                if (leg2d_level<T>(h, lv, l)) {
+                    Level<T>& F = lv[l];
+                    Level<T>& C = lv[l + 1];
+                    const int init = level_init<T>(h, lv, l + 1);
+                    const bool paper = c.transfer == GMG_TRANSFER_PAPER;
+                    cudaError_t e = cudaSuccess;
+                    timed(
+                        h, K_LEG_DOWN, l, p, F.n, true,
+                        [&] {
+                            e = legs2d::down(F.n, c.smoother, c.nu1, done[l], c.omega, paper,
+                                             c.smoother == GMG_RBGS && !paper, init, F.u[cur[l]],
+                                             F.u[cur[l] ^ 1], F.q, C.q, C.u[0], h->stream);
+                        },
+                        1, 2 * c.nu1);
+                    GMG_CUDA_TRY(e);
+                    cur[l] ^= 1;
+                    cur[l + 1] = 0;
+                    done[l + 1] = init > INIT_EXACT;
+                    continue;
+                }
+            }
             // level 0 of the plain FP64 form: the residual of the full
             // iterate, unbiased in 3D (lk::gs_value)
             const bool unbiased = l == 0 && std::is_same<T, double>::value && d == 3;
@@ -728,17 +767,33 @@ gmg_status enqueue_vcycle(gmg_handle h, std::vector<Level<T>>& lv, bool first_re
                 cur[l] ^= 1;
                 continue;
             }
-            bool done = false;
+            if constexpr (std::is_same<T, double>::value) {
+                if (leg2d_level<T>(h, lv, l)) {
+                    cudaError_t e = cudaSuccess;
+                    timed(
+                        h, K_LEG_UP, l, p, F.n, true,
+                        [&] {
+                            e = legs2d::up(F.n, c.smoother, c.nu2, c.omega,
+                                           c.transfer == GMG_TRANSFER_PAPER, C.u[cur[l + 1]],
+                                           F.u[cur[l]], F.u[cur[l] ^ 1], F.q, h->stream);
+                        },
+                        1, 2 * c.nu2);
+                    GMG_CUDA_TRY(e);
+                    cur[l] ^= 1;
+                    continue;
+                }
+            }
+            bool prolonged = false;
             if constexpr (std::is_same<T, double>::value) {
                 if (c.transfer == GMG_TRANSFER_PAPER) {
                     timed(h, K_PROLONG_PAPER, l, p, F.n, false, [&] {
                         lk::prolong_paper<T>(d, C.lay, F.lay, C.u[cur[l + 1]], F.u[cur[l]],
                                              h->stream);
                     });
-                    done = true;
+                    prolonged = true;
                 }
             }
-            if (!done) {
+            if (!prolonged) {
                 const bool black = red_sweep_next<T>(h, c.nu2);
                 timed(h, K_PROLONG, l, p, F.n, black, [&] {
                     lk::prolong_add<T>(d, C.lay, F.lay, C.u[cur[l + 1]], F.u[cur[l]], h->stream,
@@ -1489,7 +1544,7 @@ gmg_status alloc_hierarchy(gmg_handle h, std::vector<Level<T>>& lv, int levels, 
         if (l > 0 || alloc_u0)
             if ((st = dev_alloc(h, &v.u[0], v.nodes)) != GMG_OK) return st;
         const bool pingpong =
-            c.smoother == GMG_WJACOBI || use_fused_rb<T>(h) || (l + 1 < levels && leg_possible<T>(h, v.n));
+            c.smoother == GMG_WJACOBI || use_fused_rb<T>(h) || (l + 1 < levels && (leg_possible<T>(h, v.n) || leg2d_possible<T>(h, v.n)));
         if (pingpong && (st = dev_alloc(h, &v.u[1], v.nodes)) != GMG_OK) return st;
         if ((st = dev_alloc(h, &v.q, v.nodes)) != GMG_OK) return st;
         const bool need_r = l + 1 < levels || c.smoother == GMG_LEARNED;

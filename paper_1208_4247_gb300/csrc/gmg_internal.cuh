@@ -105,10 +105,11 @@ template <typename T>
 void prolong_add(int d, const Lay& C, const Lay& F, const T* uc, T* u, cudaStream_t s,
                  bool black_only = false);
 
-// The paper's own variant on dense FP64 levels: one colour of the 4/8-colour
-// Gauss-Seidel, the 7/15-point restriction, the diagonal prolongation.
+// The paper's own variant on dense FP64 levels: the colours with `bits` set
+// bits of the 4/8-colour Gauss-Seidel, the 7/15-point restriction, the
+// diagonal prolongation.
 template <typename T>
-void mc_sweep(int d, const Lay& L, T* u, const T* q, int color, cudaStream_t s);
+void mc_sweep(int d, const Lay& L, T* u, const T* q, int bits, cudaStream_t s);
 template <typename T>
 void restrict_paper(int d, const Lay& F, const Lay& C, const T* r, T* qc, T* uc, int init,
                     cudaStream_t s, double omega = 0.0);
@@ -243,6 +244,19 @@ void df_red_restore(int d, const Lay& in, df32* e, const df32* r, const int* fla
 namespace fused {
 void rb_sweep3_f32(int n, const float* uin, float* uout, const float* q, cudaStream_t s);
 }  // namespace fused
+
+// One level of a 2D FP64 cycle as two launches (legs2d.cu): the pre-smoothing
+// steps, residual and restriction (u -> uo, q_c, u_c), and the prolongation
+// with correction and the post-smoothing steps (u -> uo).  nmax: the largest
+// n that takes them (0: where they beat a launch per step).
+namespace legs2d {
+bool applies(int n, int nmax, int smoother, int nu1, int nu2);
+cudaError_t down(int n, int smoother, int nu1, bool first_done, double omega, bool paper,
+                 bool red_only, int init, const double* u, double* uo, const double* q, double* qc,
+                 double* uc, cudaStream_t s);
+cudaError_t up(int n, int smoother, int nu2, double omega, bool paper, const double* uc,
+               const double* u, double* uo, const double* q, cudaStream_t s);
+}  // namespace legs2d
 
 // Persistent single-CTA tail (tail.cu): the V-cycle on levels n_top, n_top/2,
 // ... (levels of them) in shared memory; u_top in/out, q_top in.

@@ -966,22 +966,27 @@ __global__ void __launch_bounds__(256, 4) k_prolong3_zwalk(const T* __restrict__
 inline bool zwalk_applies(int d, const Lay& F) { return d == 3 && !F.he && F.n >= 128; }
 
 // ------------------------------------------- the paper's own variant
-// (dense levels).  Multi-colour Gauss-Seidel: the nodes of colour
-// (i&1) + 2(j&1) + 4(k&1) = color, one thread per node of the colour's rows.
+// (dense levels).  Multi-colour Gauss-Seidel with colour c = (i&1) + 2(j&1) +
+// 4(k&1): nodes of two colours are neighbours only if the colours differ in
+// one bit, so the colours with the same number of set bits do not touch, and
+// sweeping them together, by increasing number of bits, gives every node the
+// operands it has in the order 0 .. 2^d - 1 (a colour's neighbours with one bit
+// less come before it in both orders, those with one more after it): 3
+// launches a sweep in 2D and 4 in 3D instead of 4 and 8, the same bits.
+// Here: the nodes of the colours with `bits` set bits, one thread per node.
 template <int DIM, typename T>
 __global__ void __launch_bounds__(256) k_mc_sweep(T* __restrict__ u, const T* __restrict__ q,
-                                                  Lay L, int color) {
+                                                  Lay L, int bits) {
     using N = Num<T>;
     using C = typename N::C;
     const C c = DIM == 3 ? C(1.0 / 6.0) : C(0.25);
     const int n = L.n;
-    const int cx = color & 1, cy = (color >> 1) & 1, cz = (color >> 2) & 1;
-    // rows j = jb, jb+2, ... with j = cy (mod 2), j >= 1; planes likewise
-    const int j = (cy ? 1 : 2) + 2 * (int)(blockIdx.x * blockDim.y + threadIdx.y);
-    const int k = DIM == 3 ? (cz ? 1 : 2) + 2 * (int)blockIdx.y : 0;
-    if (j >= n || (DIM == 3 && k >= n)) return;
+    const int j = blockIdx.x * blockDim.y + threadIdx.y + 1;
+    const int k = DIM == 3 ? blockIdx.y + 1 : 0;
+    const int odd = bits - (j & 1) - (k & 1);  // i & 1 in this row
+    if (j >= n || odd < 0 || odd > 1) return;
     const int64_t row = k * L.sz + j * L.sy;
-    for (int i = (cx ? 1 : 2) + 2 * threadIdx.x; i < n; i += 2 * blockDim.x) {
+    for (int i = (odd ? 1 : 2) + 2 * threadIdx.x; i < n; i += 2 * blockDim.x) {
         const int64_t p = row + i;
         u[p] = N::st(fma(c, nbr_sum<DIM>(u, p, L.sy, L.sz), N::ld(q[p])));
     }
@@ -1286,17 +1291,12 @@ void prolong_add(int d, const Lay& C, const Lay& F, const T* uc, T* u, cudaStrea
 }
 
 template <typename T>
-void mc_sweep(int d, const Lay& L, T* u, const T* q, int color, cudaStream_t s) {
-    const int n = L.n;
-    int bx = 32;
-    while (bx < n / 2 && bx < 128) bx *= 2;
-    const int by = 256 / bx;
-    const int rows = n / 2;  // rows of one parity in 1..n-1 (at most n/2)
-    dim3 grid((unsigned)((rows + by - 1) / by), d == 3 ? (unsigned)(n / 2) : 1u, 1);
+void mc_sweep(int d, const Lay& L, T* u, const T* q, int bits, cudaStream_t s) {
+    const RowLaunch R = row_launch(d, L.n, L.n / 2);
     if (d == 3)
-        k_mc_sweep<3, T><<<grid, dim3(bx, by, 1), 0, s>>>(u, q, L, color);
+        k_mc_sweep<3, T><<<R.grid, R.block, 0, s>>>(u, q, L, bits);
     else
-        k_mc_sweep<2, T><<<grid, dim3(bx, by, 1), 0, s>>>(u, q, L, color);
+        k_mc_sweep<2, T><<<R.grid, R.block, 0, s>>>(u, q, L, bits);
 }
 
 template <typename T>

@@ -91,19 +91,21 @@ __device__ void rb_half(X& x, int lg, T* u, const T* q, int color, bool ex = fal
     x.sync();
 }
 
-// One colour (i&1) + 2(j&1) + 4(k&1) of the paper's Gauss-Seidel (FP64).
+// The colours (i&1) + 2(j&1) + 4(k&1) with `bits` set bits of the paper's
+// Gauss-Seidel (FP64; lk::k_mc_sweep), n/2 slots per row.
 template <int DIM, typename T, class X>
-__device__ void mc_color(X& x, int lg, T* u, const T* q, int color) {
+__device__ void mc_colors(X& x, int lg, T* u, const T* q, int bits) {
     using N = Num<T>;
     using C = typename N::C;
     const C c = DIM == 3 ? C(1.0 / 6.0) : C(0.25);
-    const int n = 1 << lg, h = n / 2 - 1;
+    const int n = 1 << lg;
     const int sy = n + 1, sz = DIM == 3 ? sy * sy : 0;
-    for (int idx = x.tid(); idx < 1 << (DIM * (lg - 1)); idx += x.nt()) {
-        const int i = 2 * (idx & h) + ((color & 1) ? 1 : 2);
-        const int j = 2 * ((idx >> (lg - 1)) & h) + ((color & 2) ? 1 : 2);
-        const int k = DIM == 3 ? 2 * (idx >> (2 * (lg - 1))) + ((color & 4) ? 1 : 2) : 0;
-        if (i >= n || j >= n || (DIM == 3 && k >= n)) continue;
+    for (int idx = x.tid(); idx < color_slots<DIM>(lg); idx += x.nt()) {
+        const int row = idx >> (lg - 1);
+        const int j = row & (n - 1), k = DIM == 3 ? row >> lg : 0;
+        const int odd = bits - (j & 1) - (k & 1);
+        const int i = 2 * (idx & (n / 2 - 1)) + (odd ? 1 : 2);
+        if (odd < 0 || odd > 1 || i >= n || j == 0 || (DIM == 3 && k == 0)) continue;
         const int p = node_at<DIM>(lg, i, j, k);
         u[p] = N::st(fma(c, lk::nbr_sum<DIM>(u, p, sy, sz), N::ld(q[p])));
     }
@@ -170,9 +172,8 @@ __device__ void relax(X& x, const LV& lv, int l, const Cycle& cy, int sweeps, in
         }
         if constexpr (std::is_same<typename LV::Type, double>::value) {
             if (cy.smoother == GMG_MCGS) {
-                constexpr int ncol = 1 << DIM;
-                for (int t = first ? 1 : 0; t < ncol; ++t)
-                    mc_color<DIM>(x, lg, lv.u(l, cur), lv.q(l), backward ? ncol - 1 - t : t);
+                for (int t = first ? 1 : 0; t <= DIM; ++t)
+                    mc_colors<DIM>(x, lg, lv.u(l, cur), lv.q(l), backward ? DIM - t : t);
                 continue;
             }
         }

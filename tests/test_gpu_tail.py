@@ -23,6 +23,10 @@ def cycles(monkeypatch, tail_n, d, n, kw, count=3):
     from paper_1208_4247_gb300.gmg import Solver
     build.build()
     monkeypatch.setenv("GMG_TAIL_N", str(tail_n))
+    if tail_n == 1:  # every level on grid kernels
+        monkeypatch.setenv("GMG_FUSED_LEGS", "0")
+    else:
+        monkeypatch.delenv("GMG_FUSED_LEGS", raising=False)
     f = torch.from_numpy(inputs.rhs_uniform(d, n, 11)).cuda()
     u = torch.from_numpy(inputs.rhs_uniform(d, n, 12)).cuda()
     with Solver(d, n, **kw) as S:
@@ -75,5 +79,29 @@ def test_slab_tail_equals_grid_kernels(monkeypatch, n, prec, kw):
         kw["inner_cycles"] = 2 if prec == "fp32" else 1
     ref, rel_ref = cycles(monkeypatch, 1, 3, n, kw)
     u, rel = cycles(monkeypatch, 0, 3, n, kw)
+    assert np.array_equal(u, ref), np.max(np.abs(u - ref))
+    assert rel == rel_ref
+
+
+LEGS = [(n, dict(smoother=sm, transfer=tr, nu1=nu1, nu2=nu2, **kw))
+        for sm, tr, nu1, nu2, kw in (
+            ("wjacobi", "fw", 2, 2, {}), ("wjacobi", "paper", 1, 3, {}), ("rbgs", "fw", 2, 2, {}),
+            ("rbgs", "fw", 1, 3, {"cycle": "fmg"}), ("rbgs", "paper", 3, 1, {}),
+            ("mcgs", "paper", 1, 1, {}), ("mcgs", "fw", 2, 1, {}), ("mcgs", "paper", 1, 2, {"cycle": "fmg"}))
+        for n in (32, 64, 128, 256, 512)]
+LEGS += [(1024, dict(smoother="mcgs", transfer="paper", nu1=1, nu2=1)),
+         (128, dict(smoother="wjacobi", nu1=6, nu2=6)), (64, dict(smoother="rbgs", nu1=2, nu2=2, levels=1)),
+         (64, dict(smoother="rbgs", nu1=2, nu2=2, levels=2, coarse_sweeps=7))]
+
+
+@pytest.mark.parametrize("n,kw", LEGS)
+def test_legs_2d_equal_grid_kernels(monkeypatch, n, kw):
+    """The 2D leg kernels (a level's down and up half as one launch each,
+    halos computed again) against a launch per step, bit for bit: every tile
+    size, each smoother with odd and even step counts, both transfers, the
+    first cycle a full-multigrid pass, hierarchies cut short."""
+    pytest.importorskip("torch")
+    ref, rel_ref = cycles(monkeypatch, 1, 2, n, kw)
+    u, rel = cycles(monkeypatch, 0, 2, n, kw)
     assert np.array_equal(u, ref), np.max(np.abs(u - ref))
     assert rel == rel_ref
