@@ -176,45 +176,108 @@ __device__ inline int64_t interior_node(int d, int n, int64_t idx) {
 
 // Weight-gradient partials over `rpb` consecutive interior rows, one thread
 // per (channel, tap):  KIND 1: sum_p gz_c(p) x(p + o_t);  KIND 2: sum_p gy(p)
-// relu(z_c(p + o_t)).  FP32 within the block, one double per (block, c, t).
+// relu(z_c(p + o_t)).  FP32 within the block, one double per (block, c, t),
+// the nodes in row order.
+// Each thread's sum is one chain of dependent FMAs, and a CTA of 216 of them
+// per SM is all there is at 65^3, so what matters is how fast a step's two
+// operands arrive: rows of up to kSeg nodes are staged in shared memory as
+// floats, converted (and ReLU'd) once instead of once per tap and channel --
+// the conversions from double run on the FP64 pipe (65^3: 235 -> 83 and 211
+// -> 148 us).
+constexpr int kSegW = 94;  // + 2 halo nodes: three 32-lane loads a row
+template <int DIM, int KIND>
+constexpr int wgrad_rows() {  // staged rows: the dense array's, then the channels'
+    return KIND == 1 ? (DIM == 3 ? 9 : 3) + H : 1 + H * (DIM == 3 ? 9 : 3);
+}
 template <int DIM, int KIND>
 __global__ void __launch_bounds__(256) k_wgrad(const double* __restrict__ dense,
                                                const float* __restrict__ chan, int n, int64_t zs,
                                                int rpb, double* __restrict__ partial) {
     constexpr int T = taps<DIM>();
+    constexpr int NB = DIM == 3 ? 9 : 3;          // neighbour rows (dy, dz)
+    constexpr int ND = KIND == 1 ? NB : 1;        // staged rows of the dense array
+    constexpr int NC = KIND == 1 ? 1 : NB;        // of each channel
+    // nodes i0 - 1 .. i0 + kSegW, rows 3 banks apart (W = 3 mod 32): a warp's 27
+    // taps of a channel, and the next channel's, lie in different banks
+    constexpr int W = kSegW + 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ float rows_s[wgrad_rows<DIM, KIND>() * W];
     const int ct = threadIdx.x;
-    if (ct >= H * T) return;
-    const int c = ct / T, t = ct % T;
+    const bool on = ct < H * T;
+    const int c = on ? ct / T : 0, t = on ? ct % T : 0;
     const int64_t sy = sy_of(n), sz = sz_of<DIM>(n);
-    const int64_t off = tap_offset<DIM>(t, sy, sz);
     const int64_t rows = DIM == 3 ? (int64_t)(n - 1) * (n - 1) : (n - 1);
     const int64_t r0 = (int64_t)blockIdx.x * rpb;
     const int64_t r1 = r0 + rpb < rows ? r0 + rpb : rows;
-    const float* ch = chan + c * zs;
+    // this thread's two operand rows; the tapped one starts at dx = t % 3
+    const float* plain = rows_s + (KIND == 1 ? ND + c : 0) * W + 1;
+    const float* tapped = rows_s + (KIND == 1 ? t / 3 : ND + c * NC + t / 3) * W + t % 3;
     float acc = 0.f;
     for (int64_t r = r0; r < r1; ++r) {
         const int j = (int)(r % (n - 1)) + 1;
         const int k = DIM == 3 ? (int)(r / (n - 1)) + 1 : 0;
-        const int64_t row = k * sz + j * sy;
-        for (int i = 1; i < n; ++i) {
-            const int64_t p = row + i;
-            if (KIND == 1)
-                acc = fmaf(ch[p], (float)dense[p + off], acc);
-            else
-                acc = fmaf((float)dense[p], fmaxf(ch[p + off], 0.f), acc);
+        for (int i0 = 1; i0 < n; i0 += kSegW) {
+            const int cnt = n - i0 < kSegW ? n - i0 : kSegW;
+            __syncthreads();
+            // element x of staged row g holds node i0 - 1 + x: a warp takes rows
+            // g = warp, warp + 8, .., four at a time
+            constexpr int R = wgrad_rows<DIM, KIND>();
+            for (int g0 = warp; g0 < R; g0 += 32) {
+                float v[4][3];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int g = g0 + 8 * q;
+                    if (g >= R) break;
+                    const bool is_dense = g < ND;
+                    const int h = is_dense ? g : g - ND;
+                    // neighbour row of the row's (j, k); the centre one if it is alone
+                    const int nb = is_dense == (KIND == 1) ? h % NB : NB / 2;
+                    const int dy = nb % 3 - 1, dz = DIM == 2 ? 0 : nb / 3 - 1;
+                    const int64_t p = (k + dz) * sz + (j + dy) * sy + i0 - 1;
+                    const float* cp = chan + (KIND == 1 ? h : h / NB) * zs;
+#pragma unroll
+                    for (int x3 = 0; x3 < 3; ++x3) {
+                        const int x = lane + 32 * x3;
+                        v[q][x3] = 0.f;
+                        if (x < cnt + 2)
+                            v[q][x3] = is_dense    ? (float)dense[p + x]
+                                       : KIND == 1 ? cp[p + x]
+                                                   : fmaxf(cp[p + x], 0.f);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int x3 = 0; x3 < 3; ++x3)
+                        if (g0 + 8 * q < R) rows_s[(g0 + 8 * q) * W + lane + 32 * x3] = v[q][x3];
+            }
+            __syncthreads();
+            if (!on) continue;
+#pragma unroll 8
+            for (int i = 0; i < cnt; ++i) acc = fmaf(plain[i], tapped[i], acc);
         }
     }
-    partial[(int64_t)blockIdx.x * (2 * H * T) + (KIND == 1 ? 0 : H * T) + ct] = (double)acc;
+    if (on)
+        partial[(int64_t)blockIdx.x * (2 * H * T) + (KIND == 1 ? 0 : H * T) + ct] = (double)acc;
 }
 
-// grad[i] += scale * sum_b partial[b][i] (fixed order) for the KIND's half
-__global__ void k_wgrad_reduce(const double* __restrict__ partial, int blocks, int half, int base,
-                               const double* __restrict__ scale_dev, double sign,
-                               double* __restrict__ grad) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= half) return;
+// grad[i] += scale * sum_b partial[b][i] (fixed order) for the KIND's half:
+// four strided sums per entry, added in order (one thread per entry and part).
+__global__ void __launch_bounds__(1024) k_wgrad_reduce(const double* __restrict__ partial,
+                                                       int blocks, int half, int base,
+                                                       const double* __restrict__ scale_dev,
+                                                       double sign, double* __restrict__ grad) {
+    __shared__ double part_sum[4][256];
+    const int i = threadIdx.x & 255, part = threadIdx.x >> 8;
     double s = 0.0;
-    for (int b = 0; b < blocks; ++b) s += partial[(int64_t)b * 2 * half + base + i];
+    if (i < half) {
+#pragma unroll 8
+        for (int b = part; b < blocks; b += 4) s += partial[(int64_t)b * 2 * half + base + i];
+    }
+    part_sum[part][i] = s;
+    __syncthreads();
+    if (part != 0 || i >= half) return;
+    s = ((part_sum[0][i] + part_sum[1][i]) + part_sum[2][i]) + part_sum[3][i];
     grad[base + i] += sign * scale_dev[0] * s;
 }
 
@@ -263,11 +326,12 @@ __global__ void __launch_bounds__(256) k_sumsq_partial(const double* __restrict_
 
 // scalars: out[0] = op(partials) ; op 0: sum ; 1: 2 / sum (gradient scale) ;
 // 2: acc[0] += sum * inv_den[0] / batch (loss)
-__global__ void k_scalar(const double* __restrict__ partial, int count, int op, double batch,
-                         const double* __restrict__ inv_den, double* __restrict__ out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double s = 0.0;
-    for (int i = 0; i < count; ++i) s += partial[i];
+__global__ void __launch_bounds__(1024) k_scalar(const double* __restrict__ partial, int count,
+                                                 int op, double batch,
+                                                 const double* __restrict__ inv_den,
+                                                 double* __restrict__ out) {
+    const double s = fp64::block_sum(partial, count);
+    if (threadIdx.x != 0) return;
     if (op == 0) out[0] = s;
     if (op == 1) out[0] = 2.0 / s;
     if (op == 2) out[0] += s * inv_den[0] * 0.5 / batch;
@@ -394,8 +458,8 @@ void wgrad(int d, int n, const double* x, const float* gz, const double* gy, con
         k_wgrad<2, 2><<<blocks, 256, 0, s>>>(gy, z, n, zs, rpb, partial);
     }
     const int half = H * T;
-    k_wgrad_reduce<<<1, 256, 0, s>>>(partial, blocks, half, 0, scale_dev, sign, grad);
-    k_wgrad_reduce<<<1, 256, 0, s>>>(partial, blocks, half, half, scale_dev, sign, grad);
+    k_wgrad_reduce<<<1, 1024, 0, s>>>(partial, blocks, half, 0, scale_dev, sign, grad);
+    k_wgrad_reduce<<<1, 1024, 0, s>>>(partial, blocks, half, half, scale_dev, sign, grad);
 }
 
 void scaled_apply(int d, int n, const double* e, double* out, cudaStream_t s) {
@@ -417,21 +481,24 @@ struct Trainer {
     float *z1 = nullptr, *z3 = nullptr, *gz = nullptr;
     double *partial = nullptr, *wpart = nullptr, *scal = nullptr;  // scal: [0] 1/||e0||^2*2, [1] loss
     double* grad = nullptr;
+    char* extra_mem = nullptr;
     std::vector<Level<double>> coarse;  // hierarchy of the n/2 grid (coarse solve)
     std::vector<Level<double>> pair;    // hierarchy of the n grid (sample generation)
-    std::vector<void*> allocs;
+    // one device allocation, dealt out in 256-byte steps: measured first (base
+    // NULL), then made
+    char* base = nullptr;
+    size_t used = 0;
 
     cudaError_t alloc(void** p, size_t bytes) {
-        cudaError_t e = cudaMalloc(p, bytes);
-        if (e != cudaSuccess) return e;
-        allocs.push_back(*p);
-        return cudaMemsetAsync(*p, 0, bytes, s);
+        *p = base ? base + used : nullptr;
+        used += (bytes + 255) / 256 * 256;
+        return cudaSuccess;
     }
     void release() {
-        for (void* p : allocs) cudaFree(p);
-        allocs.clear();
+        cudaFree(base);
+        base = nullptr;
     }
-    cudaError_t hierarchy(std::vector<Level<double>>& lv, int nn) {
+    void hierarchy(std::vector<Level<double>>& lv, int nn) {
         int L = 0;
         while ((2 << L) <= nn) ++L;
         lv.resize(L);
@@ -439,14 +506,27 @@ struct Trainer {
             lv[l].n = nn >> l;
             lv[l].nodes = nodes_of(d, lv[l].n);
             const size_t b = sizeof(double) * lv[l].nodes;
-            cudaError_t e;
-            if ((e = alloc((void**)&lv[l].u[0], b)) != cudaSuccess) return e;
-            if ((e = alloc((void**)&lv[l].q, b)) != cudaSuccess) return e;
-            if (l + 1 < L && (e = alloc((void**)&lv[l].r, b)) != cudaSuccess) return e;
+            alloc((void**)&lv[l].u[0], b);
+            if (leg_level(lv, l)) alloc((void**)&lv[l].u[1], b);
+            alloc((void**)&lv[l].q, b);
+            if (l + 1 < L) alloc((void**)&lv[l].r, b);
         }
-        return cudaSuccess;
     }
-    cudaError_t init(int d_, int n_, int cc, int pc, cudaStream_t st) {
+    void deal(size_t extra) {
+        used = 0;
+        const size_t b = sizeof(double) * nodes, bz = sizeof(float) * nodes * H;
+        for (double** p : {&e0, &e1, &e2, &e3, &s1, &s2, &s3, &g, &gx, &w}) alloc((void**)p, b);
+        for (float** p : {&z1, &z3, &gz}) alloc((void**)p, bz);
+        alloc((void**)&partial, sizeof(double) * 152 * 8);
+        alloc((void**)&wpart, sizeof(double) * wgrad_blocks(d, n) * 2 * H * T);
+        alloc((void**)&scal, sizeof(double) * 4);
+        alloc((void**)&grad, sizeof(double) * 2 * H * T);
+        hierarchy(coarse, n / 2);
+        if (pair_cycles >= 0) hierarchy(pair, n);
+        alloc((void**)&extra_mem, extra);
+    }
+    // pc < 0: no samples are drawn.  extra: bytes at extra_mem.  Everything zeroed.
+    cudaError_t init(int d_, int n_, int cc, int pc, size_t extra, cudaStream_t st) {
         d = d_;
         n = n_;
         T = d == 3 ? 27 : 9;
@@ -454,49 +534,82 @@ struct Trainer {
         pair_cycles = pc;
         s = st;
         nodes = nodes_of(d, n);
-        const size_t b = sizeof(double) * nodes, bz = sizeof(float) * nodes * H;
-        cudaError_t e = cudaSuccess;
-        for (double** p : {&e0, &e1, &e2, &e3, &s1, &s2, &s3, &g, &gx, &w})
-            if (e == cudaSuccess) e = alloc((void**)p, b);
-        for (float** p : {&z1, &z3, &gz})
-            if (e == cudaSuccess) e = alloc((void**)p, bz);
-        if (e == cudaSuccess) e = alloc((void**)&partial, sizeof(double) * 152 * 8);
-        if (e == cudaSuccess)
-            e = alloc((void**)&wpart, sizeof(double) * wgrad_blocks(d, n) * 2 * H * T);
-        if (e == cudaSuccess) e = alloc((void**)&scal, sizeof(double) * 4);
-        if (e == cudaSuccess) e = alloc((void**)&grad, sizeof(double) * 2 * H * T);
-        if (e == cudaSuccess) e = hierarchy(coarse, n / 2);
-        if (e == cudaSuccess) e = hierarchy(pair, n);
-        return e;
+        deal(extra);
+        const size_t total = used;
+        cudaError_t e = cudaMalloc((void**)&base, total);
+        if (e != cudaSuccess) {
+            base = nullptr;
+            return e;
+        }
+        deal(extra);
+        return cudaMemsetAsync(base, 0, total, s);
     }
 
-    // RB-GS V(nu,nu) cycle on hierarchy lv (level-0 iterate lv[0].u[0], rhs lv[0].q)
-    void vcycle(std::vector<Level<double>>& lv, int nu) {
+    bool leg_level(const std::vector<Level<double>>& lv, int l) const {
+        return d == 2 && l + 1 < (int)lv.size() &&
+               legs2d::applies(lv[l].n, 0, GMG_RBGS, 1, 1);
+    }
+    // RB-GS V(nu,nu) cycle on hierarchy lv (level-0 iterate lv[0].u[0], rhs
+    // lv[0].q) with the solver's kernels: grid kernels (2D: legs) and the
+    // cluster or single-CTA tail.  first_done: the first red half sweep ran.
+    void vcycle(std::vector<Level<double>>& lv, int nu, bool first_done = false) {
         const int L = (int)lv.size();
-        for (int l = 0; l + 1 < L; ++l) {
-            for (int k = 0; k < nu; ++k)
-                for (int c = 0; c < 2; ++c) lk::rb_half<double>(d, lv[l].n, lv[l].u[0], lv[l].q, c, s);
-            lk::residual<double>(d, lv[l].n, lv[l].u[0], lv[l].q, lv[l].r, nu > 0, s);
-            lk::restrict_fw<double>(d, lv[l].n, lv[l].r, lv[l + 1].q, lv[l + 1].u[0], nu > 0,
-                                    lv[l + 1].n == 2 ? INIT_EXACT : INIT_ZERO, s);
+        int lt = L;
+        for (int l = 0; l < L && lt == L; ++l)
+            if (nu > 0 && (tail::slab_applies(d, lv[l].n, L - l, GMG_RBGS, false, true) ||
+                           (lv[l].n <= (d == 3 ? 8 : 16) && L - l >= 2)))
+                lt = l;
+        std::vector<char> done(L + 1, 0);
+        done[0] = first_done;
+        int down = 0;  // levels run by grid kernels or legs
+        for (int l = 0; l < lt && l + 1 < L; ++l, ++down) {
+            Level<double>&F = lv[l], &C = lv[l + 1];
+            const int init = C.n == 2 ? INIT_EXACT : nu > 0 ? INIT_RED : INIT_ZERO;
+            done[l + 1] = init == INIT_RED;
+            if (leg_level(lv, l) && F.u[1]) {
+                legs2d::down(F.n, GMG_RBGS, nu, done[l], 0.0, false, true, init, F.u[0], F.u[1], F.q,
+                             C.q, C.u[0], s);
+                continue;
+            }
+            half_sweeps(F, nu, done[l]);
+            lk::residual<double>(d, F.n, F.u[0], F.q, F.r, nu > 0, s);
+            lk::restrict_fw<double>(d, F.n, F.r, C.q, C.u[0], nu > 0, init, s);
         }
-        if (L == 1)
-            for (int k = 0; k < nu; ++k)
-                for (int c = 0; c < 2; ++c) lk::rb_half<double>(d, lv[0].n, lv[0].u[0], lv[0].q, c, s);
-        for (int l = L - 2; l >= 0; --l) {
-            lk::prolong_add<double>(d, lv[l + 1].n, lv[l + 1].u[0], lv[l].u[0], s);
-            for (int k = 0; k < nu; ++k)
-                for (int c = 0; c < 2; ++c) lk::rb_half<double>(d, lv[l].n, lv[l].u[0], lv[l].q, c, s);
+        if (lt < L) {
+            Level<double>& t = lv[lt];
+            const Lay lay = dense_lay(d, t.n);
+            if (tail::slab_applies(d, t.n, L - lt, GMG_RBGS, false, true))
+                tail::launch_slab<double>(lay, L - lt, t.u[0], t.q, GMG_RBGS, nu, nu, 0, s, false,
+                                          done[lt]);
+            else
+                tail::launch<double>(d, lay, L - lt, t.u[0], t.q, GMG_RBGS, 0.8, nu, nu, 0, s, false,
+                                     false, done[lt]);
+        } else if (L == 1) {
+            half_sweeps(lv[0], nu, first_done);
         }
+        for (int l = down - 1; l >= 0; --l) {
+            Level<double>&F = lv[l], &C = lv[l + 1];
+            if (leg_level(lv, l) && F.u[1]) {
+                legs2d::up(F.n, GMG_RBGS, nu, 0.0, false, C.u[0], F.u[1], F.u[0], F.q, s);
+                continue;
+            }
+            lk::prolong_add<double>(d, C.n, C.u[0], F.u[0], s, nu > 0);
+            half_sweeps(F, nu, false);
+        }
+    }
+    void half_sweeps(Level<double>& F, int nu, bool first_done) {
+        for (int k = first_done ? 1 : 0; k < 2 * nu; ++k)
+            lk::rb_half<double>(d, F.n, F.u[0], F.q, k & 1, s);
     }
 
     // u_c = (2d) A_c'^{-1} q_c with q_c = 4 FW(src) restricted from src (fine)
     void coarse_solve_of(double* src) {
         Level<double>& C = coarse[0];
-        // restrict_fw writes q_c and zeroes u_c (or u_c = q_c on a one-unknown grid)
-        lk::restrict_fw<double>(d, n, src, C.q, C.u[0], false, C.n == 2 ? INIT_EXACT : INIT_ZERO, s);
+        // q_c, and u_c after the first red half sweep from zero (or u_c = q_c on a
+        // one-unknown grid)
+        lk::restrict_fw<double>(d, n, src, C.q, C.u[0], false, C.n == 2 ? INIT_EXACT : INIT_RED, s);
         if (C.n > 2)
-            for (int k = 0; k < coarse_cycles; ++k) vcycle(coarse, 2);
+            for (int k = 0; k < coarse_cycles; ++k) vcycle(coarse, 2, k == 0);
     }
 
     // e_out = e_in - P u_c (error-form coarse-grid correction), s2 = A'e_in/(2d)
@@ -529,7 +642,7 @@ struct Trainer {
     void sumsq(const double* x, int op, double batch) {
         const int blocks = flat_blocks(nodes);
         k_sumsq_partial<<<blocks, 256, 0, s>>>(x, nodes, partial);
-        k_scalar<<<1, 32, 0, s>>>(partial, blocks, op, batch, scal, op == 2 ? scal + 1 : scal);
+        k_scalar<<<1, 1024, 0, s>>>(partial, blocks, op, batch, scal, op == 2 ? scal + 1 : scal);
     }
 
     // loss (accumulated into scal[1] / batch) and, if want_grad, its
@@ -646,10 +759,9 @@ gmg_status gmg_learned_loss_grad(int d, int n, const float* weights, const doubl
     }
     Trainer tr;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    GMG_TRY_CUDA_RELEASE(tr.init(d, n, coarse_cycles, 0, s), tr);
-    const int W = 2 * H * tr.T;
-    float* wd = nullptr;
-    GMG_TRY_CUDA_RELEASE(tr.alloc((void**)&wd, sizeof(float) * 2 * W), tr);
+    const int W = 2 * H * (d == 3 ? 27 : 9);
+    GMG_TRY_CUDA_RELEASE(tr.init(d, n, coarse_cycles, -1, sizeof(float) * 2 * W, s), tr);
+    float* wd = reinterpret_cast<float*>(tr.extra_mem);
     GMG_TRY_CUDA_RELEASE(cudaMemcpyAsync(wd, weights, sizeof(float) * W, cudaMemcpyHostToDevice, s),
                          tr);
     k_round_bf16<<<(W + 255) / 256, 256, 0, s>>>(wd, wd + W, W);
@@ -687,14 +799,13 @@ gmg_status gmg_learned_train(int d, int n, int steps, int batch, int pair_cycles
     }
     Trainer tr;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    GMG_TRY_CUDA_RELEASE(tr.init(d, n, coarse_cycles, pair_cycles, s), tr);
-    const int W = 2 * H * tr.T;
-    float *master = nullptr, *work = nullptr;
-    double *m1 = nullptr, *m2 = nullptr;
-    GMG_TRY_CUDA_RELEASE(tr.alloc((void**)&master, sizeof(float) * W), tr);
-    GMG_TRY_CUDA_RELEASE(tr.alloc((void**)&work, sizeof(float) * W), tr);
-    GMG_TRY_CUDA_RELEASE(tr.alloc((void**)&m1, sizeof(double) * W), tr);
-    GMG_TRY_CUDA_RELEASE(tr.alloc((void**)&m2, sizeof(double) * W), tr);
+    const int W = 2 * H * (d == 3 ? 27 : 9);
+    GMG_TRY_CUDA_RELEASE(tr.init(d, n, coarse_cycles, pair_cycles,
+                                 (sizeof(float) + sizeof(double)) * 2 * W, s), tr);
+    double* m1 = reinterpret_cast<double*>(tr.extra_mem);
+    double* m2 = m1 + W;
+    float* master = reinterpret_cast<float*>(m2 + W);
+    float* work = master + W;
     GMG_TRY_CUDA_RELEASE(cudaMemcpyAsync(master, w_init, sizeof(float) * W, cudaMemcpyHostToDevice, s),
                          tr);
     k_round_bf16<<<(W + 255) / 256, 256, 0, s>>>(master, work, W);
