@@ -115,6 +115,20 @@ __host__ __device__ __forceinline__ split_t split(double x) {
     const float scale = bits_f((ex - (1075 - 127)) << 23);  // 2^(ex - 1075)
     return split_t{bits_f(hb), int_to_float(r) * scale};
 }
+
+// (float)x: x's 24 leading significand bits rounded to nearest even, as the
+// cast does (which takes a slot of the FP64 pipe).  Zero keeps its sign; results
+// outside the normal range, infinite and NaN operands take the cast.
+__host__ __device__ __forceinline__ float narrow(double x) {
+    const uint64_t b = d_bits(x);
+    const uint32_t a = (uint32_t)(b >> 32) & 0x7fffffffu, sign = (uint32_t)(b >> 32) & 0x80000000u;
+    if (a - 0x38100000u >= 0x47e00000u - 0x38100000u)
+        return (b << 1) == 0 ? bits_f(sign) : (float)x;
+    // exponent rebiased by 1023 - 127 (modulo 2^32), fraction cut to 23 bits
+    const uint32_t f = (uint32_t)(b >> 29) - (896u << 23);
+    const uint32_t rest = (uint32_t)b & 0x1fffffffu;
+    return bits_f(((f & 0x7fffffffu) + ((rest + 0x0fffffffu + (f & 1u)) >> 29)) | sign);
+}
 }  // namespace cvt
 
 // Round-to-nearest float operations that the compiler may not fuse or

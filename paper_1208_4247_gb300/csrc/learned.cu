@@ -18,6 +18,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "gmg_internal.cuh"
@@ -876,7 +877,7 @@ __device__ inline uint32_t pack_bf16(float lo, float hi) {
 }
 
 __device__ inline void mma_bf16(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
-    asm volatile(
+    asm(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
         "{%8,%9}, {%0,%1,%2,%3};\n"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
@@ -1026,193 +1027,305 @@ __global__ void __launch_bounds__(256) k_conv_tc(const double* __restrict__ sigm
 }
 
 // ---------------------------------------------------------------------------
-// z-streaming 3D network: u += N(sigma) with conv2 as a GEMM over taps.
+// z-streaming 3D network: u += N(sigma), the hidden layer in registers.
 //
-// A CTA owns a 14 x 14 column of output nodes and a chunk of planes and walks
-// the planes.  Per plane kk (with a one-plane halo on either side of the
-// chunk):
-//  1. conv1 on the 16 x 16 halo-1 nodes of plane kk: per 16-node row a
-//     [16 nodes x 48] x [48 x 8 channels] product, K = 9 (dz, dy) groups x 4
-//     dx slots (dx = -1, 0, +1, one zero-weight slot); sigma (planes kk-1 ..
-//     kk+1) sits in a ring of four BF16 planes stored twice (element e, and
-//     shifted by one), so each A register is one aligned 32-bit load (three
-//     mma.sync m16n8k16 BF16 per row);
-//  2. the ReLU'd accumulators, rounded to BF16, are directly the A operand
-//     of z = h W2 ([16 x 8(16)] x [16 x 32 taps], four mma): z[t][node], the
-//     contribution of the node's hidden vector to tap t, FP32, one plane in
-//     shared memory (zero outside the interior: h is zero there);
-//  3. each thread owns one output column (x, y) and adds plane kk's
-//     contributions to its three open outputs, planes kk+1, kk, kk-1 (taps
-//     dz = -1, 0, +1), in registers; plane kk-1 is then complete: u += y.
-// Sigma of plane kk+2 is fetched into registers while plane kk is computed.
+// A warp owns 14 x kR output columns and walks the planes of its CTA's chunk (one
+// halo plane on either side).  Per plane kk and per hidden row y of 16 halo-1
+// nodes (mma.sync m16n8k16 / m16n8k8, BF16 operands, FP32 sums):
+//  1. conv1 is a [16 nodes x 48] x [48 x 8 channels] product, K = 3 dy x 4 groups
+//     (three planes, one zero-weight group) x 4 dx slots (dx = -1, 0, +1, one
+//     zero-weight slot).  One sigma row is one A operand of four registers, used
+//     with the three dy's weights by the three hidden rows it belongs to: a
+//     lane loads 4 words a row instead of 12.  sigma sits in a ring of four BF16
+//     planes stored twice (element e, and shifted by one), so each pair is one
+//     aligned word.
+//  2. The ReLU'd accumulators, rounded to BF16, are the A operand of conv2 as
+//     they are: two rows' make K = 16.  Output row y takes rows y-1 .. y+1 as a
+//     pair in one m16n8k16 and one in m16n8k8; the columns are the three dx of the
+//     three open output planes (4 columns each: two n-tiles), and the FP32
+//     accumulators stay in the tensor core's registers from plane to plane.
+//     The output plane's number modulo 3 is its column group, so the B operands
+//     rotate (the plane loop is unrolled by 3) instead of the sums.
+//  3. The plane that is complete adds its three dx columns, shifted by one
+//     node against each other (4 shuffles a row), and u += y runs over full
+//     warps (an FP64 instruction costs the same with 8 lanes on).  The
+//     conversions from and to double run on the integer pipe, with the casts'
+//     results (df.cuh): as casts they took 30% of the FP64 pipe.
+// Nothing of the hidden layer goes through shared memory; the kernel this
+// replaces kept the 27 contributions of a node there and was bound by that: 501
+// us per application at 257^3 and 315 M warp instructions, 291 us and 139 M now.
+// What bounds it now is latency at two CTAs per SM (128 registers: 24 of them
+// weights, 32 accumulators): 47% of the issue slots, 31% of the tensor pipe.
 // The hidden activations and sigma enter the tensor cores in BF16, weights
-// are BF16, every sum is FP32 -- the numerics of k_conv_tc, with the taps of
-// conv2 summed in a different order.
-constexpr int ZS_T = 14;              // output tile (x and y)
-constexpr int ZS_H1 = ZS_T + 2;       // halo-1 width: 16 nodes = one mma row group
-constexpr int ZS_H2 = ZS_T + 4;       // halo-2 rows
-constexpr int ZS_SW = 20;             // smem row stride of a sigma plane (18 + pad)
-constexpr int ZS_SP = ZS_H2 * ZS_SW + 4;  // elements per sigma plane (+4: planes
-                                          // 182 words apart, not a multiple of 32 banks)
-constexpr int ZS_TS = 260;            // floats per tap of the z plane (256 nodes + pad)
-constexpr int ZS_ZP = 27 * ZS_TS;     // floats of the z plane
-constexpr int ZS_PLANES = 16;         // output planes per CTA
-constexpr int ZS_PF = (ZS_SP + 255) / 256;  // sigma elements fetched per thread
+// are BF16, every sum is FP32 -- the numerics of k_conv_tc, with the taps
+// summed in a different order.
+constexpr int kR = 4;                      // output rows per warp
+constexpr int kWX = 2, kWY = 4;            // warps of a CTA along x, y
+constexpr int kTX = 14 * kWX, kTY = kR * kWY;  // output tile
+constexpr int kSX = kTX + 4, kSY = kTY + 4;    // sigma tile (halo 2): kSX = 32
+constexpr int kSRow = kSX + 2;             // elements per row (the last pair's pad)
+// words per plane and to the shifted copy: 11 and 5 banks apart, so that a
+// warp's four runs of 5 words (two copies, two planes) rarely meet in a bank
+constexpr int kPlaneW = 363, kCopyW = 4 * kPlaneW + 25;
+constexpr int kSmemW = kCopyW + 4 * kPlaneW;
+static_assert(kSX == 32 && kSY * kSRow / 2 <= kPlaneW && kPlaneW % 32 == 11 && kCopyW % 32 == 5,
+              "sigma ring layout");
+constexpr int kPF = (kSX * kSY + 255) / 256;  // sigma elements fetched per thread
 
-constexpr size_t zs_smem_bytes() {
-    return sizeof(float) * ZS_ZP + sizeof(__nv_bfloat16) * 2 * 4 * ZS_SP;
+// d = A B, from zero accumulators
+__device__ inline void mma_bf16_first(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
+    asm(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+        "{%8,%9}, {%10,%10,%10,%10};\n"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+__device__ inline void mma_bf16_k8(float* c, uint32_t a0, uint32_t a1, uint32_t b0) {
+    asm(
+        "mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, "
+        "{%0,%1,%2,%3};\n"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(b0));
 }
 
-// sigma value of the halo-2 element m of plane k (0 outside the interior)
-__device__ inline float zs_sigma(const double* sigma, int64_t sy, int64_t sz, int n, int i0,
-                                 int j0, int k, int m) {
-    const int x2 = m % ZS_SW, y2 = m / ZS_SW;
-    const int i = i0 - 2 + x2, j = j0 - 2 + y2;
-    if (m >= ZS_SP || x2 >= ZS_H2 || y2 >= ZS_H2 || i < 1 || i >= n || j < 1 || j >= n || k < 1 || k >= n)
-        return 0.f;
-    return (float)sigma[(int64_t)k * sz + (int64_t)j * sy + i];
+// BF16 of max(lo, 0) and max(hi, 0) (rounding and the maximum commute; NaN -> 0)
+__device__ inline uint32_t relu_pack(float lo, float hi) {
+    const __nv_bfloat162 v = __hmax2(__floats2bfloat162_rn(lo, hi), __float2bfloat162_rn(0.f));
+    return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+// MODE 1: u += N(sigma);  MODE 0: u = N(sigma) (interior nodes)
 template <int MODE>
-__global__ void __launch_bounds__(256, 4) k_conv_zs(const double* __restrict__ sigma,
+__global__ void __launch_bounds__(256, 2) k_conv_zs(const double* __restrict__ sigma,
                                                     double* __restrict__ u, int n,
-                                                    const float* __restrict__ W) {
-    extern __shared__ __align__(16) unsigned char zs_smem[];
-    float* zp = reinterpret_cast<float*>(zs_smem);                         // [27][260]
-    __nv_bfloat16* sa = reinterpret_cast<__nv_bfloat16*>(zp + ZS_ZP);      // [4][SP]
-    __nv_bfloat16* sb = sa + 4 * ZS_SP;                                    // shifted copy
+                                                    const float* __restrict__ W, int planes) {
+    __shared__ __align__(16) uint32_t ring[kSmemW];
+    __shared__ float ybuf[8][kR][16];
+    __nv_bfloat16* sa = reinterpret_cast<__nv_bfloat16*>(ring);
+    __nv_bfloat16* sb = reinterpret_cast<__nv_bfloat16*>(ring + kCopyW);  // shifted copy
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int gid = lane >> 2, tig = lane & 3;
-    const int i0 = 1 + ZS_T * blockIdx.x, j0 = 1 + ZS_T * blockIdx.y;
-    const int k0 = 1 + ZS_PLANES * blockIdx.z;
-    const int kend = min(k0 + ZS_PLANES, n);  // output planes k0 .. kend-1
+    const int gid = lane >> 2, tig = lane & 3, hf = tig >> 1;
+    const int wx = warp % kWX, wy = warp / kWX;
+    const int i0 = 1 + kTX * blockIdx.x, j0 = 1 + kTY * blockIdx.y;
+    const int k0 = 1 + planes * blockIdx.z;
+    const int kend = min(k0 + planes, n);  // output planes k0 .. kend-1
     const int64_t sy = (int64_t)n + 1, sz = sy * sy;
 
-    // conv1 B operand: k = 16 kh + (0..15) -> group g = k / 4 (dz, dy), slot
-    // k % 4 (dx = slot - 1; slot 3 and groups >= 9 have weight 0)
+    for (int e = threadIdx.x; e < kSmemW; e += 256) ring[e] = 0u;
+
+    // conv1 B operands, one per dy: k = 0..7 are the lane halves' first planes (half
+    // 0 dz = -1, half 1 dz = +1), k = 8..15 their second (half 0 dz = 0, half 1 none)
     uint32_t b1w[3][2];
 #pragma unroll
-    for (int kh = 0; kh < 3; ++kh) {
-        auto w1 = [&](int g, int slot) {
-            return (g < 9 && slot < 3) ? W[gid * 27 + 3 * g + slot] : 0.f;
+    for (int dy = 0; dy < 3; ++dy) {
+        const int sl = 2 * (tig & 1);
+        auto w1 = [&](int dz, int slot) {
+            return slot < 3 ? W[gid * 27 + dz * 9 + dy * 3 + slot] : 0.f;
         };
-        const int g = 4 * kh + (tig >> 1), sl = 2 * (tig & 1);
-        b1w[kh][0] = pack_bf16(w1(g, sl), w1(g, sl + 1));
-        b1w[kh][1] = pack_bf16(w1(g + 2, sl), w1(g + 2, sl + 1));
+        const int dz0 = hf ? 2 : 0;
+        b1w[dy][0] = pack_bf16(w1(dz0, sl), w1(dz0, sl + 1));
+        b1w[dy][1] = hf ? 0u : pack_bf16(w1(1, sl), w1(1, sl + 1));
     }
-    // z-GEMM B operand: k = channel (8..15 zero), n = tap 8 jn + gid
-    uint32_t b2w[4];
+    // conv2 B operands [phase][n-tile][dy] of this lane's column
+    uint32_t b2w[3][2][3];
+    {
+        const float* W2 = W + 8 * 27;
 #pragma unroll
-    for (int jn = 0; jn < 4; ++jn) {
-        const int t = 8 * jn + gid;
-        auto w2 = [&](int c) { return t < 27 ? W[8 * 27 + c * 27 + t] : 0.f; };
-        b2w[jn] = pack_bf16(w2(2 * tig), w2(2 * tig + 1));
+        for (int ph = 0; ph < 3; ++ph)  // t % 3, t = plane - (k0 - 1)
+#pragma unroll
+            for (int tile = 0; tile < 2; ++tile) {
+                const int s = 2 * tile + (gid >> 2), dx = gid & 3;
+                // group s holds the output plane k0 + p with p % 3 = s, p = t, t - 1, t - 2
+                const int back = (ph - s + 3) % 3;  // 0: dz = -1, 1: dz = 0, 2: dz = +1
+#pragma unroll
+                for (int dy = 0; dy < 3; ++dy) {
+                    auto w2 = [&](int c) {
+                        return (s < 3 && dx < 3) ? W2[c * 27 + back * 9 + dy * 3 + dx] : 0.f;
+                    };
+                    b2w[ph][tile][dy] = pack_bf16(w2(2 * tig), w2(2 * tig + 1));
+                }
+            }
     }
 
-    float pf[ZS_PF];
-    auto fetch = [&](int k) {
+    // sigma tile elements of this thread (row m >> 5, column m & 31): offset in a
+    // plane of sigma (-1 outside the interior) and in a ring slot.  They stay
+    // doubles until they are stored, a plane later, so that nothing waits for
+    // the loads.
+    double pf[kPF];
+    int goff[kPF];
+    const int soff = (threadIdx.x >> 5) * kSRow + lane;  // element r: 8 r rows on
 #pragma unroll
-        for (int r = 0; r < ZS_PF; ++r)
-            pf[r] = zs_sigma(sigma, sy, sz, n, i0, j0, k, threadIdx.x + 256 * r);
+    for (int r = 0; r < kPF; ++r) {
+        const int m = threadIdx.x + 256 * r;
+        const int i = i0 - 2 + (m & 31), j = j0 - 2 + (m >> 5);
+        const bool in = m < kSX * kSY && i >= 1 && i < n && j >= 1 && j < n;
+        goff[r] = in ? j * (n + 1) + i : -1;
+    }
+    auto fetch = [&](int k) {
+        const double* plane = sigma + (int64_t)k * sz;
+        const bool kin = k >= 1 && k < n;
+#pragma unroll
+        for (int r = 0; r < kPF; ++r) pf[r] = kin && goff[r] >= 0 ? plane[goff[r]] : 0.0;
     };
     auto store = [&](int k) {  // the fetched plane k -> ring slot k & 3, both copies
-        __nv_bfloat16* a = sa + (k & 3) * ZS_SP;
-        __nv_bfloat16* b = sb + (k & 3) * ZS_SP;
+        __nv_bfloat16* a = sa + (k & 3) * 2 * kPlaneW;
+        __nv_bfloat16* b = sb + (k & 3) * 2 * kPlaneW;
 #pragma unroll
-        for (int r = 0; r < ZS_PF; ++r) {
+        for (int r = 0; r < kPF; ++r) {
             const int m = threadIdx.x + 256 * r;
-            if (m < ZS_SP) {
-                const __nv_bfloat16 v = __float2bfloat16_rn(pf[r]);
-                a[m] = v;
-                if (m > 0) b[m - 1] = v;
+            if (m < kSX * kSY) {
+                const __nv_bfloat16 v = __float2bfloat16_rn(cvt::narrow(pf[r]));
+                a[soff + 8 * r * kSRow] = v;
+                if (lane) b[soff + 8 * r * kSRow - 1] = v;
             }
         }
     };
+    __syncthreads();
     for (int k = k0 - 2; k <= k0; ++k) {
         fetch(k);
         store(k);
     }
     fetch(k0 + 1);
 
-    // this thread's conv1 rows are x = gid, gid + 8 of each 16-node row: the
-    // 32-bit pair of x-adjacent sigma values it reads starts at halo-2
-    // column x (dx = -1, 0) or x + 2 (dx = +1, pad); its parity is gid's
-    const int xoff = (tig & 1) ? 2 : 0;
-    const __nv_bfloat16* src = (gid & 1) ? sb : sa;
-    const int sh = (gid & 1) ? -1 : 0;  // element index in the chosen copy
-    // the output column of this thread and its open sums (planes kk-1, kk, kk+1)
-    const bool owner = threadIdx.x < ZS_T * ZS_T;
-    const int ox = threadIdx.x % ZS_T, oy = threadIdx.x / ZS_T;
-    const bool col_in = owner && i0 + ox < n && j0 + oy < n;
-    float y_prev = 0.f, y_cur = 0.f, y_next = 0.f;
-    for (int kk = k0 - 1; kk <= kend; ++kk) {
-        // u of the output finished this plane, read early (used after conv1)
-        const int64_t po = (int64_t)(kk - 1) * sz + (int64_t)(j0 + oy) * sy + i0 + ox;
-        const bool out = col_in && kk - 1 >= k0;
-        const double u_old = (MODE == 1 && out) ? u[po] : 0.0;
-        __syncthreads();  // sigma planes kk-1 .. kk+1 stored; z plane free
-        for (int ry = warp; ry < ZS_H1; ry += 8) {
-            const int j = j0 - 1 + ry;
-            const bool yk = j >= 1 && j < n && kk >= 1 && kk < n;
-            const int ia = i0 - 1 + gid, ib = ia + 8;
-            const bool ina = yk && ia >= 1 && ia < n, inb = yk && ib >= 1 && ib < n;
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
+    // the word of this lane's first node (x = gid) in row 0 of the warp's sigma rows:
+    // columns x + (0, 1) for tig even, x + (2, 3) for tig odd
+    const uint32_t* src = ring + ((gid & 1) ? kCopyW : 0) +
+                          (kR * wy * kSRow + 14 * wx + gid - (gid & 1) + 2 * (tig & 1)) / 2;
+    // hidden nodes outside the interior are zero: masks of the warp's two node
+    // sets and its first and last row, for the warps that have any outside
+    const int ia = i0 - 1 + 14 * wx + gid;
+    const uint32_t xm0 = ia >= 1 && ia < n ? ~0u : 0u, xm1 = ia + 8 >= 1 && ia + 8 < n ? ~0u : 0u;
+    const int jw = j0 - 1 + kR * wy;  // global row of hidden row 0
+    const bool edge_warp = i0 - 1 + 14 * wx < 1 || i0 - 1 + 14 * wx + 15 >= n || jw < 1 ||
+                           jw + kR + 1 >= n;
+
+    // the two outputs of this lane: rows o / 14, columns o % 14 of the warp's tile
+    int ooff[2];
+    const float* yout[2];
 #pragma unroll
-            for (int kh = 0; kh < 3; ++kh) {
-                uint32_t a[4];
+    for (int h = 0; h < 2; ++h) {
+        const int o = lane + 32 * h;
+        const int i = i0 + 14 * wx + o % 14, j = j0 + kR * wy + o / 14;
+        ooff[h] = o < 14 * kR && i < n && j < n ? j * (n + 1) + i : -1;
+        yout[h] = &ybuf[warp][o / 14 % kR][1 + o % 14];
+    }
+
+    float acc[kR][2][4];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    int g = 4 * kh + (tig >> 1) + 2 * h;
-                    if (g >= 9) g = 4;  // zero-weight group: any in-tile pair
-                    const int dz = g / 3 - 1, dy = g % 3 - 1;
-                    const int e = ((kk + dz) & 3) * ZS_SP + (ry + 1 + dy) * ZS_SW + xoff + sh;
-                    a[2 * h] = *reinterpret_cast<const uint32_t*>(src + e + gid);
-                    a[2 * h + 1] = *reinterpret_cast<const uint32_t*>(src + e + gid + 8);
+    for (int y = 0; y < kR; ++y)
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[y][t][e] = 0.f;
+
+    // plane kk, the PH-th modulo 3 from k0 - 1 on
+    auto plane_step = [&](auto phase, int kk) {
+        constexpr int PH = decltype(phase)::value;
+        constexpr int FIN = (PH + 1) % 3;       // the column group complete after this plane
+        constexpr int FT = FIN == 2 ? 1 : 0;    // its n-tile
+        constexpr int FL = FIN == 1 ? 2 : 0;    // its lanes: tig = FL (dx = -1, 0), FL + 1 (+1)
+        // u of the outputs finished this plane, read early
+        double* uo = u + (int64_t)(kk - 1) * sz;
+        const bool out = kk - 1 >= k0;
+        double u_old[2] = {0.0, 0.0};
+        if (MODE == 1 && out) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (ooff[h] >= 0) u_old[h] = uo[ooff[h]];
+        }
+        __syncthreads();  // sigma planes kk-1 .. kk+1 stored
+        const bool kin = kk >= 1 && kk < n, masked = edge_warp || !kin;
+        // this lane's planes: half 0 kk-1 and kk, half 1 kk+1 (twice)
+        const uint32_t* p0 = src + ((kk + (hf ? 1 : -1)) & 3) * kPlaneW;
+        const uint32_t* p1 = src + ((kk + hf) & 3) * kPlaneW;
+        // sigma row r of the warp as conv1's A operand: nodes gid, gid + 8 of the two
+        // planes (the same registers serve the three hidden rows it belongs to)
+        uint32_t sg[3][4];
+        auto load_row = [&](int r) {
+            sg[r % 3][0] = p0[r * (kSRow / 2)];
+            sg[r % 3][1] = p0[r * (kSRow / 2) + 4];
+            sg[r % 3][2] = p1[r * (kSRow / 2)];
+            sg[r % 3][3] = p1[r * (kSRow / 2) + 4];
+        };
+        load_row(0);
+        load_row(1);
+        // hidden rows of the nodes gid, gid + 8, two rows to an A operand; two rows at
+        // a time, so that two to four independent products are in flight
+        uint32_t h[(kR + 2) / 2][4];
+#pragma unroll
+        for (int hp = 0; hp < (kR + 2) / 2; ++hp) {
+            const int ra = 2 * hp;  // rows ra, ra + 1
+            load_row(ra + 2);
+            uint32_t last[4] = {p0[(ra + 3) * (kSRow / 2)], p0[(ra + 3) * (kSRow / 2) + 4],
+                                p1[(ra + 3) * (kSRow / 2)], p1[(ra + 3) * (kSRow / 2) + 4]};
+            float ca[4], cb[4];
+            mma_bf16_first(ca, sg[ra % 3], b1w[0][0], b1w[0][1]);
+            mma_bf16_first(cb, sg[(ra + 1) % 3], b1w[0][0], b1w[0][1]);
+            mma_bf16(ca, sg[(ra + 1) % 3], b1w[1][0], b1w[1][1]);
+            mma_bf16(cb, sg[(ra + 2) % 3], b1w[1][0], b1w[1][1]);
+            mma_bf16(ca, sg[(ra + 2) % 3], b1w[2][0], b1w[2][1]);
+            mma_bf16(cb, last, b1w[2][0], b1w[2][1]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) sg[ra % 3][e] = last[e];  // row ra + 3
+            h[hp][0] = relu_pack(ca[0], ca[1]);
+            h[hp][1] = relu_pack(ca[2], ca[3]);
+            h[hp][2] = relu_pack(cb[0], cb[1]);
+            h[hp][3] = relu_pack(cb[2], cb[3]);
+            if (masked) {
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const int j = jw + ra + r;
+                    const uint32_t ym = kin && j >= 1 && j < n ? ~0u : 0u;
+                    h[hp][2 * r] &= xm0 & ym;
+                    h[hp][2 * r + 1] &= xm1 & ym;
                 }
-                mma_bf16(c, a, b1w[kh][0], b1w[kh][1]);
             }
-            uint32_t ah[4];
-            ah[0] = ina ? pack_bf16(fmaxf(c[0], 0.f), fmaxf(c[1], 0.f)) : 0u;
-            ah[1] = inb ? pack_bf16(fmaxf(c[2], 0.f), fmaxf(c[3], 0.f)) : 0u;
-            ah[2] = 0u;
-            ah[3] = 0u;
+            if (hp == 0) continue;
+            // output rows ya = ra - 2 (hidden rows ra - 2, ra - 1 | ra) and yb = ra - 1
+            // (ra - 1 | ra, ra + 1): a pair of rows that shares an operand in one
+            // m16n8k16, the third in one m16n8k8
+            const int ya = ra - 2, yb = ra - 1;
 #pragma unroll
-            for (int jn = 0; jn < 4; ++jn) {
-                float z[4] = {0.f, 0.f, 0.f, 0.f};
-                mma_bf16(z, ah, b2w[jn], 0u);
-                const int t = 8 * jn + 2 * tig;
-                float* zt = zp + t * ZS_TS + ry * ZS_H1;
-                if (t < 27) {
-                    zt[gid] = z[0];
-                    zt[gid + 8] = z[2];
-                }
-                if (t + 1 < 27) {
-                    zt[ZS_TS + gid] = z[1];
-                    zt[ZS_TS + gid + 8] = z[3];
-                }
+            for (int t = 0; t < 2; ++t) {
+                mma_bf16(acc[ya][t], h[hp - 1], b2w[PH][t][0], b2w[PH][t][1]);
+                mma_bf16(acc[yb][t], h[hp], b2w[PH][t][1], b2w[PH][t][2]);
+            }
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                mma_bf16_k8(acc[ya][t], h[hp][0], h[hp][1], b2w[PH][t][2]);
+                mma_bf16_k8(acc[yb][t], h[hp - 1][2], h[hp - 1][3], b2w[PH][t][0]);
             }
         }
-        store(kk + 2);  // slot (kk+2) & 3 is not read by this plane's conv1
+        // out(x) = [x-1][dx = -1] + [x][0] + [x+1][+1] of group FIN, nodes x = gid, gid + 8
+#pragma unroll
+        for (int y = 0; y < kR; ++y) {
+            float* d = acc[y][FT];
+            const float m0 = __shfl_sync(0xffffffffu, d[0], (lane - 4) & 31);
+            const float m1 = __shfl_sync(0xffffffffu, d[2], (lane - 4) & 31);
+            const float q0 = __shfl_sync(0xffffffffu, d[0], (lane + 5) & 31);
+            const float q1 = __shfl_sync(0xffffffffu, d[2], (lane + 5) & 31);
+            if (tig == FL) {
+                ybuf[warp][y][gid] = (m0 + d[1]) + (gid == 7 ? q1 : q0);
+                ybuf[warp][y][gid + 8] = ((gid == 0 ? m0 : m1) + d[3]) + q1;
+            }
+            // the group starts its next plane from zero
+#pragma unroll
+            for (int e = 0; e < 4; ++e) d[e] = FIN == 2 || hf == FIN ? 0.f : d[e];
+        }
+        store(kk + 2);  // slot (kk + 2) & 3 is not read by this plane's conv1
         fetch(kk + 3);
-        __syncthreads();  // z plane kk complete
-        if (col_in) {
-            // plane kk's taps: dz = +1 -> output kk-1, 0 -> kk, -1 -> kk+1
+        __syncwarp();
+        if (out) {
 #pragma unroll
-            for (int t = 0; t < 27; ++t) {
-                const int dx = t % 3 - 1, dy = (t / 3) % 3 - 1, dz = t / 9 - 1;
-                const float v = zp[t * ZS_TS + (oy + 1 + dy) * ZS_H1 + ox + 1 + dx];
-                if (dz == 1)
-                    y_prev += v;
-                else if (dz == 0)
-                    y_cur += v;
-                else
-                    y_next += v;
-            }
-            if (out) u[po] = u_old + (double)y_prev;
+            for (int e = 0; e < 2; ++e)
+                if (ooff[e] >= 0) uo[ooff[e]] = u_old[e] + cvt::widen(*yout[e]);
         }
-        y_prev = y_cur;
-        y_cur = y_next;
-        y_next = 0.f;
+        __syncwarp();
+    };
+    for (int kk = k0 - 1; kk <= kend; kk += 3) {
+        plane_step(std::integral_constant<int, 0>{}, kk);
+        if (kk + 1 <= kend) plane_step(std::integral_constant<int, 1>{}, kk + 1);
+        if (kk + 2 <= kend) plane_step(std::integral_constant<int, 2>{}, kk + 2);
     }
 }
 
@@ -1231,12 +1344,25 @@ bool conv_zs_enabled() {
 void conv_tc(int d, int n, const double* sigma, double* u, int mode, const float* W,
              cudaStream_t s) {
     if (d == 3 && conv_zs_enabled()) {
-        const size_t bytes = zs_smem_bytes();
-        auto kern = mode == 1 ? k_conv_zs<1> : k_conv_zs<0>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        dim3 grid((n - 1 + ZS_T - 1) / ZS_T, (n - 1 + ZS_T - 1) / ZS_T,
-                  (n - 1 + ZS_PLANES - 1) / ZS_PLANES);
-        kern<<<grid, 256, bytes, s>>>(sigma, u, n, W);
+        // planes per CTA: the number with the fewest plane steps in all waves of two
+        // CTAs per SM, where a CTA also computes two halo planes and spends
+        // about four steps' time on its operands
+        const int tx = (n - 1 + kTX - 1) / kTX, ty = (n - 1 + kTY - 1) / kTY;
+        int planes = 2;
+        int64_t best = INT64_MAX;
+        for (int p = 2; p <= 64; ++p) {
+            const int64_t ctas = (int64_t)tx * ty * ((n - 1 + p - 1) / p);
+            const int64_t steps = (ctas + 2 * 152 - 1) / (2 * 152) * (p + 6);
+            if (steps < best) {
+                best = steps;
+                planes = p;
+            }
+        }
+        const dim3 grid(tx, ty, (n - 1 + planes - 1) / planes);
+        if (mode == 1)
+            k_conv_zs<1><<<grid, 256, 0, s>>>(sigma, u, n, W, planes);
+        else
+            k_conv_zs<0><<<grid, 256, 0, s>>>(sigma, u, n, W, planes);
         return;
     }
     if (d == 3) {
