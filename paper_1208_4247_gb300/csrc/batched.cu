@@ -17,6 +17,7 @@
 #include <string>
 #include <vector>
 
+#include "batch_tiles.h"
 #include "gmg_internal.cuh"
 #include "level_kernels.cuh"
 #include "timing.cuh"
@@ -139,7 +140,9 @@ __device__ inline int64_t group_of(const BLevel& L, uint32_t gid, int& x0, int& 
 // nodes are written back unchanged, and no other thread writes them).  Per
 // group: one 16-byte load each of the row, its y and z neighbour rows and q,
 // the two x neighbours beyond the group as single loads, one 16-byte store;
-// nodes outside 1..n-1 are written as 0 (Jacobi) or left unchanged.  The
+// nodes outside 1..n-1 are written as 0 (Jacobi) or left unchanged.  zero: bit
+// 0 / 1: the source is zero on the solves' finest level / coarser levels and is
+// not read (Jacobi).  The
 // neighbour sum is ((x- + x+) + y- + y+) + z- + z+ in this order.  pool_in and pool_out are the
 // same pool: what a launch reads through pool_in is never written during the
 // launch (the Jacobi source, q; in red-black the other colour).
@@ -150,7 +153,7 @@ __global__ void __launch_bounds__(256) k_smooth(const Item* __restrict__ items, 
                                                 const T* __restrict__ pool_in,
                                                 T* __restrict__ pool_out,
                                                 const int* __restrict__ active, int src, int dst,
-                                                int color, float omega2, float omega3) {
+                                                int color, int zero, float omega2, float omega3) {
     constexpr int V = 16 / (int)sizeof(T);
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const Item w = items[it];
@@ -159,20 +162,25 @@ __global__ void __launch_bounds__(256) k_smooth(const Item* __restrict__ items, 
         const bool three = L.d == 3;
         const float c = three ? 1.f / 6.f : 0.25f;
         const float omega = three ? omega3 : omega2;
+        const bool zs = (zero >> (w.level > 0)) & 1;
         const T* u = pool_in + off_u(L, src);
         T* uo = pool_out + off_u(L, dst);
         const T* q = pool_in + L.q;
         for (int t = threadIdx.x; t < w.count; t += blockDim.x) {
             int x0, j, k;
             const int64_t p = group_of<V>(L, (uint32_t)(w.start + t), x0, j, k);
-            float x[V], ym[V], yp[V], zm[V], zp[V], qv[V], out[V];
-            ldv(u + p, x);
-            const float xl = Num<T>::ld(u[p - 1]), xr = Num<T>::ld(u[p + V]);
-            ldv(u + p - L.sy, ym);
-            ldv(u + p + L.sy, yp);
-            if (three) {
-                ldv(u + p - L.sz, zm);
-                ldv(u + p + L.sz, zp);
+            float x[V] = {}, ym[V] = {}, yp[V] = {}, zm[V] = {}, zp[V] = {}, qv[V], out[V];
+            float xl = 0.f, xr = 0.f;
+            if (!zs) {
+                ldv(u + p, x);
+                xl = Num<T>::ld(u[p - 1]);
+                xr = Num<T>::ld(u[p + V]);
+                ldv(u + p - L.sy, ym);
+                ldv(u + p + L.sy, yp);
+                if (three) {
+                    ldv(u + p - L.sz, zm);
+                    ldv(u + p + L.sz, zp);
+                }
             }
             ldv(q + p, qv);
 #pragma unroll
@@ -197,91 +205,585 @@ __global__ void __launch_bounds__(256) k_smooth(const Item* __restrict__ items, 
     }
 }
 
-// r = sigma over the items' groups (0 outside the interior); pool_in /
-// pool_out: the same pool, as in k_smooth (u and q are not written here)
+// ----------------------------------------------------------------- legs
+// One kernel takes a level down (last pre-smoothing sweep, residual, full
+// weighting) and one takes it up (prolongation, first post-smoothing sweep):
+// each reads u and q once and writes u once, 12.5 bytes per FP32 node and leg;
+// a kernel per operation moved 29 down and 20.5 up.  The 512-solve batch's step
+// g = 6 (50 solves of 129^3 among them) took 326 + 326 + 261 us down and 251 +
+// 326 us up that way and takes 271 and 206 us now, at the rate of a plain copy;
+// g = 9 (50 of 1025^2) 141 + 140 + 100 and 142 + 141 us, now 146 and 147; the
+// batch 121.1 -> 73.7 ms.
+//
+// A thread owns 4 nodes of x (one vector) and, in 3D, two rows of y, and
+// walks z (2D: y) with the planes it still needs in registers; x neighbours
+// come from the neighbour lanes by shuffles, y neighbours inside the pair of
+// rows from its own registers and across pairs from shared memory (5 vectors
+// per thread and plane, double buffered, so one barrier per plane).  A row of
+// up to 128 nodes is at most a warp wide; wider rows are cut into pieces of 30
+// groups with one halo group on each side.  In 3D the CTA is as wide as the
+// rows of a tile ask for; in 2D nothing is shared and every warp (n < 128:
+// part of a warp) walks alone.
+//
+// Per node and direction the neighbour sum runs ahead of the sweep: P(s) =
+// ((x- + x+) + y- + y+) + z- of plane s is formed when plane s arrives, z+ is
+// added when the next one does, so that a plane is kept as P and its centre
+// values only.  The order of the additions is that of k_smooth, and r and the
+// prolonged u are rounded to the storage type, so each result has the bits the
+// separate kernels gave.
+
+constexpr int kHaloLanes = 30;  // groups a warp keeps of a row wider than 32 groups
+
+struct Tile {
+    int solve, level;
+    int g0;      // first lane's group (-1 mod 30 for rows wider than a warp)
+    int y0;      // 3D: first row of the tile; even
+    int ja, jb;  // down: coarse rows; up: fine rows [ja, jb) written
+    int ka, kb;  // 3D: the same in z (2D: unused)
+};
+
 template <typename T>
-__global__ void __launch_bounds__(256) k_residual(const Item* __restrict__ items, int nitems,
-                                                  const BSolve* __restrict__ sv,
-                                                  const BLevel* __restrict__ lv,
-                                                  const T* __restrict__ pool_in,
-                                                  T* __restrict__ pool_out,
-                                                  const int* __restrict__ active, int src) {
-    constexpr int V = 16 / (int)sizeof(T);
-    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-        const Item w = items[it];
-        if (!active[w.solve]) continue;
-        const BLevel L = lv[sv[w.solve].lev0 + w.level];
-        const bool three = L.d == 3;
-        const float c = three ? 1.f / 6.f : 0.25f;
-        const T* u = pool_in + off_u(L, src);
-        const T* q = pool_in + L.q;
-        T* r = pool_out + L.r;
-        for (int t = threadIdx.x; t < w.count; t += blockDim.x) {
-            int x0, j, k;
-            const int64_t p = group_of<V>(L, (uint32_t)(w.start + t), x0, j, k);
-            float x[V], ym[V], yp[V], zm[V], zp[V], qv[V], out[V];
-            ldv(u + p, x);
-            const float xl = Num<T>::ld(u[p - 1]), xr = Num<T>::ld(u[p + V]);
-            ldv(u + p - L.sy, ym);
-            ldv(u + p + L.sy, yp);
-            if (three) {
-                ldv(u + p - L.sz, zm);
-                ldv(u + p + L.sz, zp);
-            }
-            ldv(q + p, qv);
+__device__ inline void ld4(const T* p, bool ok, float* v);
+template <>
+__device__ inline void ld4<float>(const float* p, bool ok, float* v) {
+    const float4 a = ok ? __ldg(reinterpret_cast<const float4*>(p)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    v[0] = a.x;
+    v[1] = a.y;
+    v[2] = a.z;
+    v[3] = a.w;
+}
+template <>
+__device__ inline void ld4<__nv_bfloat16>(const __nv_bfloat16* p, bool ok, float* v) {
+    const uint2 a = ok ? __ldg(reinterpret_cast<const uint2*>(p)) : make_uint2(0u, 0u);
+    v[0] = __uint_as_float(a.x << 16);
+    v[1] = __uint_as_float(a.x & 0xffff0000u);
+    v[2] = __uint_as_float(a.y << 16);
+    v[3] = __uint_as_float(a.y & 0xffff0000u);
+}
+__device__ inline void st4(float* p, const float* v) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ inline void st4(__nv_bfloat16* p, const float* v) {
+    __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
+    *reinterpret_cast<uint2*>(p) =
+        make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
+}
+__device__ inline void st2(float* p, float a, float b) {
+    *reinterpret_cast<float2*>(p) = make_float2(a, b);
+}
+__device__ inline void st2(__nv_bfloat16* p, float a, float b) {
+    *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(a, b);
+}
+__device__ inline float2 ld2(const float* p, bool ok) {
+    return ok ? __ldg(reinterpret_cast<const float2*>(p)) : make_float2(0.f, 0.f);
+}
+__device__ inline float2 ld2(const __nv_bfloat16* p, bool ok) {
+    const uint32_t a = ok ? __ldg(reinterpret_cast<const uint32_t*>(p)) : 0u;
+    return make_float2(__uint_as_float(a << 16), __uint_as_float(a & 0xffff0000u));
+}
+template <typename T>
+__device__ inline float rnd(float v) {
+    return Num<T>::ld(Num<T>::st(v));
+}
+
+// x- + x+ of the lane's 4 nodes (lanes: the width of a row in the warp); past
+// the last lane lies the boundary, or a value no kept node uses
+__device__ inline void xsum(const float* x, int lanes, bool last, float* s) {
+    const float l = __shfl_up_sync(0xffffffffu, x[3], 1, lanes);
+    float r = __shfl_down_sync(0xffffffffu, x[0], 1, lanes);
+    if (last) r = 0.f;
+    s[0] = l + x[1];
+    s[1] = x[0] + x[2];
+    s[2] = x[1] + x[3];
+    s[3] = x[2] + r;
+}
+
+__device__ inline void get4(const float4* p, bool ok, float* v) {
+    const float4 a = ok ? *p : make_float4(0.f, 0.f, 0.f, 0.f);
+    v[0] = a.x;
+    v[1] = a.y;
+    v[2] = a.z;
+    v[3] = a.w;
+}
+__device__ inline void put4(float4* p, const float* v) { *p = make_float4(v[0], v[1], v[2], v[3]); }
+
+// the coarse nodes 2g and 2g + 1 take row values r (l = the value left of the
+// lane's first) with weight w at dx = 0
+__device__ inline void fw_row(float* acc, float l, const float* r, float w) {
+    const float h = 0.5f * w;
+    acc[0] = fmaf(h, l, acc[0]);
+    acc[0] = fmaf(w, r[0], acc[0]);
+    acc[0] = fmaf(h, r[1], acc[0]);
+    acc[1] = fmaf(h, r[1], acc[1]);
+    acc[1] = fmaf(w, r[2], acc[1]);
+    acc[1] = fmaf(h, r[3], acc[1]);
+}
+
+// SWEEP: u1 = weighted-Jacobi step of u0 (buffer src), written to buffer dst,
+// then the residual of u1 and its restriction; otherwise the residual and
+// restriction of u0 alone.  zero: bit 0 / 1: u0 is zero on the solve's finest
+// level / on its coarser levels and is not read.  clear: write u_c = 0 (the
+// coarse level reads it); the one unknown of an n = 2 grid gets u_c = q_c.
+template <typename T, bool SWEEP>
+__global__ void __launch_bounds__(640, 1)
+    k_down3(const Tile* __restrict__ tiles, int ntiles, const BSolve* __restrict__ sv,
+            const BLevel* __restrict__ lv, const T* __restrict__ pool_in, T* __restrict__ pool_out,
+            const int* __restrict__ active, int src, int dst, int zero, int clear, float omega) {
+    extern __shared__ float4 edge[];  // [2][u0 row 0, u0 row 1, u1 row 0, u1 row 1, r row 1][thread]
+    const int nt = blockDim.x, tid = threadIdx.x;
+    const float c = 1.f / 6.f;
+    int buf = 0;
+    for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
+        const Tile t = tiles[it];
+        if (!active[t.solve]) continue;
+        const BLevel F = lv[sv[t.solve].lev0 + t.level];
+        const BLevel C = lv[sv[t.solve].lev0 + t.level + 1];
+        const int n = F.n, G = n >> 2, lanes = min(G, 32), lg = __ffs(lanes) - 1;
+        const int gx = tid & (lanes - 1), pair = tid >> lg, pairs = nt >> lg;
+        const int g = t.g0 + gx, y = t.y0 + 2 * pair;
+        const bool gok = g >= 0 && g < G, last = gx == lanes - 1;
+        const bool core = gok && (G <= 32 || (gx >= 1 && gx <= kHaloLanes));
+        const bool in0 = gok && y >= 1 && y < n, in1 = gok && y + 1 >= 1 && y + 1 < n;
+        const bool zs = SWEEP && ((zero >> (t.level > 0)) & 1);
+        const int jl = 2 * t.jb - 2 + (t.jb == n / 2);  // last fine row the tile writes
+        const int kl = 2 * t.kb - 2 + (t.kb == n / 2);
+        const bool w0 = core && in0 && y >= 2 * t.ja - 1 && y <= jl;
+        const bool w1 = core && in1 && y + 1 >= 2 * t.ja - 1 && y + 1 <= jl;
+        const bool wc = core && y >= 2 * t.ja && y < 2 * t.jb;
+        const int64_t o = (int64_t)y * F.sy + 4 * g;
+        const T* u = pool_in + off_u(F, src) + o;
+        const T* q = pool_in + F.q + o;
+        T* uo = pool_out + off_u(F, dst) + o;
+        const int64_t oc = (int64_t)(y >> 1) * C.sy + 2 * g;
+        float uc[2][4], un[2][4], vc[2][4] = {}, P0[2][4] = {}, P1[2][4] = {}, qo[2][4] = {},
+                                               qc[2][4] = {}, acc[2] = {};
+        auto load = [&](const T* a, int z, bool ok, float (*v)[4]) {
+            ok = ok && z >= 1 && z < n;
+            ld4(a + (int64_t)z * F.sz, ok && in0, v[0]);
+            ld4(a + (int64_t)z * F.sz + F.sy, ok && in1, v[1]);
+        };
+        const int s0 = 2 * t.ka - (SWEEP ? 3 : 2), s1 = 2 * t.kb;
+        load(u, s0, !zs, uc);
+        load(u, s0 + 1, !zs, un);
+        if (!SWEEP) load(q, s0, true, qc);
+        for (int s = s0; s <= s1; ++s) {
+            float u2[2][4], qn[2][4], v[2][4], r[2][4];
+            load(u, s + 2, !zs && s < s1, u2);
+            load(q, s + 1, s < s1, qn);
+            const bool zin = s >= 1 && s < n;
 #pragma unroll
-            for (int v = 0; v < V; ++v) {
-                float s = (v > 0 ? x[v - 1] : xl) + (v < V - 1 ? x[v + 1] : xr);
-                s += ym[v];
-                s += yp[v];
-                if (three) {
-                    s += zm[v];
-                    s += zp[v];
+            for (int h = 0; h < 2; ++h) {
+                const bool in = zin && (h ? in1 : in0);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if (SWEEP) {
+                        const float gs = fmaf(c, P0[h][e] + un[h][e], qc[h][e]);
+                        const float w = rnd<T>(fmaf(omega, gs - uc[h][e], uc[h][e]));
+                        v[h][e] = in && !(e == 0 && g == 0) ? w : 0.f;
+                    } else {
+                        v[h][e] = uc[h][e];
+                    }
                 }
-                const int xi = x0 + v;
-                out[v] = xi >= 1 && xi <= L.n - 1 ? fmaf(c, s, qv[v]) - x[v] : 0.f;
             }
-            stv(r + p, out);
+            if (SWEEP && s >= 2 * t.ka - 1 && s <= kl) {
+                if (w0) st4(uo + (int64_t)s * F.sz, v[0]);
+                if (w1) st4(uo + (int64_t)s * F.sz + F.sy, v[1]);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    r[h][e] = rnd<T>(fmaf(c, P1[h][e] + v[h][e], qo[h][e]) - vc[h][e]);
+            float4* E = edge + buf * 5 * nt + tid;
+            if (SWEEP && !zs) {
+                put4(E, un[0]);
+                put4(E + nt, un[1]);
+            }
+            put4(E + 2 * nt, v[0]);
+            put4(E + 3 * nt, v[1]);
+            put4(E + 4 * nt, r[1]);
+            __syncthreads();
+            const bool up = pair > 0, dn = pair + 1 < pairs;
+            float a[4], b[4], x[4];
+            if (SWEEP && !zs) {
+                get4(E + nt - lanes, up, a);
+                get4(E + lanes, dn, b);
+                xsum(un[0], lanes, last, x);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) P0[0][e] = ((x[e] + a[e]) + un[1][e]) + uc[0][e];
+                xsum(un[1], lanes, last, x);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) P0[1][e] = ((x[e] + un[0][e]) + b[e]) + uc[1][e];
+            }
+            get4(E + 3 * nt - lanes, up, a);
+            get4(E + 2 * nt + lanes, dn, b);
+            xsum(v[0], lanes, last, x);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) P1[0][e] = ((x[e] + a[e]) + v[1][e]) + vc[0][e];
+            xsum(v[1], lanes, last, x);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) P1[1][e] = ((x[e] + v[0][e]) + b[e]) + vc[1][e];
+            // plane s - 1 of r: dz = 0 of a coarse plane, or dz = +1 of one and -1 of the next
+            get4(E + 4 * nt - lanes, up, a);
+            const float la = __shfl_up_sync(0xffffffffu, a[3], 1, lanes),
+                        l0 = __shfl_up_sync(0xffffffffu, r[0][3], 1, lanes),
+                        l1 = __shfl_up_sync(0xffffffffu, r[1][3], 1, lanes);
+            if (s & 1) {
+                fw_row(acc, la, a, 0.25f);
+                fw_row(acc, l0, r[0], 0.5f);
+                fw_row(acc, l1, r[1], 0.25f);
+            } else {
+                fw_row(acc, la, a, 0.125f);
+                fw_row(acc, l0, r[0], 0.25f);
+                fw_row(acc, l1, r[1], 0.125f);
+                const int K = (s >> 1) - 1;
+                if (wc && K >= t.ka) {
+                    const int64_t P = (int64_t)K * C.sz + oc;
+                    if (g == 0) acc[0] = 0.f;
+                    st2(pool_out + C.q + P, acc[0], acc[1]);
+                    if (C.n == 2)
+                        st2(pool_out + C.u0 + P, acc[0], acc[1]);
+                    else if (clear)
+                        st2(pool_out + C.u0 + P, 0.f, 0.f);
+                }
+                acc[0] = acc[1] = 0.f;
+                fw_row(acc, la, a, 0.125f);
+                fw_row(acc, l0, r[0], 0.25f);
+                fw_row(acc, l1, r[1], 0.125f);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    uc[h][e] = un[h][e];
+                    un[h][e] = u2[h][e];
+                    vc[h][e] = v[h][e];
+                    qo[h][e] = qc[h][e];
+                    qc[h][e] = qn[h][e];
+                }
+            buf ^= 1;
+        }
+    }
+}
+// the same in 2D: a warp (or part of one) walks y by itself
+template <typename T, bool SWEEP>
+__global__ void __launch_bounds__(128)
+    k_down2(const Tile* __restrict__ tiles, int ntiles, const BSolve* __restrict__ sv,
+            const BLevel* __restrict__ lv, const T* __restrict__ pool_in, T* __restrict__ pool_out,
+            const int* __restrict__ active, int src, int dst, int zero, int clear, float omega,
+            int lanes) {
+    const int lane = threadIdx.x & 31, gx = lane & (lanes - 1), per = 32 / lanes;
+    const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+              nw = (gridDim.x * blockDim.x) >> 5;
+    const float c = 0.25f;
+    const bool last = gx == lanes - 1;
+    for (int first = wid * per; first < ntiles; first += nw * per) {
+        const int it = first + lane / lanes;
+        const Tile t = tiles[min(it, ntiles - 1)];
+        const bool on = it < ntiles && active[t.solve] != 0;
+        const BLevel F = lv[sv[t.solve].lev0 + t.level];
+        const BLevel C = lv[sv[t.solve].lev0 + t.level + 1];
+        const int n = F.n, G = n >> 2, g = t.g0 + gx;
+        const bool gok = on && g >= 0 && g < G;
+        const bool core = gok && (G <= 32 || (gx >= 1 && gx <= kHaloLanes));
+        const bool uok = gok && !(SWEEP && ((zero >> (t.level > 0)) & 1));
+        const int s0 = 2 * t.ja - (SWEEP ? 3 : 2), s1 = 2 * t.jb;
+        const int jl = 2 * t.jb - 2 + (t.jb == n / 2);
+        const int steps = __reduce_max_sync(0xffffffffu, on ? s1 - s0 + 1 : 0);
+        const T* u = pool_in + off_u(F, src) + 4 * g;
+        const T* q = pool_in + F.q + 4 * g;
+        T* uo = pool_out + off_u(F, dst) + 4 * g;
+        float uc[4], un[4], qc[4] = {}, qo[4] = {}, vc[4] = {}, P0[4] = {}, P1[4] = {}, acc[2] = {};
+        auto load = [&](const T* a, int y, bool ok, float* v) {
+            ld4(a + (int64_t)y * F.sy, ok && y >= 1 && y < n, v);
+        };
+        load(u, s0, uok, uc);
+        load(u, s0 + 1, uok, un);
+        if (!SWEEP) load(q, s0, gok, qc);
+        for (int i = 0; i < steps; ++i) {
+            const int s = s0 + i;
+            float u2[4], qn[4], v[4], r[4], x[4];
+            load(u, s + 2, uok && s < s1, u2);
+            load(q, s + 1, gok && s < s1, qn);
+            const bool in = gok && s >= 1 && s < n;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (SWEEP) {
+                    const float gs = fmaf(c, P0[e] + un[e], qc[e]);
+                    const float w = rnd<T>(fmaf(omega, gs - uc[e], uc[e]));
+                    v[e] = in && !(e == 0 && g == 0) ? w : 0.f;
+                } else {
+                    v[e] = uc[e];
+                }
+                r[e] = rnd<T>(fmaf(c, P1[e] + v[e], qo[e]) - vc[e]);
+            }
+            if (SWEEP && core && s >= 2 * t.ja - 1 && s <= jl) st4(uo + (int64_t)s * F.sy, v);
+            if (SWEEP) {
+                xsum(un, lanes, last, x);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) P0[e] = x[e] + uc[e];
+            }
+            xsum(v, lanes, last, x);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) P1[e] = x[e] + vc[e];
+            const float l = __shfl_up_sync(0xffffffffu, r[3], 1, lanes);
+            if (s & 1) {  // row s - 1 even: dy = 0
+                fw_row(acc, l, r, 1.f);
+            } else {
+                fw_row(acc, l, r, 0.5f);
+                const int J = (s >> 1) - 1;
+                if (core && J >= t.ja && J < t.jb) {
+                    const int64_t P = (int64_t)J * C.sy + 2 * g;
+                    if (g == 0) acc[0] = 0.f;
+                    st2(pool_out + C.q + P, acc[0], acc[1]);
+                    if (C.n == 2)
+                        st2(pool_out + C.u0 + P, acc[0], acc[1]);
+                    else if (clear)
+                        st2(pool_out + C.u0 + P, 0.f, 0.f);
+                }
+                acc[0] = acc[1] = 0.f;
+                fw_row(acc, l, r, 0.5f);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                uc[e] = un[e];
+                un[e] = u2[e];
+                vc[e] = v[e];
+                qo[e] = qc[e];
+                qc[e] = qn[e];
+            }
         }
     }
 }
 
-// q_c = 4 FW(r) on the items' coarse interior nodes (item level = fine
-// level); u_c = 0, or u_c = q_c on a one-unknown coarsest grid.  pool_in /
-// pool_out: the same pool, as in k_smooth (r is not written here).
+// the three coarse values of a row between which a lane's 4 fine nodes lie
+__device__ inline void widen3(float2 a, int lanes, bool last, float* c) {
+    c[0] = a.x;
+    c[1] = a.y;
+    c[2] = __shfl_down_sync(0xffffffffu, a.x, 1, lanes);
+    if (last) c[2] = 0.f;
+}
+
+// dst = weighted-Jacobi step of u + P u_c (u in buffer src, u_c in buffer
+// ccur).  The corners a fine node lies between are added in k_prolong's order
+// (x, then y, then z), so the plane above is added value by value.
 template <typename T>
-__global__ void __launch_bounds__(256) k_restrict(const Item* __restrict__ items, int nitems,
-                                                  const BSolve* __restrict__ sv,
-                                                  const BLevel* __restrict__ lv,
-                                                  const T* __restrict__ pool_in,
-                                                  T* __restrict__ pool_out,
-                                                  const int* __restrict__ active) {
-    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-        const Item w = items[it];
-        if (!active[w.solve]) continue;
-        const BLevel F = lv[sv[w.solve].lev0 + w.level];
-        const BLevel C = lv[sv[w.solve].lev0 + w.level + 1];
-        const bool three = F.d == 3;
-        const int64_t sy = F.sy, sz = three ? F.sz : 0;
-        const T* r = pool_in + F.r;
-        for (int t = threadIdx.x; t < w.count; t += blockDim.x) {
-            int I, J, K;
-            const int64_t P = node_of(C, (uint32_t)(w.start + t), I, J, K);
-            const int64_t p = (2 * K) * sz + (2 * J) * sy + 2 * I;
-            float v = 0.f;
-            for (int dz = three ? -1 : 0; dz <= (three ? 1 : 0); ++dz)
-                for (int dy = -1; dy <= 1; ++dy)
-                    for (int dx = -1; dx <= 1; ++dx) {
-                        // 4 x [1/4 1/2 1/4]^d: 2^(1 - zeros... ) as a power of two
-                        const int nz = (dx == 0) + (dy == 0) + (three ? (dz == 0) : 0);
-                        const int odd = (three ? 3 : 2) - nz;
-                        const float wgt = (three ? 0.5f : 1.f) * ldexpf(1.f, -odd);
-                        v = fmaf(wgt, Num<T>::ld(r[p + dz * sz + dy * sy + dx]), v);
+__global__ void __launch_bounds__(640, 1)
+    k_up3(const Tile* __restrict__ tiles, int ntiles, const BSolve* __restrict__ sv,
+          const BLevel* __restrict__ lv, const T* __restrict__ pool_in, T* __restrict__ pool_out,
+          const int* __restrict__ active, int src, int dst, int ccur, float omega) {
+    extern __shared__ float4 edge[];  // [2][row 0, row 1][thread]
+    const int nt = blockDim.x, tid = threadIdx.x;
+    const float c = 1.f / 6.f;
+    int buf = 0;
+    for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
+        const Tile t = tiles[it];
+        if (!active[t.solve]) continue;
+        const BLevel F = lv[sv[t.solve].lev0 + t.level];
+        const BLevel C = lv[sv[t.solve].lev0 + t.level + 1];
+        const int n = F.n, G = n >> 2, lanes = min(G, 32), lg = __ffs(lanes) - 1;
+        const int gx = tid & (lanes - 1), pair = tid >> lg, pairs = nt >> lg;
+        const int g = t.g0 + gx, y = t.y0 + 2 * pair;
+        const bool gok = g >= 0 && g < G, last = gx == lanes - 1;
+        const bool core = gok && (G <= 32 || (gx >= 1 && gx <= kHaloLanes));
+        const bool in0 = gok && y >= 1 && y < n, in1 = gok && y + 1 < n;
+        const bool w0 = core && in0 && y >= t.ja && y < t.jb;
+        const bool w1 = core && in1 && y + 1 >= t.ja && y + 1 < t.jb;
+        const int64_t o = (int64_t)y * F.sy + 4 * g;
+        const T* u = pool_in + off_u(F, src) + o;
+        const T* q = pool_in + F.q + o;
+        T* uo = pool_out + off_u(F, dst) + o;
+        const bool cok = gok && y < n;
+        const T* uk = pool_in + off_u(C, ccur) + (int64_t)(y >> 1) * C.sy + 2 * g;
+        auto load = [&](const T* a, int z, bool ok, float (*v)[4]) {
+            ok = ok && z >= 1 && z < n;
+            ld4(a + (int64_t)z * F.sz, ok && in0, v[0]);
+            ld4(a + (int64_t)z * F.sz + F.sy, ok && in1, v[1]);
+        };
+        float2 raw[2];
+        auto cload = [&](int K) {
+            const bool ok = cok && K < C.n;
+            raw[0] = ld2(uk + (int64_t)K * C.sz, ok);
+            raw[1] = ld2(uk + (int64_t)K * C.sz + C.sy, ok);
+        };
+        float ca[2][3] = {}, un[2][4], wc[2][4], P[2][4] = {}, qc[2][4] = {};
+        // w = u + P u_c on plane z (planes in order: ca = coarse plane z / 2)
+        auto correct = [&](int z, float (*v)[4]) {
+            float m[2][4];
+            m[0][0] = ca[0][0];
+            m[0][1] = ca[0][0] + ca[0][1];
+            m[0][2] = ca[0][1];
+            m[0][3] = ca[0][1] + ca[0][2];
+            m[1][0] = ca[0][0] + ca[1][0];
+            m[1][1] = (m[0][1] + ca[1][0]) + ca[1][1];
+            m[1][2] = ca[0][1] + ca[1][1];
+            m[1][3] = (m[0][3] + ca[1][1]) + ca[1][2];
+            float w = 1.f;
+            if (z & 1) {
+                float cb[2][3];
+                widen3(raw[0], lanes, last, cb[0]);
+                widen3(raw[1], lanes, last, cb[1]);
+                m[0][0] += cb[0][0];
+                m[0][1] = (m[0][1] + cb[0][0]) + cb[0][1];
+                m[0][2] += cb[0][1];
+                m[0][3] = (m[0][3] + cb[0][1]) + cb[0][2];
+                m[1][0] = (m[1][0] + cb[0][0]) + cb[1][0];
+                m[1][1] = (((m[1][1] + cb[0][0]) + cb[0][1]) + cb[1][0]) + cb[1][1];
+                m[1][2] = (m[1][2] + cb[0][1]) + cb[1][1];
+                m[1][3] = (((m[1][3] + cb[0][1]) + cb[0][2]) + cb[1][1]) + cb[1][2];
+                w = 0.5f;
+#pragma unroll
+                for (int e = 0; e < 3; ++e) {
+                    ca[0][e] = cb[0][e];
+                    ca[1][e] = cb[1][e];
+                }
+                cload((z >> 1) + 2);
+            }
+            const bool zin = z >= 1 && z < n;
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float f = w * (h ? 0.5f : 1.f) * (e & 1 ? 0.5f : 1.f);
+                    const bool in = zin && (h ? in1 : in0) && !(e == 0 && g == 0);
+                    v[h][e] = in ? rnd<T>(v[h][e] + f * m[h][e]) : 0.f;
+                }
+        };
+        const int s0 = t.ka - 1, s1 = t.kb - 1;
+        cload(s0 >> 1);
+        widen3(raw[0], lanes, last, ca[0]);
+        widen3(raw[1], lanes, last, ca[1]);
+        cload((s0 >> 1) + 1);
+        load(u, s0, true, wc);
+        load(u, s0 + 1, true, un);
+        correct(s0, wc);
+        for (int s = s0; s <= s1; ++s) {
+            float u2[2][4], qn[2][4], v[2][4], x[4], a[4], b[4];
+            load(u, s + 2, s < s1, u2);
+            load(q, s + 1, s < s1, qn);
+            correct(s + 1, un);
+            if (s >= t.ka) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float gs = fmaf(c, P[h][e] + un[h][e], qc[h][e]);
+                        v[h][e] = e == 0 && g == 0 ? 0.f : fmaf(omega, gs - wc[h][e], wc[h][e]);
                     }
-            T* qc = pool_out + C.q;
-            T* uc = pool_out + C.u0;
-            qc[P] = Num<T>::st(v);
-            uc[P] = C.n == 2 ? Num<T>::st(v) : Num<T>::st(0.f);
+                if (w0) st4(uo + (int64_t)s * F.sz, v[0]);
+                if (w1) st4(uo + (int64_t)s * F.sz + F.sy, v[1]);
+            }
+            float4* E = edge + buf * 2 * nt + tid;
+            put4(E, un[0]);
+            put4(E + nt, un[1]);
+            __syncthreads();
+            get4(E + nt - lanes, pair > 0, a);
+            get4(E + lanes, pair + 1 < pairs, b);
+            xsum(un[0], lanes, last, x);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) P[0][e] = ((x[e] + a[e]) + un[1][e]) + wc[0][e];
+            xsum(un[1], lanes, last, x);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) P[1][e] = ((x[e] + un[0][e]) + b[e]) + wc[1][e];
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    wc[h][e] = un[h][e];
+                    un[h][e] = u2[h][e];
+                    qc[h][e] = qn[h][e];
+                }
+            buf ^= 1;
+        }
+    }
+}
+
+// the same in 2D
+template <typename T>
+__global__ void __launch_bounds__(128)
+    k_up2(const Tile* __restrict__ tiles, int ntiles, const BSolve* __restrict__ sv,
+          const BLevel* __restrict__ lv, const T* __restrict__ pool_in, T* __restrict__ pool_out,
+          const int* __restrict__ active, int src, int dst, int ccur, float omega, int lanes) {
+    const int lane = threadIdx.x & 31, gx = lane & (lanes - 1), per = 32 / lanes;
+    const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+              nw = (gridDim.x * blockDim.x) >> 5;
+    const float c = 0.25f;
+    const bool last = gx == lanes - 1;
+    for (int first = wid * per; first < ntiles; first += nw * per) {
+        const int it = first + lane / lanes;
+        const Tile t = tiles[min(it, ntiles - 1)];
+        const bool on = it < ntiles && active[t.solve] != 0;
+        const BLevel F = lv[sv[t.solve].lev0 + t.level];
+        const BLevel C = lv[sv[t.solve].lev0 + t.level + 1];
+        const int n = F.n, G = n >> 2, g = t.g0 + gx;
+        const bool gok = on && g >= 0 && g < G;
+        const bool core = gok && (G <= 32 || (gx >= 1 && gx <= kHaloLanes));
+        const int s0 = t.ja - 1, s1 = t.jb - 1;
+        const int steps = __reduce_max_sync(0xffffffffu, on ? s1 - s0 + 1 : 0);
+        const T* u = pool_in + off_u(F, src) + 4 * g;
+        const T* q = pool_in + F.q + 4 * g;
+        T* uo = pool_out + off_u(F, dst) + 4 * g;
+        const T* uk = pool_in + off_u(C, ccur) + 2 * g;
+        auto load = [&](const T* a, int y, bool ok, float* v) {
+            ld4(a + (int64_t)y * F.sy, gok && ok && y >= 1 && y < n, v);
+        };
+        float2 raw;
+        auto cload = [&](int J) { raw = ld2(uk + (int64_t)J * C.sy, gok && J < C.n); };
+        float ca[3] = {}, un[4], wc[4], P[4] = {}, qc[4] = {};
+        // the lanes of a warp whose rows are of the other parity take the same
+        // shuffles: odd is the lane's own
+        auto correct = [&](int y, float* v) {
+            const bool odd = y & 1;
+            float cb[3], m[4];
+            widen3(raw, lanes, last, cb);
+            m[0] = ca[0];
+            m[1] = ca[0] + ca[1];
+            m[2] = ca[1];
+            m[3] = ca[1] + ca[2];
+            if (odd) {
+                m[0] += cb[0];
+                m[1] = (m[1] + cb[0]) + cb[1];
+                m[2] += cb[1];
+                m[3] = (m[3] + cb[1]) + cb[2];
+#pragma unroll
+                for (int e = 0; e < 3; ++e) ca[e] = cb[e];
+                cload((y >> 1) + 2);
+            }
+            const bool yin = gok && y >= 1 && y < n;
+            const float w = odd ? 0.5f : 1.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float f = e & 1 ? 0.5f * w : w;
+                v[e] = yin && !(e == 0 && g == 0) ? rnd<T>(v[e] + f * m[e]) : 0.f;
+            }
+        };
+        cload(s0 >> 1);
+        widen3(raw, lanes, last, ca);
+        cload((s0 >> 1) + 1);
+        load(u, s0, true, wc);
+        load(u, s0 + 1, true, un);
+        correct(s0, wc);
+        for (int i = 0; i < steps; ++i) {
+            const int s = s0 + i;
+            float u2[4], qn[4], v[4], x[4];
+            load(u, s + 2, s < s1, u2);
+            load(q, s + 1, s < s1, qn);
+            correct(s + 1, un);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float gs = fmaf(c, P[e] + un[e], qc[e]);
+                v[e] = e == 0 && g == 0 ? 0.f : fmaf(omega, gs - wc[e], wc[e]);
+            }
+            if (core && s >= t.ja && s < t.jb) st4(uo + (int64_t)s * F.sy, v);
+            xsum(un, lanes, last, x);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) P[e] = x[e] + wc[e];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                wc[e] = un[e];
+                un[e] = u2[e];
+                qc[e] = qn[e];
+            }
         }
     }
 }
@@ -519,10 +1021,15 @@ using namespace gmg::batch;
 
 namespace {
 
-enum Op { OP_FINE, OP_COARSE, OP_CELLS, OP_COUNT };
-
 struct Range {
     int off = 0, count = 0;
+    int64_t nodes = 0;  // the items' work
+};
+// a level step of the solves of one dimension: plain items (chunks) and legs'
+// tiles with their launch shapes
+struct Step {
+    Range fine, cells, down, up;
+    int down_threads = 0, up_threads = 0, lanes = 32;
 };
 
 }  // namespace
@@ -530,16 +1037,23 @@ struct Range {
 struct gmg_batch_s {
     gmg_config cfg{};
     int count = 0, chunk = 1024, ctas = 608, device = 0, G = 0, elem = 4;
-    cudaStream_t user_stream = nullptr, stream = nullptr;
-    cudaEvent_t ev = nullptr;
+    int sms = 152;
+    // stream2: the 2D solves' launches inside the captured step, which depend
+    // on none of the 3D solves'
+    cudaStream_t user_stream = nullptr, stream = nullptr, stream2 = nullptr;
+    cudaEvent_t ev = nullptr, fork = nullptr, join = nullptr;
     std::vector<BSolve> hs;
     std::vector<BLevel> hl;
     std::vector<Item> items;
-    std::vector<Range> fine, coarse, cells;  // per level step g
-    Range level0;                            // level-0 interior items (all solves)
+    std::vector<Tile> tiles;
+    std::vector<Step> steps[2];  // per level step g: 2D, 3D
+    int leg_warps[4] = {0, 0, 0, 0};
+    bool has_d[2] = {false, false};
+    Range level0;                // level-0 interior items (all solves)
     BSolve* ds = nullptr;
     BLevel* dl = nullptr;
     Item* di = nullptr;
+    Tile* dt = nullptr;
     void* pool = nullptr;
     double* pool64 = nullptr;
     double* partial = nullptr;
@@ -568,18 +1082,126 @@ struct PrecName<__nv_bfloat16> {
 };
 
 template <typename T, class F>
-void launch_op(gmg_batch b, const char* name, int g, const Range& r, double bytes_per_item_node,
-               double ops_per_node, int64_t nodes, F&& body) {
+void launch_op(gmg_batch b, cudaStream_t st, const char* name, int g, const Range& r,
+               double bytes_per_node, double ops_per_node, F&& body) {
     if (r.count == 0) return;
     const int grid = std::min(r.count, b->ctas);
-    b->timer.run(b->stream, std::string(name) + PrecName<T>::s, g, ops_per_node * nodes,
-                 bytes_per_item_node * nodes, 1, [&] { body(grid, b->di + r.off, r.count); });
+    b->timer.run(st, std::string(name) + PrecName<T>::s, g, ops_per_node * r.nodes,
+                 bytes_per_node * r.nodes, 1, [&] { body(grid, b->di + r.off, r.count); });
 }
 
-int64_t range_nodes(gmg_batch b, const Range& r) {
-    int64_t s = 0;
-    for (int i = r.off; i < r.off + r.count; ++i) s += b->items[i].count;
-    return s;
+// The inner cycles of the solves of dimension d on stream st.
+template <typename T>
+gmg_status enqueue_cycles(gmg_batch b, int d, cudaStream_t st) {
+    const gmg_config& c = b->cfg;
+    const std::vector<Step>& steps = b->steps[d - 2];
+    T* pool = static_cast<T*>(b->pool);
+    const double w = sizeof(T);
+    const bool rbgs = c.smoother == GMG_RBGS;
+    // weighted-Jacobi weight per dimension: the configured one, or with
+    // omega = 0 the defaults 4/5 (2D) and 6/7 (3D)
+    const float omega2 = c.omega > 0.0 ? (float)c.omega : 0.8f;
+    const float omega3 = c.omega > 0.0 ? (float)c.omega : (float)(6.0 / 7.0);
+    const float omega = d == 3 ? omega3 : omega2;
+    // a weighted-Jacobi sweep next to the transfer goes into the leg; the first
+    // one from zero does not read u, so that u_c = 0 need not be written
+    const bool sweep_down = !rbgs && c.nu1 >= 1, sweep_up = !rbgs && c.nu2 >= 1;
+    int G = 0;
+    for (int g = 1; g <= b->G; ++g)
+        if (steps[g].fine.count) G = g;
+    std::vector<int> cur(G + 1, 0);  // which u buffer holds each level step's iterate
+    auto relax = [&](int g, int sweeps, int zero) {
+        const Range& r = steps[g].fine;
+        for (int s = 0; s < sweeps; ++s) {
+            if (rbgs) {
+                for (int color = 0; color < 2; ++color)
+                    launch_op<T>(b, st, "b_rb_half", g, r, 1.5 * w, 3.0,
+                                 [&](int grid, const Item* it, int ni) {
+                                     k_smooth<T><<<grid, 256, 0, st>>>(
+                                         it, ni, b->ds, b->dl, pool, pool, b->active, cur[g],
+                                         cur[g], color, 0, omega2, omega3);
+                                 });
+            } else {
+                launch_op<T>(b, st, "b_wj_sweep", g, r, 3 * w, 8.0,
+                             [&](int grid, const Item* it, int ni) {
+                                 k_smooth<T><<<grid, 256, 0, st>>>(
+                                     it, ni, b->ds, b->dl, pool, pool, b->active, cur[g],
+                                     cur[g] ^ 1, -1, s == 0 ? zero : 0, omega2, omega3);
+                             });
+                cur[g] ^= 1;
+            }
+        }
+    };
+    auto down = [&](int g, int zero) {
+        const Step& S = steps[g];
+        const Tile* t = b->dt + S.down.off;
+        const int nt = S.down.count, clear = !sweep_down, th = S.down_threads;
+        const int src = cur[g], dst = sweep_down ? cur[g] ^ 1 : cur[g];
+        b->timer.run(st, std::string(sweep_down ? "b_down_leg" : "b_res_restrict") + PrecName<T>::s,
+                     g, (sweep_down ? 18.0 : 10.0) * S.down.nodes,
+                     (sweep_down ? 3.125 : 2.125) * w * S.down.nodes, 1, [&] {
+                         if (d == 3) {
+                             auto k = sweep_down ? k_down3<T, true> : k_down3<T, false>;
+                             k<<<std::min(nt, b->ctas), th, 160 * th, st>>>(
+                                 t, nt, b->ds, b->dl, pool, pool, b->active, src, dst, zero, clear,
+                                 omega);
+                         } else {
+                             const int ctas = (nt * S.lanes + 127) / 128;
+                             auto k = sweep_down ? k_down2<T, true> : k_down2<T, false>;
+                             k<<<std::min(ctas, b->ctas), 128, 0, st>>>(
+                                 t, nt, b->ds, b->dl, pool, pool, b->active, src, dst, zero, clear,
+                                 omega, S.lanes);
+                         }
+                     });
+        cur[g] = dst;
+    };
+    auto up = [&](int g) {
+        const Step& S = steps[g];
+        const Tile* t = b->dt + S.up.off;
+        const int nt = S.up.count, th = S.up_threads, src = cur[g], cc = cur[g - 1];
+        b->timer.run(st, std::string("b_up_leg") + PrecName<T>::s, g, 12.0 * S.up.nodes,
+                     3.125 * w * S.up.nodes, 1, [&] {
+                         if (d == 3)
+                             k_up3<T><<<std::min(nt, b->ctas), th, 64 * th, st>>>(
+                                 t, nt, b->ds, b->dl, pool, pool, b->active, src, src ^ 1, cc,
+                                 omega);
+                         else
+                             k_up2<T><<<std::min((nt * S.lanes + 127) / 128, b->ctas), 128, 0, st>>>(
+                                 t, nt, b->ds, b->dl, pool, pool, b->active, src, src ^ 1, cc,
+                                 omega, S.lanes);
+                     });
+        cur[g] ^= 1;
+    };
+    for (int k = 0; k < c.inner_cycles; ++k) {
+        std::fill(cur.begin(), cur.end(), 0);
+        // which levels start from zero: the coarse ones, in the first cycle all
+        const int zero = 2 | (k == 0 ? 1 : 0);
+        // down: level steps g = G..1 (fine levels of the deepest solves first)
+        for (int g = G; g >= 1; --g) {
+            relax(g, sweep_down ? c.nu1 - 1 : c.nu1, zero);
+            down(g, sweep_down && c.nu1 == 1 ? zero : 0);
+            cur[g - 1] = 0;
+        }
+        // up: g = 1..G
+        for (int g = 1; g <= G; ++g) {
+            if (sweep_up) {
+                up(g);
+            } else {
+                const int fc = cur[g], cc = cur[g - 1];
+                launch_op<T>(b, st, "b_prolong_add", g, steps[g].cells, 17 * w, 20.0,
+                             [&](int grid, const Item* it, int ni) {
+                                 k_prolong<T><<<grid, 256, 0, st>>>(it, ni, b->ds, b->dl, pool,
+                                                                    b->active, fc, cc);
+                             });
+            }
+            relax(g, sweep_up ? c.nu2 - 1 : c.nu2, 0);
+        }
+        if (cur[G] != 0) {
+            set_error("batched weighted Jacobi needs an even nu1 + nu2 on the finest levels");
+            return GMG_ERR_UNSUPPORTED;
+        }
+    }
+    return GMG_OK;
 }
 
 // One refinement step of the whole batch (captured): e = 0, k inner
@@ -589,81 +1211,36 @@ gmg_status enqueue_step(gmg_batch b, double rtol2) {
     const gmg_config& c = b->cfg;
     T* pool = static_cast<T*>(b->pool);
     const double w = sizeof(T);
-    const bool rbgs = c.smoother == GMG_RBGS;
-    // weighted-Jacobi weight per dimension: the configured one, or with
-    // omega = 0 the defaults 4/5 (2D) and 6/7 (3D)
-    const float omega2 = c.omega > 0.0 ? (float)c.omega : 0.8f;
-    const float omega3 = c.omega > 0.0 ? (float)c.omega : (float)(6.0 / 7.0);
     b->timer.begin_capture();
-    const int64_t n0 = range_nodes(b, b->level0);
-    launch_op<T>(b, "b_zero", 0, b->level0, w, 0, n0, [&](int grid, const Item* it, int ni) {
-        k_zero<T><<<grid, 256, 0, b->stream>>>(it, ni, b->ds, b->dl, pool, b->active);
-    });
-    std::vector<int> cur(b->G + 1, 0);  // which u buffer holds each level step's iterate
-    auto relax = [&](int g, int sweeps) {
-        const Range& r = b->fine[g];
-        const int64_t nn = range_nodes(b, r) * (16 / b->elem);  // groups x V nodes
-        for (int s = 0; s < sweeps; ++s) {
-            if (rbgs) {
-                for (int color = 0; color < 2; ++color)
-                    launch_op<T>(b, "b_rb_half", g, r, 1.5 * w, 3.0, nn,
-                                 [&](int grid, const Item* it, int ni) {
-                                     k_smooth<T><<<grid, 256, 0, b->stream>>>(
-                                         it, ni, b->ds, b->dl, pool, pool, b->active, cur[g],
-                                         cur[g], color, omega2, omega3);
-                                 });
-            } else {
-                launch_op<T>(b, "b_wj_sweep", g, r, 3 * w, 8.0, nn,
-                             [&](int grid, const Item* it, int ni) {
-                                 k_smooth<T><<<grid, 256, 0, b->stream>>>(
-                                     it, ni, b->ds, b->dl, pool, pool, b->active, cur[g],
-                                     cur[g] ^ 1, -1, omega2, omega3);
-                             });
-                cur[g] ^= 1;
-            }
-        }
-    };
-    for (int k = 0; k < c.inner_cycles; ++k) {
-        std::fill(cur.begin(), cur.end(), 0);
-        // down: level steps g = G..1 (fine levels of the deepest solves first)
-        for (int g = b->G; g >= 1; --g) {
-            relax(g, c.nu1);
-            const int64_t nn = range_nodes(b, b->fine[g]) * (16 / b->elem);
-            launch_op<T>(b, "b_residual", g, b->fine[g], 3 * w, 7.0, nn,
-                         [&](int grid, const Item* it, int ni) {
-                             k_residual<T><<<grid, 256, 0, b->stream>>>(
-                                 it, ni, b->ds, b->dl, pool, pool, b->active, cur[g]);
-                         });
-            const int64_t nc = range_nodes(b, b->coarse[g]);
-            launch_op<T>(b, "b_restrict", g, b->coarse[g], 10 * w, 27.0, nc,
-                         [&](int grid, const Item* it, int ni) {
-                             k_restrict<T><<<grid, 256, 0, b->stream>>>(it, ni, b->ds, b->dl,
-                                                                        pool, pool, b->active);
-                         });
-            cur[g - 1] = 0;
-        }
-        // up: g = 1..G
-        for (int g = 1; g <= b->G; ++g) {
-            const int64_t ncell = range_nodes(b, b->cells[g]);
-            const int fc = cur[g], cc = cur[g - 1];
-            launch_op<T>(b, "b_prolong_add", g, b->cells[g], 17 * w, 20.0, ncell,
-                         [&](int grid, const Item* it, int ni) {
-                             k_prolong<T><<<grid, 256, 0, b->stream>>>(it, ni, b->ds, b->dl, pool,
-                                                                       b->active, fc, cc);
-                         });
-            relax(g, c.nu2);
-        }
-        if (cur[b->G] != 0) {
-            set_error("batched weighted Jacobi needs an even nu1 + nu2 on the finest levels");
-            return GMG_ERR_UNSUPPORTED;
-        }
+    if (c.smoother == GMG_RBGS || c.nu1 == 0)
+        launch_op<T>(b, b->stream, "b_zero", 0, b->level0, w, 0,
+                     [&](int grid, const Item* it, int ni) {
+                         k_zero<T><<<grid, 256, 0, b->stream>>>(it, ni, b->ds, b->dl, pool,
+                                                                b->active);
+                     });
+    // The 2D and the 3D solves' launches are two branches of the graph: the
+    // small levels of one fill the chip beside the other's.  While kernels are
+    // timed they run one after the other.
+    const bool both = b->has_d[0] && b->has_d[1] && !b->timer.enabled;
+    cudaStream_t st2 = both ? b->stream2 : b->stream;
+    gmg_status rc = GMG_OK;
+    if (both) {
+        GMG_CUDA_TRY(cudaEventRecord(b->fork, b->stream));
+        GMG_CUDA_TRY(cudaStreamWaitEvent(st2, b->fork, 0));
     }
-    launch_op<T>(b, "b_update", 0, b->level0, 16 + w, 1.0, n0,
+    if (b->has_d[1]) rc = enqueue_cycles<T>(b, 3, b->stream);
+    if (rc == GMG_OK && b->has_d[0]) rc = enqueue_cycles<T>(b, 2, st2);
+    if (both) {
+        GMG_CUDA_TRY(cudaEventRecord(b->join, st2));
+        GMG_CUDA_TRY(cudaStreamWaitEvent(b->stream, b->join, 0));
+    }
+    if (rc != GMG_OK) return rc;
+    launch_op<T>(b, b->stream, "b_update", 0, b->level0, 16 + w, 1.0,
                  [&](int grid, const Item* it, int ni) {
                      k_update<T><<<grid, 256, 0, b->stream>>>(it, ni, b->ds, b->dl, pool,
                                                               b->active);
                  });
-    launch_op<T>(b, "b_outer_residual", 0, b->level0, 16 + w, 8.0, n0,
+    launch_op<T>(b, b->stream, "b_outer_residual", 0, b->level0, 16 + w, 8.0,
                  [&](int grid, const Item* it, int ni) {
                      k_outer<T><<<grid, 256, 0, b->stream>>>(it, ni, b->ds, b->dl, pool,
                                                              b->pool64, b->active, b->partial);
@@ -708,6 +1285,31 @@ bool dev_ptr_ok(const void* p) {
 
 }  // namespace
 
+namespace {
+
+// warps of each leg kernel that fit on an SM: leg_warps[2D up, 2D down, 3D up,
+// 3D down]; the 3D kernels' shared memory is opted into here
+template <typename T>
+cudaError_t leg_occupancy(gmg_batch b) {
+    const bool rbgs = b->cfg.smoother == GMG_RBGS;
+    const bool sweep = !rbgs && b->cfg.nu1 >= 1;
+    auto d3 = sweep ? k_down3<T, true> : k_down3<T, false>;
+    auto d2 = sweep ? k_down2<T, true> : k_down2<T, false>;
+    cudaError_t e = cudaFuncSetAttribute(d3, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 640);
+    auto occ = [&](auto k, int threads, int smem, int& warps) {
+        int n = 0;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem);
+        warps = std::max(1, n) * threads / 32;
+    };
+    occ(k_up2<T>, 128, 0, b->leg_warps[0]);
+    occ(d2, 128, 0, b->leg_warps[1]);
+    occ(k_up3<T>, 128, 64 * 128, b->leg_warps[2]);
+    occ(d3, 128, 160 * 128, b->leg_warps[3]);
+    return e;
+}
+
+}  // namespace
+
 extern "C" {
 
 gmg_status gmg_batch_destroy(gmg_batch b) {
@@ -718,13 +1320,15 @@ gmg_status gmg_batch_destroy(gmg_batch b) {
     if (b->stream) cudaStreamSynchronize(b->stream);
     if (b->graph) cudaGraphExecDestroy(b->graph);
     b->timer.destroy();
-    for (void* p : {(void*)b->ds, (void*)b->dl, (void*)b->di, b->pool, (void*)b->pool64,
+    for (void* p : {(void*)b->ds, (void*)b->dl, (void*)b->di, (void*)b->dt, b->pool, (void*)b->pool64,
                     (void*)b->partial, (void*)b->res0_2, (void*)b->relres, (void*)b->active,
                     (void*)b->iters, (void*)b->num_active})
         if (p) cudaFree(p);
     if (b->h_active) cudaFreeHost(b->h_active);
-    if (b->ev) cudaEventDestroy(b->ev);
-    if (b->stream) cudaStreamDestroy(b->stream);
+    for (cudaEvent_t ev : {b->ev, b->fork, b->join})
+        if (ev) cudaEventDestroy(ev);
+    for (cudaStream_t st : {b->stream, b->stream2})
+        if (st) cudaStreamDestroy(st);
     delete b;
     if (prev >= 0) cudaSetDevice(prev);
     return GMG_OK;
@@ -783,11 +1387,13 @@ gmg_status gmg_batch_create(int count, const int* d, const int* n, const gmg_con
         return st;
     };
     if (cudaGetDevice(&b->device) != cudaSuccess) return fail(GMG_ERR_CUDA, "no device");
-    int sms = 152;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
-    b->ctas = ctas > 0 ? ctas : 4 * sms;
+    cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device);
+    b->ctas = ctas > 0 ? ctas : 4 * b->sms;
     if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess)
+        cudaStreamCreateWithFlags(&b->stream2, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming) != cudaSuccess)
         return fail(GMG_ERR_CUDA, "stream/event creation failed");
     // layout: per solve, per level: u0 [u1] q [r] in the inner pool (256-byte
     // aligned regions); FP64 q64 per solve
@@ -844,10 +1450,6 @@ gmg_status gmg_batch_create(int count, const int* d, const int* n, const gmg_con
             dst.push_back({s, level, st, (int)std::min<int64_t>(b->chunk, total - st)});
     };
     auto pw = [](int64_t v, int d_) { return d_ == 3 ? v * v * v : v * v; };
-    b->fine.resize(b->G + 1);
-    b->coarse.resize(b->G + 1);
-    b->cells.resize(b->G + 1);
-    std::vector<Item> tmp;
     {  // level 0 interior items, grouped by solve (the finalize sums them in order)
         b->level0.off = (int)b->items.size();
         for (int s = 0; s < count; ++s) {
@@ -856,32 +1458,81 @@ gmg_status gmg_batch_create(int count, const int* d, const int* n, const gmg_con
             b->hs[s].item1 = (int)b->items.size() - b->level0.off;
         }
         b->level0.count = (int)b->items.size() - b->level0.off;
+        for (int i = 0; i < b->level0.count; ++i)
+            b->level0.nodes += b->items[b->level0.off + i].count;
     }
-    for (int g = 1; g <= b->G; ++g) {
-        for (int kind = 0; kind < OP_COUNT; ++kind) {
-            Range r;
-            r.off = (int)b->items.size();
-            for (int s = 0; s < count; ++s) {
-                const BSolve& S = b->hs[s];
-                const int l = S.levels - 1 - g;
-                if (l < 0) continue;
-                const int nl = S.n >> l, nc = nl / 2;
-                if (kind == OP_FINE) {
-                    // the vector kernels' items: (interior row, 16-byte group)
-                    // pairs, chunk / V groups per item
-                    const int V = 16 / b->elem;
-                    const int64_t groups = (int64_t)(S.d == 3 ? (nl - 1) * (nl - 1) : nl - 1)
-                                           << b->hl[S.lev0 + l].lgG;
-                    const int64_t gchunk = std::max<int64_t>(1, b->chunk / V);
-                    for (int64_t st = 0; st < groups; st += gchunk)
-                        b->items.push_back({s, l, st, (int)std::min<int64_t>(gchunk, groups - st)});
-                    continue;
-                }
-                const int64_t total = kind == OP_COARSE ? pw(nc - 1, S.d) : pw(nc, S.d);
-                add_items(s, l, total, b->items);
+    const bool rbgs = common->smoother == GMG_RBGS;
+    const cudaError_t oe = b->elem == 4 ? leg_occupancy<float>(b) : leg_occupancy<__nv_bfloat16>(b);
+    if (oe != cudaSuccess) return fail(GMG_ERR_CUDA, cudaGetErrorString(oe));
+    for (int dim = 2; dim <= 3; ++dim) {
+        b->steps[dim - 2].resize(b->G + 1);
+        for (int g = 1; g <= b->G; ++g) {
+            Step& S = b->steps[dim - 2][g];
+            const int n_g = 2 << g, nc = n_g / 2;  // the same size for every solve
+            std::vector<int> members;
+            for (int s = 0; s < count; ++s)
+                if (b->hs[s].d == dim && b->hs[s].levels - 1 >= g) members.push_back(s);
+            if (members.empty()) continue;
+            b->has_d[dim - 2] = true;
+            auto level_of = [&](int s) { return b->hs[s].levels - 1 - g; };
+            // plain sweeps: (interior row, 16-byte group) pairs, chunk / V groups per item
+            S.fine.off = (int)b->items.size();
+            const int V = 16 / b->elem;
+            for (int s : members) {
+                const int l = level_of(s);
+                const int64_t groups = (int64_t)(dim == 3 ? (n_g - 1) * (n_g - 1) : n_g - 1)
+                                       << b->hl[b->hs[s].lev0 + l].lgG;
+                const int64_t gchunk = std::max<int64_t>(1, b->chunk / V);
+                for (int64_t st = 0; st < groups; st += gchunk)
+                    b->items.push_back({s, l, st, (int)std::min<int64_t>(gchunk, groups - st)});
+                S.fine.nodes += groups * V;
             }
-            r.count = (int)b->items.size() - r.off;
-            (kind == OP_FINE ? b->fine : kind == OP_COARSE ? b->coarse : b->cells)[g] = r;
+            S.fine.count = (int)b->items.size() - S.fine.off;
+            if (rbgs || common->nu2 == 0) {
+                S.cells.off = (int)b->items.size();
+                for (int s : members) {
+                    add_items(s, level_of(s), pw(nc, dim), b->items);
+                    S.cells.nodes += pw(nc, dim);
+                }
+                S.cells.count = (int)b->items.size() - S.cells.off;
+            }
+            // legs' tiles, a solve's side by side
+            S.lanes = std::min(n_g / 4, 32);
+            const std::vector<int> cols = leg_columns(n_g / 4, kHaloLanes);
+            const int64_t nm = (int64_t)members.size();
+            for (int down = 0; down < 2; ++down) {
+                if (!down && (rbgs || common->nu2 == 0)) continue;
+                Range& r = down ? S.down : S.up;
+                r.off = (int)b->tiles.size();
+                // walk: coarse planes 1..nc-1 down (2 fine planes each), fine planes 1..n-1 up
+                const int len = down ? nc - 1 : n_g - 1, unit = down ? 2 : 1, extra = down ? 4 : 2;
+                int& th = down ? S.down_threads : S.up_threads;
+                std::vector<Rows> rows(1, Rows{0, 0, 0});
+                int64_t slots;
+                if (dim == 3) {
+                    th = leg_threads(n_g, down);
+                    const int R = leg_rows(n_g, th);
+                    rows = down ? rows_down(n_g, R) : rows_up(n_g, R);
+                    slots = (int64_t)b->sms * std::max(1, b->leg_warps[2 + down] / (th / 32));
+                } else {
+                    slots = (int64_t)b->sms * b->leg_warps[down] * (32 / S.lanes);
+                }
+                const int np = leg_pieces(nm * (int64_t)(rows.size() * cols.size()), slots, len,
+                                          unit, extra);
+                for (int s : members)
+                    for (int pc = 0; pc < np; ++pc) {
+                        const int a = 1 + (int)((int64_t)len * pc / np),
+                                  e = 1 + (int)((int64_t)len * (pc + 1) / np);
+                        for (const Rows& rw : rows)
+                            for (int g0 : cols)
+                                b->tiles.push_back(dim == 3 ? Tile{s, level_of(s), g0, rw.y0, rw.ja,
+                                                                   rw.jb, a, e}
+                                                            : Tile{s, level_of(s), g0, 0, a, e, 0,
+                                                                   0});
+                    }
+                r.count = (int)b->tiles.size() - r.off;
+                r.nodes = nm * pw(n_g - 1, dim);
+            }
         }
     }
     cudaError_t e = cudaSuccess;
@@ -892,6 +1543,7 @@ gmg_status gmg_batch_create(int count, const int* d, const int* n, const gmg_con
     al((void**)&b->ds, sizeof(BSolve) * count);
     al((void**)&b->dl, sizeof(BLevel) * b->hl.size());
     al((void**)&b->di, sizeof(Item) * b->items.size());
+    al((void**)&b->dt, sizeof(Tile) * b->tiles.size());
     al(&b->pool, (size_t)b->elem * poff);
     al((void**)&b->pool64, sizeof(double) * off64);
     al((void**)&b->partial, sizeof(double) * b->level0.count);
@@ -909,6 +1561,9 @@ gmg_status gmg_batch_create(int count, const int* d, const int* n, const gmg_con
                         b->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->di, b->items.data(), sizeof(Item) * b->items.size(),
+                            cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess && !b->tiles.empty())
+        e = cudaMemcpyAsync(b->dt, b->tiles.data(), sizeof(Tile) * b->tiles.size(),
                             cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return fail(GMG_ERR_CUDA, cudaGetErrorString(e));
