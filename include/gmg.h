@@ -143,7 +143,8 @@ gmg_status gmg_config_init(gmg_config* cfg, int d, int n);
  * cycle.  Cycle counts are the same; iterates agree to the double-float
  * rounding of the correction (far below 1e-12 of u per cycle).
  * GMG_FUSED_LEGS=0/1 turns the fused leg kernels off / on for every FP32
- * and double-float level that takes them (default: FP32 levels n >= 512);
+ * and double-float level that takes them, and those of the 2D FP64 levels up to
+ * 512 (default: FP32 levels n >= 256, 2D FP64 levels);
  * GMG_LEG_NMIN / GMG_LEG_NMAX bound the level sizes; results are the same bit
  * for bit.  GMG_GRID_TAIL_N=m runs the levels with n <= m (red-black) and
  * all smaller ones as one cooperative launch with grid barriers between the

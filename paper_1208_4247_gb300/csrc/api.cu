@@ -117,10 +117,11 @@ struct gmg_handle_s {
     // cycle's first level-0 red half sweep (norm_ahead_ok)
     bool ahead = false;
     int tail_max = 0;       // GMG_TAIL_N at create: largest tail level n (0 = default)
-    // fused leg kernels (legs.cu) on large 3D levels of the red-black inner
-    // hierarchies.  legs_mode 1 (default): FP32 levels with n >= 512, where
-    // they beat the unfused kernels; 2 (GMG_FUSED_LEGS=1 at create): FP32
-    // and double-float levels with n >= 128; 0 (GMG_FUSED_LEGS=0): off.
+    // fused leg kernels (legs_reg.cu, legs.cu) on large 3D levels of the
+    // red-black inner hierarchies.  legs_mode 1 (default): FP32 levels with n
+    // >= 256, where they beat the unfused kernels; 2 (GMG_FUSED_LEGS=1 at
+    // create): FP32 and double-float levels with n >= 128; 0
+    // (GMG_FUSED_LEGS=0): off.
     // GMG_LEG_NMIN overrides the smallest level n.
     int legs_mode = 1;
     int leg_nmin = 0;
@@ -459,19 +460,28 @@ void relax(gmg_handle h, std::vector<Level<T>>& lv, int l, int sweeps, int& cur,
     }
 }
 
-// The fused leg kernels (legs.cu) run level l of an FP32 / double-float 3D
-// red-black hierarchy: ping-pong iterate arrays, a level that legs::applies
-// takes, at least GMG_LEG_NMIN intervals.
+// The fused leg kernels run level l of a 3D red-black inner hierarchy
+// (ping-pong iterate arrays, a level that the kernels take, at least
+// GMG_LEG_NMIN intervals): FP32 by legs_reg.cu, double-float (on request) by
+// legs.cu.  FP32 from n = 256: one refinement step of 3 V(2,2) cycles takes
+// 2.79 ms with them and 3.20 without at 256, 15.2 and 20.4 at 512 (V(1,1), 2
+// cycles: 2.04 and 2.04, 12.8 and 13.3), but 0.83 and 0.82 at 128.  In BF16,
+// whose sweeps move half the bytes, the same kernels lost (2.95 and 2.58 ms at
+// 256, 16.1 and 15.7 at 512).
 template <typename T>
 bool leg_possible(gmg_handle h, int n) {
     const gmg_config& c = h->cfg;
-    const int nmin = h->leg_nmin > 0 ? h->leg_nmin : h->legs_mode == 1 ? 512 : 128;
-    const bool type_ok = std::is_same<T, float>::value ||
-                         (std::is_same<T, df32>::value && h->legs_mode == 2);
-    if constexpr (std::is_same<T, float>::value || std::is_same<T, df32>::value)
-        return h->legs_mode > 0 && type_ok && c.d == 3 && c.smoother == GMG_RBGS &&
-               c.transfer != GMG_TRANSFER_PAPER && !use_fused_rb<T>(h) && n >= nmin &&
-               (h->leg_nmax == 0 || n <= h->leg_nmax) && legs::applies<T>(c.d, n);
+    if constexpr (std::is_same<T, float>::value || std::is_same<T, df32>::value) {
+        if (h->legs_mode <= 0 || c.d != 3 || c.smoother != GMG_RBGS ||
+            c.transfer == GMG_TRANSFER_PAPER || use_fused_rb<T>(h) ||
+            (h->leg_nmax > 0 && n > h->leg_nmax))
+            return false;
+        if (std::is_same<T, df32>::value)
+            return h->legs_mode == 2 && n >= (h->leg_nmin > 0 ? h->leg_nmin : 128) &&
+                   legs::applies<df32>(c.d, n);
+        const int nmin = h->leg_nmin > 0 ? h->leg_nmin : h->legs_mode == 1 ? 256 : 128;
+        return n >= nmin && rlegs::applies(c.d, n);
+    }
     return false;
 }
 template <typename T>
@@ -654,17 +664,24 @@ gmg_status enqueue_vcycle(gmg_handle h, std::vector<Level<T>>& lv, bool first_re
                 Level<T>& F = lv[l];
                 Level<T>& C = lv[l + 1];
                 cudaError_t e = cudaSuccess;
+                constexpr bool kReg = std::is_same<T, float>::value;
+                const int init = kReg ? level_init<T>(h, lv, l + 1) : INIT_ZERO;
                 timed(
                     h, K_LEG_DOWN, l, p, F.n, true,
                     [&] {
-                        e = legs::down<T>(F.lay, C.lay, F.u[cur[l]], F.u[cur[l] ^ 1], F.q, C.q,
-                                          C.u[0], s_down, h->stream);
+                        if constexpr (kReg)
+                            e = rlegs::down(F.lay, C.lay, F.u[cur[l]], F.u[cur[l] ^ 1], F.q,
+                                            C.q, C.u[0], init, s_down, h->stream);
+                        else if constexpr (std::is_same<T, df32>::value)
+                            e = legs::down<T>(F.lay, C.lay, F.u[cur[l]], F.u[cur[l] ^ 1], F.q,
+                                              C.q, C.u[0], s_down, h->stream);
                     },
                     1, s_down);
                 GMG_CUDA_TRY(e);
-                h->legs_used = true;
+                h->legs_used = h->legs_used || !kReg;
                 cur[l] ^= 1;
                 cur[l + 1] = 0;
+                done[l + 1] = init > INIT_EXACT;
                 continue;
             }
             if constexpr (std::is_same<T, double>::value) {
@@ -758,12 +775,16 @@ gmg_status enqueue_vcycle(gmg_handle h, std::vector<Level<T>>& lv, bool first_re
                 timed(
                     h, K_LEG_UP, l, p, F.n, true,
                     [&] {
-                        e = legs::up<T>(C.lay, F.lay, C.u[cur[l + 1]], F.u[cur[l]],
-                                        F.u[cur[l] ^ 1], F.q, s_up, h->stream);
+                        if constexpr (std::is_same<T, float>::value)
+                            e = rlegs::up(C.lay, F.lay, C.u[cur[l + 1]], F.u[cur[l]],
+                                          F.u[cur[l] ^ 1], F.q, s_up, h->stream);
+                        else if constexpr (std::is_same<T, df32>::value)
+                            e = legs::up<T>(C.lay, F.lay, C.u[cur[l + 1]], F.u[cur[l]],
+                                            F.u[cur[l] ^ 1], F.q, s_up, h->stream);
                     },
                     1, s_up);
                 GMG_CUDA_TRY(e);
-                h->legs_used = true;
+                h->legs_used = h->legs_used || std::is_same<T, df32>::value;
                 cur[l] ^= 1;
                 continue;
             }

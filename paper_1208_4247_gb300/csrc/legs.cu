@@ -1,4 +1,5 @@
-// Fused leg kernels (legs.cuh) on the GPU: the plane boxes arrive by TMA
+// Fused leg kernels (legs.cuh) on the GPU, double-float storage (FP32 takes
+// legs_reg.cu): the plane boxes arrive by TMA
 // (cp.async.bulk.tensor, one tensor map per array, this GPU's own memory),
 // each batch signalled by an mbarrier; the waits are bounded, and a CTA that
 // gives up records a fault word (read by the solve) instead of hanging.
@@ -148,7 +149,7 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 }
 
 // A 3D tensor map over a colour-split level array {sy, n+1, n+1} (elements
-// of es bytes) with box {bx, by, 1}; rows and planes beyond the grid and
+// of es = 8 bytes) with box {bx, by, 1}; rows and planes beyond the grid and
 // entries beyond the row read as zero.
 bool make_map(CUtensorMap* m, const void* base, const LayS& L, int es, int bx, int by) {
     auto fn = encode_fn();
@@ -160,7 +161,7 @@ bool make_map(CUtensorMap* m, const void* base, const LayS& L, int es, int bx, i
     const cuuint64_t strides[2] = {(cuuint64_t)L.sy * es, (cuuint64_t)L.sz * es};
     const cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, 1u};
     const cuuint32_t estr[3] = {1u, 1u, 1u};
-    const CUresult r = fn(m, es == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64,
+    const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT64,
                           3, const_cast<void*>(base), dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -281,14 +282,9 @@ int fault() {
     return v;
 }
 
-template bool applies<float>(int, int);
 template bool applies<df32>(int, int);
-template cudaError_t down<float>(const Lay&, const Lay&, const float*, float*, const float*,
-                                 float*, float*, int, cudaStream_t);
 template cudaError_t down<df32>(const Lay&, const Lay&, const df32*, df32*, const df32*, df32*,
                                 df32*, int, cudaStream_t);
-template cudaError_t up<float>(const Lay&, const Lay&, const float*, const float*, float*,
-                               const float*, int, cudaStream_t);
 template cudaError_t up<df32>(const Lay&, const Lay&, const df32*, const df32*, df32*,
                               const df32*, int, cudaStream_t);
 

@@ -11,7 +11,7 @@
 namespace gmg {
 namespace legs {
 // whether a 3D level of n intervals takes the leg kernels for storage T
-// (float or df32): n a multiple of the column width and at least two columns
+// (df32): n a multiple of the column width and at least two columns
 template <typename T>
 bool applies(int d, int n);
 // down leg on fine level F (coarse C): S half sweeps of u_in (colours
@@ -28,4 +28,15 @@ cudaError_t up(const Lay& C, const Lay& F, const T* ec, const T* u_in, T* u_out,
 // nonzero once a leg kernel gave up waiting for its plane loads (sticky)
 int fault();
 }  // namespace legs
+
+// FP32 storage, planes in registers (legs_reg.cu): n a power of two from 128
+// up.  init: what u_c starts from (INIT_ZERO or INIT_RED).  S: 2 to 4 down, 2
+// or 4 up.
+namespace rlegs {
+inline bool applies(int d, int n) { return d == 3 && n >= 128; }
+cudaError_t down(const Lay& F, const Lay& C, const float* u_in, float* u_out, const float* q,
+                 float* qc, float* uc, int init, int S, cudaStream_t s);
+cudaError_t up(const Lay& C, const Lay& F, const float* ec, const float* u_in, float* u_out,
+               const float* q, int S, cudaStream_t s);
+}  // namespace rlegs
 }  // namespace gmg
