@@ -961,7 +961,7 @@ __global__ void __launch_bounds__(256) k_outer(const Item* __restrict__ items, i
                 s += u[p + sz];
             }
             const double sig = fma(c, s, q[p]) - u[p];
-            qin[pin] = Num<T>::st((float)sig);
+            qin[pin] = Num<T>::st(cvt::narrow(sig));  // FP64 pipe: one slot less
             acc = fma(sig, sig, acc);
         }
         for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);

@@ -50,7 +50,14 @@ __device__ inline void store_inner(T* __restrict__ q_in, T* __restrict__ e_init,
                                    double sig, bool red, float* __restrict__ resid) {
     using N = lk::Num<T>;
     using C = typename N::C;
-    const T s = N::st(C(sig));
+    // FP32 / BF16 storage: rounded on the integer pipe, because the cast takes
+    // a slot of the FP64 pipe, which bounds the kernel (257^3, BF16: 307 us with
+    // the cast, 281 without)
+    T s;
+    if constexpr (std::is_same<C, float>::value)
+        s = N::st(cvt::narrow(sig));
+    else
+        s = N::st(C(sig));
     q_in[idx] = s;
     if (e_init) e_init[idx] = red ? s : N::st(C(0));
     if constexpr (std::is_same<T, df32>::value) {
@@ -98,7 +105,7 @@ __device__ inline void zero_iterate_sigma(const double* __restrict__ q, T* __res
                         resid);
             acc = fma(sig, sig, acc);
             if (qsum) {
-                const float qf = (float)q[row + i];
+                const float qf = cvt::narrow(q[row + i]);
                 accq = fmaf(qf, qf, accq);
             }
         }
@@ -139,7 +146,7 @@ __global__ void __launch_bounds__(kThreads) k_outer_residual(const double* __res
                         resid);
             acc = fma(sig, sig, acc);
             if (qpart) {  // FP32: a threshold test, kept off the FP64 pipe
-                const float qf = (float)q[p];
+                const float qf = cvt::narrow(q[p]);
                 accq = fmaf(qf, qf, accq);
             }
         }
@@ -181,7 +188,7 @@ __global__ void __launch_bounds__(256, 4) k_outer_residual3_walk(const double* _
                             color == 0, resid);
                 acc = fma(sig, sig, acc);
                 if (qpart) {  // FP32: a threshold test, kept off the FP64 pipe
-                const float qf = (float)q[p];
+                const float qf = cvt::narrow(q[p]);
                 accq = fmaf(qf, qf, accq);
             }
             });
