@@ -116,24 +116,29 @@ __global__ void __launch_bounds__(kNormThreads) k_resnorm(const double* __restri
     }
 }
 
-// One-colour norm by the diagonal walkers (3D, 128 <= n <= 512).  Colour 0
-// (red): the same sigma^2 terms as k_resnorm<3, false, true>, summed in
-// walker order.  Colour 1 (black): the black half of a solve's first norm.
-// A fixed grid strides over the walkers, so the result is deterministic.
+// The norm by the diagonal walkers (3D, 128 <= n <= 512) over the colours from
+// color0 to color1.  Red: the same sigma^2 terms as k_resnorm<3, false, true>,
+// summed in walker order.  Black: the other half of a solve's first norm.  Both
+// with STORE: k_resnorm<3, true, false>'s sigma, bit for bit (257^3: 245 us, there 278).  A
+// fixed grid strides over the walkers, so the result is deterministic.
+template <bool STORE>
 __global__ void __launch_bounds__(256, 4) k_resnorm3_walk(const double* __restrict__ u,
                                                           const double* __restrict__ q,
                                                           double* __restrict__ partial, int n,
-                                                          int segs, int color) {
+                                                          int segs, int color0, int color1,
+                                                          double* __restrict__ sig_out) {
     __shared__ double warp_sums[kNormThreads / 32];
     const double c = 1.0 / 6.0;
     const int64_t walkers = (int64_t)(n - 1) * segs;
     double acc = 0.0;
     for (int64_t w = (int64_t)blockIdx.x * blockDim.y + threadIdx.y; w < walkers;
          w += (int64_t)gridDim.x * blockDim.y)
-        lk::walk_nodes(u, n, color, w, segs, [&](int64_t p, double sum, int, int, int) {
-            const double sig = fma(c, sum, q[p]) - u[p];
-            acc = fma(sig, sig, acc);
-        });
+        for (int color = color0; color <= color1; ++color)
+            lk::walk_nodes(u, n, color, w, segs, [&](int64_t p, double sum, int, int, int) {
+                const double sig = fma(c, sum, q[p]) - u[p];
+                if (STORE) sig_out[p] = sig;
+                acc = fma(sig, sig, acc);
+            });
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
     const int t = threadIdx.y * blockDim.x + threadIdx.x;
     if ((t & 31) == 0) warp_sums[t >> 5] = acc;
@@ -373,7 +378,7 @@ void resnorm_black(int n, const double* u, const double* q, double* partial, dou
                    cudaStream_t s) {
     const lk::WalkLaunch W = lk::walk_launch(n);
     const unsigned blocks = std::min<unsigned>(W.blocks, (unsigned)resnorm_partials(3, n));
-    k_resnorm3_walk<<<blocks, W.block, 0, s>>>(u, q, partial, n, W.segs, 1);
+    k_resnorm3_walk<false><<<blocks, W.block, 0, s>>>(u, q, partial, n, W.segs, 1, 1, nullptr);
     k_sum_partials<<<1, 1024, 0, s>>>(partial, (int)blocks, out);
 }
 
@@ -385,14 +390,16 @@ void red_restore(int n, double* u, const double* save, cudaStream_t s) {
 
 int resnorm(int d, int n, const double* u, const double* q, double* partial, double* out,
             cudaStream_t s, double* sigma_out, bool red_only) {
-    if (red_only && !sigma_out && lk::walk_applies(d, n, sizeof(double))) {
+    red_only = red_only && !sigma_out;
+    if (lk::walk_applies(d, n, sizeof(double))) {
         const lk::WalkLaunch W = lk::walk_launch(n);
         const unsigned blocks = std::min<unsigned>(W.blocks, (unsigned)resnorm_partials(d, n));
-        k_resnorm3_walk<<<blocks, W.block, 0, s>>>(u, q, partial, n, W.segs, 0);
+        auto k = sigma_out ? k_resnorm3_walk<true> : k_resnorm3_walk<false>;
+        k<<<blocks, W.block, 0, s>>>(u, q, partial, n, W.segs, 0, red_only ? 0 : 1, sigma_out);
         if (out) k_sum_partials<<<1, 1024, 0, s>>>(partial, (int)blocks, out);
         return (int)blocks;
     }
-    NormLaunch L = norm_launch(d, n, red_only && !sigma_out);
+    NormLaunch L = norm_launch(d, n, red_only);
     if (sigma_out) {
         if (d == 3)
             k_resnorm<3, true, false><<<L.grid, L.block, 0, s>>>(u, q, partial, n, sigma_out);

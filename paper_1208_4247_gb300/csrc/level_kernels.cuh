@@ -618,9 +618,11 @@ __device__ inline void walk_nodes(const T* __restrict__ u, int n, int color, int
     }
 }
 
-// Red-only residual (after a black half sweep) by diagonal walkers: sigma
-// at the red nodes, equal to k_residual<3, true>'s bit for bit.
-template <typename T, bool EXACT = false>
+// Residual by diagonal walkers: sigma at the red nodes (after a black half
+// sweep; COLORS = 1) or at all (the walker goes over its nodes colour by
+// colour), equal to k_residual<3>'s bit for bit with 6.25 instead of 7 FP64
+// instructions per node.  All nodes at 257^3: 221 us (a thread per node, 246).
+template <typename T, bool EXACT = false, int COLORS = 1>
 __global__ void __launch_bounds__(256, 4) k_residual3_walk(const T* __restrict__ u,
                                                            const T* __restrict__ q,
                                                            T* __restrict__ r, int n, int segs) {
@@ -629,9 +631,10 @@ __global__ void __launch_bounds__(256, 4) k_residual3_walk(const T* __restrict__
     const C c = C(1.0 / 6.0);
     const int64_t w = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
     if (w >= (int64_t)(n - 1) * segs) return;
-    walk_nodes(u, n, 0, w, segs, [&](int64_t p, C sum, int, int, int) {
-        r[p] = N::st(gs_value<3, EXACT>(c, sum, N::ld(q[p])) - N::ld(u[p]));
-    });
+    for (int color = 0; color < COLORS; ++color)
+        walk_nodes(u, n, color, w, segs, [&](int64_t p, C sum, int, int, int) {
+            r[p] = N::st(gs_value<3, EXACT>(c, sum, N::ld(q[p])) - N::ld(u[p]));
+        });
 }
 
 // Launch shape of the walker kernels for a 3D level n (128 <= n <= 512):
@@ -859,8 +862,10 @@ constexpr int kZWalk = 4;  // restriction
 // of whose offsets are +-1.  The four of an odd fine plane 2K+1 (offsets
 // (+-1, 0) and (0, +-1) in it) belong to coarse nodes K and K+1: their sum is
 // formed once.  8 adds + 2 multiplies per node instead of 11 + 2; the same
-// terms and weights as k_restrict<3, true>, summed in another order.
-template <typename T>
+// terms and weights as k_restrict<3, true>, summed in another order.  All
+// nodes: [1 2 1] / 2 along x, y and z in turn, 19 instead of 30 FP64
+// instructions per coarse node (257^3 to 129^3: 93 us, 114 by k_restrict).
+template <typename T, bool RED_ONLY = true>
 __global__ void __launch_bounds__(256) k_restrict3_zwalk(const T* __restrict__ r,
                                                          T* __restrict__ qc, T* __restrict__ uc,
                                                          int n, int init, double omega) {
@@ -874,16 +879,26 @@ __global__ void __launch_bounds__(256) k_restrict3_zwalk(const T* __restrict__ r
     const int64_t sy = sy_of(n), sz = sz_of<3>(n);
     const int64_t cy = sy_of(nc), cz = sz_of<3>(nc);
     auto R = [&](int64_t o) { return N::ld(r[o]); };
-    // the four red fine nodes of odd plane z around column (2I, 2J)
-    auto odd_plane = [&](int64_t o) { return ((R(o - 1) + R(o + 1)) + R(o - sy)) + R(o + sy); };
+    // a fine plane around column (2I, 2J): [1 2 1] x [1 2 1] of all nodes, or
+    // the four red ones of an odd plane
+    auto row = [&](int64_t o) { return fma(C(2.0), R(o), R(o - 1) + R(o + 1)); };
+    auto plane = [&](int64_t o) {
+        if (RED_ONLY) return ((R(o - 1) + R(o + 1)) + R(o - sy)) + R(o + sy);
+        return fma(C(2.0), row(o), row(o - sy) + row(o + sy));
+    };
     int64_t p = (int64_t)(2 * K0) * sz + (int64_t)(2 * J) * sy + 2 * I;
     int64_t P = (int64_t)K0 * cz + (int64_t)J * cy + I;
-    C below = odd_plane(p - sz);
+    C below = plane(p - sz);
     const int Kend = min(K0 + kZWalk, nc);
     for (int K = K0; K < Kend; ++K, p += 2 * sz, P += cz) {
-        const C in_plane = ((R(p - 1 - sy) + R(p + 1 - sy)) + R(p - 1 + sy)) + R(p + 1 + sy);
-        const C above = odd_plane(p + sz);
-        const C v = fma(C(0.125), (in_plane + below) + above, C(0.5) * R(p));
+        const C above = plane(p + sz);
+        C v;
+        if (RED_ONLY) {
+            const C in_plane = ((R(p - 1 - sy) + R(p + 1 - sy)) + R(p - 1 + sy)) + R(p + 1 + sy);
+            v = fma(C(0.125), (in_plane + below) + above, C(0.5) * R(p));
+        } else {
+            v = C(0.0625) * fma(C(2.0), plane(p), below + above);
+        }
         qc[P] = N::st(v);
         uc[P] = coarse_init<3>(init, omega, I, J, K, N::st(v));
         below = above;
@@ -1160,12 +1175,11 @@ void residual(int d, const Lay& L, const T* u, const T* q, T* r, bool red_only, 
     const int n = L.n;
     constexpr bool kFp64 = std::is_same<T, double>::value;
     exact = exact && kFp64 && d == 3;
-    if (red_only && L.he == 0 && walk_applies(d, n, sizeof(T))) {
+    if (L.he == 0 && walk_applies(d, n, sizeof(T))) {
         const WalkLaunch W = walk_launch(n);
-        if (exact)
-            k_residual3_walk<T, kFp64><<<W.blocks, W.block, 0, s>>>(u, q, r, n, W.segs);
-        else
-            k_residual3_walk<T><<<W.blocks, W.block, 0, s>>>(u, q, r, n, W.segs);
+        auto k = red_only ? (exact ? k_residual3_walk<T, kFp64, 1> : k_residual3_walk<T, false, 1>)
+                          : (exact ? k_residual3_walk<T, kFp64, 2> : k_residual3_walk<T, false, 2>);
+        k<<<W.blocks, W.block, 0, s>>>(u, q, r, n, W.segs);
         return;
     }
     if (exact && L.he == 0) {
@@ -1232,9 +1246,10 @@ void restrict_fw(int d, const Lay& F, const Lay& C, const T* r, T* qc, T* uc, bo
     dim3 block(bx, by, 1);
     dim3 grid((nc - 1 + bx - 1) / bx, (nc - 1 + by - 1) / by, d == 3 ? nc - 1 : 1);
     if constexpr (std::is_same<T, double>::value) {
-        if (red_only && init != INIT_EXACT && zwalk_applies(d, F)) {
+        if (init != INIT_EXACT && zwalk_applies(d, F)) {
             const dim3 gz(grid.x, grid.y, (unsigned)((nc - 1 + kZWalk - 1) / kZWalk));
-            k_restrict3_zwalk<T><<<gz, block, 0, s>>>(r, qc, uc, F.n, init, omega);
+            auto k = red_only ? k_restrict3_zwalk<T, true> : k_restrict3_zwalk<T, false>;
+            k<<<gz, block, 0, s>>>(r, qc, uc, F.n, init, omega);
             return;
         }
     }
