@@ -334,7 +334,7 @@ FMG_SWEEPS = ((1, 1), (1, 2), (2, 2), (2, 3), (3, 3))
 
 def run_fmg_vs_fft(torch, args):
     """Section 5.4's comparison at 16M unknowns (2D 4097^2, 3D 257^3): one
-    FMG(nu1, nu2) pass (Algorithm 2) against the direct cuFFT DST-I solve, on
+    FMG(nu1, nu2) pass (Algorithm 2) against the direct DST-I solve, on
     the manufactured problem u = prod sin(pi x_m), f = d pi^2 u.  Each pass is
     timed with CUDA events around the public call (scaling of f, the FMG
     graph, the residual norm and its host read included); the L2(Omega)
@@ -857,7 +857,8 @@ def run_ours(args, rank, ws, local):
            "frac": alg_bytes / (ms_step * 1e-3) / 1e9 / pk["hbm_gbs"],
            "frac_of_nominal_8000": alg_bytes / (ms_step * 1e-3) / 1e9 / 8000.0}
 
-    # the paper's comparison point: direct cuFFT DST-I solve of the same system
+    # the paper's comparison point: direct DST-I solve of the same system (the
+    # record keeps the name it had when cuFFT made the transforms)
     from paper_1208_4247_gb300.gmg import FFTSolver
     F = FFTSolver(D, N)
     uf = torch.zeros_like(f)
