@@ -46,24 +46,53 @@ constexpr int kThreads = 256;
 // the part of sigma the double-float value of q_in leaves out (about 2^-49
 // of sigma; see k_black_exact_update).
 template <typename T>
-__device__ inline void store_inner(T* __restrict__ q_in, T* __restrict__ e_init, int64_t idx,
-                                   double sig, bool red, float* __restrict__ resid) {
+__device__ inline void store_value(T* __restrict__ q_in, T* __restrict__ e_init, int64_t idx,
+                                   T s, bool red) {
+    using N = lk::Num<T>;
+    q_in[idx] = s;
+    if (e_init) e_init[idx] = red ? s : N::st(typename N::C(0));
+}
+
+// sigma of a node with neighbour sum `sum`, right-hand side q and value u:
+// stored, and the factor that kScale undoes in its square returned.
+//
+// FP32 and BF16 storage in 3D: 6 sigma = 6 q + (sum - 6 u) in two fused
+// multiply-adds (the inner one cancels u with one rounding), instead of two for the
+// unbiased 1/6 and a subtraction; the division by 6 and the rounding to T go to
+// the integer and FP32 pipes (cvt::split, sixth: 2^-47 before the one rounding
+// to 24 bits).  Other types of FP32 arithmetic: rounded on the integer pipe,
+// because the cast takes a slot of the FP64 pipe, which bounds the kernel.  257^3, BF16:
+// 307 us with the cast and the subtraction, 281 without the cast, 248 in this form; 513^3, FP32: 2334, 2297, 1865 us.
+template <int DIM, typename T>
+struct Sigma {
     using N = lk::Num<T>;
     using C = typename N::C;
-    // FP32 / BF16 storage: rounded on the integer pipe, because the cast takes
-    // a slot of the FP64 pipe, which bounds the kernel (257^3, BF16: 307 us with
-    // the cast, 281 without)
-    T s;
-    if constexpr (std::is_same<C, float>::value)
-        s = N::st(cvt::narrow(sig));
-    else
-        s = N::st(C(sig));
-    q_in[idx] = s;
-    if (e_init) e_init[idx] = red ? s : N::st(C(0));
-    if constexpr (std::is_same<T, df32>::value) {
-        if (resid && !red) resid[idx] = (float)((sig - cvt::widen(s.hi)) - cvt::widen(s.lo));
+    static constexpr bool kF = std::is_same<C, float>::value, kSix = kF && DIM == 3;
+    static constexpr double kScale = kSix ? 1.0 / 36.0 : 1.0;
+    static __device__ __forceinline__ double at(double sum, double q, double u) {
+        if constexpr (kSix)
+            return fma(6.0, q, fma(-6.0, u, sum));
+        else
+            return lk::gs_value<DIM, true>(DIM == 3 ? 1.0 / 6.0 : 0.25, sum, q) - u;
     }
-}
+    static __device__ __forceinline__ double at_zero(double q) {
+        return kSix ? fma(6.0, q, 0.0) : q + 0.0;
+    }
+    static __device__ __forceinline__ void store(T* __restrict__ q_in, T* __restrict__ e_init,
+                                                 int64_t idx, double sig, bool red,
+                                                 float* __restrict__ resid) {
+        if constexpr (kSix) {
+            store_value(q_in, e_init, idx, N::st(sixth(df32(sig)).hi), red);
+        } else if constexpr (kF) {
+            store_value(q_in, e_init, idx, N::st(cvt::narrow(sig)), red);
+        } else {
+            const T s = N::st(C(sig));
+            store_value(q_in, e_init, idx, s, red);
+            if (resid && !red)
+                resid[idx] = (float)((sig - cvt::widen(s.hi)) - cvt::widen(s.lo));
+        }
+    }
+};
 
 // The block's sum of acc (a fixed order: warp shuffles, then the warps in
 // turn) into *slot; every thread of the block calls it.
@@ -100,9 +129,9 @@ __device__ inline void zero_iterate_sigma(const double* __restrict__ q, T* __res
         const int64_t row = k * sz + j * sy;
         const int64_t row_in = k * in.sz + j * in.sy;
         for (int i = 1 + tx; i < n; i += blockDim.x) {
-            const double sig = q[row + i] + 0.0;
-            store_inner(q_in, e_init, row_in + lk::xo<SPLIT>(in, i), sig, ((i + j + k) & 1) == 0,
-                        resid);
+            const double sig = Sigma<DIM, T>::at_zero(q[row + i]);
+            Sigma<DIM, T>::store(q_in, e_init, row_in + lk::xo<SPLIT>(in, i), sig,
+                                 ((i + j + k) & 1) == 0, resid);
             acc = fma(sig, sig, acc);
             if (qsum) {
                 const float qf = cvt::narrow(q[row + i]);
@@ -123,7 +152,6 @@ __global__ void __launch_bounds__(kThreads) k_outer_residual(const double* __res
                                                              double* __restrict__ qpart,
                                                              const int* __restrict__ unz) {
     __shared__ double warp_sums[kThreads / 32];
-    const double c = DIM == 3 ? 1.0 / 6.0 : 0.25;
     if (resid_flag && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) *resid_flag = 1;
     const int n = in.n;
     const int64_t sy = sy_of(n), sz = sz_of<DIM>(n);
@@ -141,9 +169,9 @@ __global__ void __launch_bounds__(kThreads) k_outer_residual(const double* __res
         const int64_t row_in = k * in.sz + j * in.sy;
         for (int i = 1 + threadIdx.x; i < n; i += blockDim.x) {
             const int64_t p = row + i;
-            const double sig = lk::gs_value<DIM, true>(c, lk::nbr_sum<DIM>(u, p, sy, sz), q[p]) - u[p];
-            store_inner(q_in, e_init, row_in + lk::xo<SPLIT>(in, i), sig, ((i + j + k) & 1) == 0,
-                        resid);
+            const double sig = Sigma<DIM, T>::at(lk::nbr_sum<DIM>(u, p, sy, sz), q[p], u[p]);
+            Sigma<DIM, T>::store(q_in, e_init, row_in + lk::xo<SPLIT>(in, i), sig,
+                                 ((i + j + k) & 1) == 0, resid);
             acc = fma(sig, sig, acc);
             if (qpart) {  // FP32: a threshold test, kept off the FP64 pipe
                 const float qf = cvt::narrow(q[p]);
@@ -151,13 +179,14 @@ __global__ void __launch_bounds__(kThreads) k_outer_residual(const double* __res
             }
         }
     }
-    block_partial(acc, warp_sums, partial + blockIdx.x);
+    block_partial(acc * Sigma<DIM, T>::kScale, warp_sums, partial + blockIdx.x);
     if (qpart) block_partial((double)accq, warp_sums, qpart + blockIdx.x);
 }
 
 // The same by the diagonal walkers of the FP64 3D sweeps (both colours per
 // walker): 6.25 instead of 7 FP64 instructions per node for sigma, the same
-// sigma values; a fixed grid strides over the walkers (deterministic sum).
+// sigma values (FP32 / BF16: 5.25, Sigma); a fixed grid strides over the walkers
+// (deterministic sum).
 template <bool SPLIT, typename T>
 __global__ void __launch_bounds__(256, 4) k_outer_residual3_walk(const double* __restrict__ u,
                                                                  const double* __restrict__ q,
@@ -170,7 +199,6 @@ __global__ void __launch_bounds__(256, 4) k_outer_residual3_walk(const double* _
                                                                  double* __restrict__ qpart,
                                                                  const int* __restrict__ unz) {
     __shared__ double warp_sums[kThreads / 32];
-    const double c = 1.0 / 6.0;
     const int n = in.n;
     const int64_t walkers = (int64_t)(n - 1) * segs;
     if (resid_flag && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) *resid_flag = 1;
@@ -183,16 +211,16 @@ __global__ void __launch_bounds__(256, 4) k_outer_residual3_walk(const double* _
          w += (int64_t)gridDim.x * blockDim.y)
         for (int color = 0; color < 2; ++color)
             lk::walk_nodes(u, n, color, w, segs, [&](int64_t p, double sum, int i, int j, int k) {
-                const double sig = lk::gs_value<3, true>(c, sum, q[p]) - u[p];
-                store_inner(q_in, e_init, k * in.sz + j * in.sy + lk::xo<SPLIT>(in, i), sig,
-                            color == 0, resid);
+                const double sig = Sigma<3, T>::at(sum, q[p], u[p]);
+                Sigma<3, T>::store(q_in, e_init, k * in.sz + j * in.sy + lk::xo<SPLIT>(in, i), sig,
+                                   color == 0, resid);
                 acc = fma(sig, sig, acc);
                 if (qpart) {  // FP32: a threshold test, kept off the FP64 pipe
                 const float qf = cvt::narrow(q[p]);
                 accq = fmaf(qf, qf, accq);
             }
             });
-    block_partial(acc, warp_sums, partial + blockIdx.x);
+    block_partial(acc * Sigma<3, T>::kScale, warp_sums, partial + blockIdx.x);
     if (qpart) block_partial((double)accq, warp_sums, qpart + blockIdx.x);
 }
 
