@@ -13,6 +13,7 @@
 // One refinement step of the whole batch is captured into one CUDA graph;
 // the host reads one counter (solves still active) per step.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <string>
 #include <vector>
@@ -1037,6 +1038,7 @@ struct Step {
 struct gmg_batch_s {
     gmg_config cfg{};
     int count = 0, chunk = 1024, ctas = 608, device = 0, G = 0, elem = 4;
+    int leg_ctas = 0;  // the legs' grids: a CTA per tile, up to the caller's ctas if given
     int sms = 152;
     // stream2: the 2D solves' launches inside the captured step, which depend
     // on none of the 3D solves'
@@ -1142,13 +1144,13 @@ gmg_status enqueue_cycles(gmg_batch b, int d, cudaStream_t st) {
                      (sweep_down ? 3.125 : 2.125) * w * S.down.nodes, 1, [&] {
                          if (d == 3) {
                              auto k = sweep_down ? k_down3<T, true> : k_down3<T, false>;
-                             k<<<std::min(nt, b->ctas), th, 160 * th, st>>>(
+                             k<<<std::min(nt, b->leg_ctas), th, 160 * th, st>>>(
                                  t, nt, b->ds, b->dl, pool, pool, b->active, src, dst, zero, clear,
                                  omega);
                          } else {
                              const int ctas = (nt * S.lanes + 127) / 128;
                              auto k = sweep_down ? k_down2<T, true> : k_down2<T, false>;
-                             k<<<std::min(ctas, b->ctas), 128, 0, st>>>(
+                             k<<<std::min(ctas, b->leg_ctas), 128, 0, st>>>(
                                  t, nt, b->ds, b->dl, pool, pool, b->active, src, dst, zero, clear,
                                  omega, S.lanes);
                          }
@@ -1162,11 +1164,11 @@ gmg_status enqueue_cycles(gmg_batch b, int d, cudaStream_t st) {
         b->timer.run(st, std::string("b_up_leg") + PrecName<T>::s, g, 12.0 * S.up.nodes,
                      3.125 * w * S.up.nodes, 1, [&] {
                          if (d == 3)
-                             k_up3<T><<<std::min(nt, b->ctas), th, 64 * th, st>>>(
+                             k_up3<T><<<std::min(nt, b->leg_ctas), th, 64 * th, st>>>(
                                  t, nt, b->ds, b->dl, pool, pool, b->active, src, src ^ 1, cc,
                                  omega);
                          else
-                             k_up2<T><<<std::min((nt * S.lanes + 127) / 128, b->ctas), 128, 0, st>>>(
+                             k_up2<T><<<std::min((nt * S.lanes + 127) / 128, b->leg_ctas), 128, 0, st>>>(
                                  t, nt, b->ds, b->dl, pool, pool, b->active, src, src ^ 1, cc,
                                  omega, S.lanes);
                      });
@@ -1389,6 +1391,7 @@ gmg_status gmg_batch_create(int count, const int* d, const int* n, const gmg_con
     if (cudaGetDevice(&b->device) != cudaSuccess) return fail(GMG_ERR_CUDA, "no device");
     cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device);
     b->ctas = ctas > 0 ? ctas : 4 * b->sms;
+    b->leg_ctas = ctas > 0 ? ctas : INT_MAX;
     if (cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&b->stream2, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess ||
