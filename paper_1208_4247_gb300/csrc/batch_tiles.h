@@ -66,7 +66,7 @@ inline int leg_rows(int n, int threads) { return 2 * (threads / std::min(n / 4, 
 inline int leg_pieces(int64_t columns, int64_t slots, int len, int unit, int extra) {
     int best = 1;
     int64_t cost = INT64_MAX;
-    for (int p = 1; p <= std::max(1, len / 4); ++p) {
+    for (int p = 1; p <= len; ++p) {
         const int64_t waves = (columns * p + slots - 1) / slots;
         const int64_t c = waves * ((int64_t)unit * ((len + p - 1) / p) + extra);
         if (c < cost) {
