@@ -317,10 +317,10 @@ gmg_status gmg_fft_destroy(gmg_fft h);
 
 /* ---------------------------------------------------------------- batches
  * Many independent solves of uneven sizes (2D and 3D mixed) advanced
- * together: every step launches one persistent kernel per level index over
- * the whole batch (work items = chunks of one solve's level grid), so the
- * coarse levels of the large solves share launches with the fine levels of
- * the small ones.  Levels are aligned at the coarsest (3^d) grid.  Cycles run
+ * together: every operation is one launch per level index over the whole
+ * batch (a leg down and a leg up per level of the weighted-Jacobi cycle, for
+ * the 2D and the 3D solves side by side), so the coarse levels of the large
+ * solves share launches with the fine levels of the small ones.  Levels are aligned at the coarsest (3^d) grid.  Cycles run
  * in the inner precision of *common (GMG_FP32_IR or GMG_BF16_IR: FP64 outer
  * residual, update and norm; GMG_FP64: plain cycles) with its smoother and
  * sweeps; each solve stops on its own FP64 relative residual (converged
@@ -334,8 +334,9 @@ typedef struct gmg_batch_s* gmg_batch;
  * levels are ignored: every solve uses all its levels).  omega = 0 gives the
  * 2D solves weighted Jacobi with 4/5 and the 3D ones 6/7 (the weight with the
  * smaller two-grid contraction in 3D); any other omega in (0, 2) applies to
- * every solve.  chunk: nodes per
- * work item (0 = 1024); ctas: CTAs per launch (0 = 4 x SM count). */
+ * every solve.  chunk: nodes per work item of the operations that take
+ * chunks of a grid (0 = 1024); ctas: CTAs per launch at most (0 = 4 x SM count
+ * for those, a CTA per tile for the legs). */
 gmg_status gmg_batch_create(int count, const int* d, const int* n, const gmg_config* common,
                             int chunk, int ctas, void* cuda_stream, gmg_batch* out);
 

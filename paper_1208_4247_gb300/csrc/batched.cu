@@ -1,14 +1,15 @@
 // Batched form: many independent Poisson solves of uneven sizes (2D and 3D
 // mixed) advanced together, FP32 or BF16-storage cycles inside FP64
-// iterative refinement, one persistent kernel per level index over the whole
-// batch.
+// iterative refinement.
 //
-// Work items are chunks of one solve's level grid (interior nodes, coarse
-// interior nodes or coarse cells, by operation).  Levels are aligned at the
-// coarsest 3^d grid: level step g processes, for every solve with at least
-// g+1 grids, its level L_s - 1 - g.  The small solves' fine levels thus share
-// launches with the large solves' coarse levels.  Each kernel's CTAs stride
-// over the items of its launch; items of converged solves are skipped
+// Levels are aligned at the coarsest 3^d grid: level step g processes, for
+// every solve with at least g+1 grids, its level L_s - 1 - g, of n = 2^(g+1)
+// intervals.  The small solves' fine levels thus share launches with the large
+// solves' coarse levels.  A step of the weighted-Jacobi cycle is a leg down and
+// a leg up over tiles of all its levels; the 2D and the 3D solves' launches are
+// two branches of the graph.  The other operations take work items that are
+// chunks of one solve's level grid (interior nodes or coarse cells), the CTAs
+// striding over them.  Tiles and items of converged solves are skipped
 // (per-solve active flags, written only by the step's final kernel).
 // One refinement step of the whole batch is captured into one CUDA graph;
 // the host reads one counter (solves still active) per step.
@@ -211,10 +212,11 @@ __global__ void __launch_bounds__(256) k_smooth(const Item* __restrict__ items, 
 // weighting) and one takes it up (prolongation, first post-smoothing sweep):
 // each reads u and q once and writes u once, 12.5 bytes per FP32 node and leg;
 // a kernel per operation moved 29 down and 20.5 up.  The 512-solve batch's step
-// g = 6 (50 solves of 129^3 among them) took 326 + 326 + 261 us down and 251 +
-// 326 us up that way and takes 271 and 206 us now, at the rate of a plain copy;
-// g = 9 (50 of 1025^2) 141 + 140 + 100 and 142 + 141 us, now 146 and 147; the
-// batch 121.1 -> 73.7 ms.
+// g = 6 (70 solves of 129^3 among them) took 326 + 326 + 261 us down and 251 +
+// 326 us up that way and takes 540 and 412 us now (both dimensions, one after
+// the other), about half of a copy's rate: a plane's loads are in flight for one
+// step.  g = 9 (59 of 1025^2) 141 + 140 + 100 and 142 + 141 us, now 146 and 147,
+// 80% of a copy's rate; the batch 121.1 -> 73.7 ms.
 //
 // A thread owns 4 nodes of x (one vector) and, in 3D, two rows of y, and
 // walks z (2D: y) with the planes it still needs in registers; x neighbours

@@ -184,8 +184,8 @@ __global__ void __launch_bounds__(kThreads) k_outer_residual(const double* __res
 }
 
 // The same by the diagonal walkers of the FP64 3D sweeps (both colours per
-// walker): 6.25 instead of 7 FP64 instructions per node for sigma, the same
-// sigma values (FP32 / BF16: 5.25, Sigma); a fixed grid strides over the walkers
+// walker): 7.25 instead of 8 FP64 instructions per node for sigma (FP32 / BF16:
+// 6.25, Sigma), the same sigma values; a fixed grid strides over the walkers
 // (deterministic sum).
 template <bool SPLIT, typename T>
 __global__ void __launch_bounds__(256, 4) k_outer_residual3_walk(const double* __restrict__ u,

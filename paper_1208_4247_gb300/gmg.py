@@ -345,7 +345,7 @@ class Batch:
     """Independent solves of uneven sizes advanced together (gmg_batch_*).
 
     dims, ns: per-solve d and n.  The inner precision ("fp32" / "bf16"),
-    smoother, sweeps and inner cycles are shared; chunk = nodes per work item,
+    smoother, sweeps and inner cycles are shared; chunk = nodes per work item of plain sweeps,
     ctas = CTAs per launch (0 = library defaults)."""
 
     def __init__(self, dims, ns, smoother: str = "wjacobi", omega: float = 0.8, nu1: int = 1,
