@@ -42,14 +42,15 @@ inline std::vector<Rows> rows_up(int n, int R) {
 // Threads of a 3D leg's CTA: n / 4 lanes per row (at most 32) times the pairs
 // of rows.  Levels up to n = 64 are one tile; above, the number of warps (one
 // pair of rows each) that holds the fewest rows in all, the halo rows of the
-// tiles counted: at n = 128 down 4 tiles of 38 rows instead of 5 of 32.
+// tiles counted, of up to 16 warps: with more, the registers of a thread (16384 a
+// scheduler) hold a plane's loads for one step only.
 inline int leg_threads(int n, bool down) {
     if (n <= 16) return 32;
     if (n <= 32) return 128;
     if (n <= 64) return 512;
     int best = 0;
     int64_t cost = 0;
-    for (int w = 20; w >= 12; --w) {
+    for (int w = 16; w >= 12; --w) {
         const int64_t c = (int64_t)2 * w * (down ? rows_down(n, 2 * w) : rows_up(n, 2 * w)).size();
         if (!best || c < cost) {
             best = w;

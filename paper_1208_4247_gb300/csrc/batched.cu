@@ -213,10 +213,11 @@ __global__ void __launch_bounds__(256) k_smooth(const Item* __restrict__ items, 
 // each reads u and q once and writes u once, 12.5 bytes per FP32 node and leg;
 // a kernel per operation moved 29 down and 20.5 up.  The 512-solve batch's step
 // g = 6 (70 solves of 129^3 among them) took 326 + 326 + 261 us down and 251 +
-// 326 us up that way and takes 540 and 412 us now (both dimensions, one after
-// the other), about half of a copy's rate: a plane's loads are in flight for one
-// step.  g = 9 (59 of 1025^2) 141 + 140 + 100 and 142 + 141 us, now 146 and 147,
-// 80% of a copy's rate; the batch 121.1 -> 73.7 ms.
+// 326 us up that way and takes 432 and 408 us now (both dimensions, one after
+// the other), 60% of a copy's rate: at one CTA per SM a plane's loads are in flight
+// for two steps (540 and 412 us with one step, 96 registers and 38 rows a tile; 32
+// rows now, 126 registers).  g = 9 (59 of 1025^2) 141 + 140 + 100 and 142 + 141 us, now 146 and 147,
+// 80% of a copy's rate; the batch 121.1 -> 70.0 ms.
 //
 // A thread owns 4 nodes of x (one vector) and, in 3D, two rows of y, and
 // walks z (2D: y) with the planes it still needs in registers; x neighbours
@@ -328,7 +329,7 @@ __device__ inline void fw_row(float* acc, float l, const float* r, float w) {
 // level / on its coarser levels and is not read.  clear: write u_c = 0 (the
 // coarse level reads it); the one unknown of an n = 2 grid gets u_c = q_c.
 template <typename T, bool SWEEP>
-__global__ void __launch_bounds__(640, 1)
+__global__ void __launch_bounds__(512, 1)
     k_down3(const Tile* __restrict__ tiles, int ntiles, const BSolve* __restrict__ sv,
             const BLevel* __restrict__ lv, const T* __restrict__ pool_in, T* __restrict__ pool_out,
             const int* __restrict__ active, int src, int dst, int zero, int clear, float omega) {
@@ -366,13 +367,17 @@ __global__ void __launch_bounds__(640, 1)
             ld4(a + (int64_t)z * F.sz + F.sy, ok && in1, v[1]);
         };
         const int s0 = 2 * t.ka - (SWEEP ? 3 : 2), s1 = 2 * t.kb;
+        float u2[2][4], qn[2][4];
         load(u, s0, !zs, uc);
         load(u, s0 + 1, !zs, un);
+        load(u, s0 + 2, !zs, u2);
         if (!SWEEP) load(q, s0, true, qc);
+        load(q, s0 + 1, true, qn);
         for (int s = s0; s <= s1; ++s) {
-            float u2[2][4], qn[2][4], v[2][4], r[2][4];
-            load(u, s + 2, !zs && s < s1, u2);
-            load(q, s + 1, s < s1, qn);
+            // two steps ahead of their use
+            float u3[2][4], q2[2][4], v[2][4], r[2][4];
+            load(u, s + 3, !zs && s + 1 < s1, u3);
+            load(q, s + 2, s + 1 < s1, q2);
             const bool zin = s >= 1 && s < n;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -460,9 +465,11 @@ __global__ void __launch_bounds__(640, 1)
                 for (int e = 0; e < 4; ++e) {
                     uc[h][e] = un[h][e];
                     un[h][e] = u2[h][e];
+                    u2[h][e] = u3[h][e];
                     vc[h][e] = v[h][e];
                     qo[h][e] = qc[h][e];
                     qc[h][e] = qn[h][e];
+                    qn[h][e] = q2[h][e];
                 }
             buf ^= 1;
         }
@@ -571,7 +578,7 @@ __device__ inline void widen3(float2 a, int lanes, bool last, float* c) {
 // ccur).  The corners a fine node lies between are added in k_prolong's order
 // (x, then y, then z), so the plane above is added value by value.
 template <typename T>
-__global__ void __launch_bounds__(640, 1)
+__global__ void __launch_bounds__(512, 1)
     k_up3(const Tile* __restrict__ tiles, int ntiles, const BSolve* __restrict__ sv,
           const BLevel* __restrict__ lv, const T* __restrict__ pool_in, T* __restrict__ pool_out,
           const int* __restrict__ active, int src, int dst, int ccur, float omega) {
@@ -659,11 +666,15 @@ __global__ void __launch_bounds__(640, 1)
         cload((s0 >> 1) + 1);
         load(u, s0, true, wc);
         load(u, s0 + 1, true, un);
+        float u2[2][4], qn[2][4];
+        load(u, s0 + 2, true, u2);
+        load(q, s0 + 1, true, qn);
         correct(s0, wc);
         for (int s = s0; s <= s1; ++s) {
-            float u2[2][4], qn[2][4], v[2][4], x[4], a[4], b[4];
-            load(u, s + 2, s < s1, u2);
-            load(q, s + 1, s < s1, qn);
+            // two steps ahead of their use
+            float u3[2][4], q2[2][4], v[2][4], x[4], a[4], b[4];
+            load(u, s + 3, s + 1 < s1, u3);
+            load(q, s + 2, s + 1 < s1, q2);
             correct(s + 1, un);
             if (s >= t.ka) {
 #pragma unroll
@@ -694,7 +705,9 @@ __global__ void __launch_bounds__(640, 1)
                 for (int e = 0; e < 4; ++e) {
                     wc[h][e] = un[h][e];
                     un[h][e] = u2[h][e];
+                    u2[h][e] = u3[h][e];
                     qc[h][e] = qn[h][e];
+                    qn[h][e] = q2[h][e];
                 }
             buf ^= 1;
         }
@@ -1299,7 +1312,7 @@ cudaError_t leg_occupancy(gmg_batch b) {
     const bool sweep = !rbgs && b->cfg.nu1 >= 1;
     auto d3 = sweep ? k_down3<T, true> : k_down3<T, false>;
     auto d2 = sweep ? k_down2<T, true> : k_down2<T, false>;
-    cudaError_t e = cudaFuncSetAttribute(d3, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 640);
+    cudaError_t e = cudaFuncSetAttribute(d3, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 512);
     auto occ = [&](auto k, int threads, int smem, int& warps) {
         int n = 0;
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem);
