@@ -27,7 +27,7 @@
 // Measured at n = 512 (four half sweeps a leg): 493 us down and 374 us up, 10.5
 // bytes per node of traffic that a copy moves in 210 us.  The legs that keep
 // every plane in shared memory (legs.cuh; FP32 took them before) took 910 and
-// 824 us with 532 M and 461 M warp instructions, about 278 M here down.  What
+// 824 us with 532 M and 461 M warp instructions, 268 M and 201 M here.  What
 // bounds it: shared memory (36 16-byte accesses per thread and step) and
 // latency at 9 to 12 warps per SM, which the registers and the rings allow, and
 // a halo of S + 2 rows that is worked through twice (half of the lanes at S =
