@@ -63,10 +63,10 @@ namespace {
 // pairs of a tile meet in a bank.
 struct Plan {
     int lg, lgP, threads;
-    __host__ __device__ int n() const { return 1 << lg; }
-    __host__ __device__ int pairs() const { return 1 << lgP; }
-    __host__ __device__ int stride() const { return ((1 << lg) + ((1 << lg) >> 3)) | 1; }
-    size_t smem() const { return sizeof(double2) * (size_t)pairs() * stride(); }
+    __host__ __device__ constexpr int n() const { return 1 << lg; }
+    __host__ __device__ constexpr int pairs() const { return 1 << lgP; }
+    __host__ __device__ constexpr int stride() const { return ((1 << lg) + ((1 << lg) >> 3)) | 1; }
+    constexpr size_t smem() const { return sizeof(double2) * (size_t)pairs() * stride(); }
 };
 // total: pairs of lines of a transform.  Tiles of 256 threads (512 from n =
 // 512 up: 8 pairs of columns there are 128-byte segments along x) where there
@@ -552,13 +552,18 @@ struct gmg_fft_s {
 
 namespace {
 
-template <int THREADS>
-cudaError_t allow_smem(size_t bytes) {
-    cudaError_t e = cudaFuncSetAttribute(k_dst_x<THREADS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+// A tile of up to 256 threads holds at most 37 KB (3D n = 128), which needs no opt-in; one
+// of 512 threads up to 144 KB (2D n = 8192).  The limit belongs to the kernel,
+// not to a plan: it is one value for all of them, so that making one plan does
+// not lower it under another's launches.
+constexpr size_t kSmem512 = Plan{13, 0, 512}.smem();
+
+cudaError_t allow_smem() {
+    cudaError_t e = cudaFuncSetAttribute(k_dst_x<512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kSmem512);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_dst_y<THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)bytes);
+        e = cudaFuncSetAttribute(k_dst_y<512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kSmem512);
     return e;
 }
 
@@ -626,8 +631,7 @@ gmg_status gmg_fft_create(int d, int n, void* cuda_stream, gmg_fft* out) {
         cudaMalloc(&h->coeffs, sizeof(double) * lines * (n / 2 + 1)) != cudaSuccess ||
         cudaMalloc(&h->work, sizeof(double) * lines * n) != cudaSuccess)
         return fail(GMG_ERR_ALLOC, "cudaMalloc failed");
-    const size_t smem = h->plan.smem();
-    if ((h->plan.threads > 256 ? allow_smem<512>(smem) : allow_smem<256>(smem)) != cudaSuccess)
+    if (h->plan.threads > 256 && allow_smem() != cudaSuccess)
         return fail(GMG_ERR_CUDA, "cudaFuncSetAttribute failed");
     std::vector<double> t(4 * (size_t)n);
     for (int k = 0; k < 2 * n; ++k) {
