@@ -531,7 +531,7 @@ int tail_level(gmg_handle h, const std::vector<Level<T>>& lv) {
         if (slab_level<T>(h, lv, l)) return l;
     for (int l = lo; l + 1 < L; ++l) {
         const int n = lv[l].n;
-        if (n <= nmax && tail::smem_bytes(c.d, n, L - l, c.smoother, sizeof(T)) <= 200 * 1024)
+        if (n <= nmax && tail::smem_bytes(c.d, n, L - l, c.smoother, sizeof(T)) <= tail::kSmemLimit)
             return l;
     }
     return L;

@@ -262,6 +262,7 @@ cudaError_t up(int n, int smoother, int nu2, double omega, bool paper, const dou
 // ... (levels of them) in shared memory; u_top in/out, q_top in.
 namespace tail {
 size_t smem_bytes(int d, int n_top, int levels, int smoother, size_t elem);
+constexpr size_t kSmemLimit = 200 * 1024;  // largest smem_bytes of a launch
 // top: layout of u_top / q_top in global memory (n_top = top.n)
 // exact_top: the top level is level 0 of a plain FP64 3D hierarchy, whose
 // last pre-smoothing half sweep and residual use the unbiased value

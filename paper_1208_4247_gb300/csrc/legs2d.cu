@@ -278,9 +278,20 @@ int kind_of(int smoother) {
     return smoother == GMG_WJACOBI ? WJ : smoother == GMG_RBGS ? RB : smoother == GMG_MCGS ? MC : -1;
 }
 
+constexpr int kSteps = 6;  // smoothing steps of a leg at most (applies)
+constexpr size_t down_bytes(int tx, int ty, int S) {
+    return sizeof(double) * 3 * (tx + 3 + 2 * S) * (ty + 3 + 2 * S);
+}
+constexpr size_t up_bytes(int arrays, int tx, int ty, int S) {
+    return sizeof(double) * arrays * (tx + 2 * S) * (ty + 2 * S);
+}
+// The limit belongs to the kernel, not to the launch: the largest tile's (64 x
+// 32, tile_of) for all, so that no thread lowers it between another's limit and
+// launch.
+constexpr size_t kSmem = std::max(down_bytes(64, 32, kSteps), up_bytes(3, 64, 32, kSteps));
 template <class K>
-cudaError_t allow(K kern, size_t bytes) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+cudaError_t allow(K kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
 }
 
 }  // namespace
@@ -289,7 +300,7 @@ bool applies(int n, int nmax, int smoother, int nu1, int nu2) {
     const int k = kind_of(smoother);
     if (k < 0 || n < 32 || nu1 < 1 || nu2 < 1) return false;
     // six steps: the halo is still smaller than the small tiles
-    return steps_of(k, nu1, false) <= 6 && steps_of(k, nu2, false) <= 6 &&
+    return steps_of(k, nu1, false) <= kSteps && steps_of(k, nu2, false) <= kSteps &&
            n <= (nmax > 0 ? nmax : 512);
 }
 
@@ -306,9 +317,9 @@ cudaError_t down(int n, int smoother, int nu1, bool first_done, double omega, bo
     A.red_only = red_only;
     A.init = init;
     A.omega = omega;
-    const size_t bytes = sizeof(double) * 3 * (A.TX + 3 + 2 * A.S) * (A.TY + 3 + 2 * A.S);
+    const size_t bytes = down_bytes(A.TX, A.TY, A.S);
     auto kern = k == WJ ? k_down<WJ> : k == RB ? k_down<RB> : k_down<MC>;
-    cudaError_t e = allow(kern, bytes);
+    cudaError_t e = allow(kern);
     if (e != cudaSuccess) return e;
     kern<<<dim3((n + A.TX - 1) / A.TX, (n + A.TY - 1) / A.TY), threads_of(n), bytes, s>>>(u, uo, q, qc,
                                                                                     uc, A);
@@ -325,9 +336,9 @@ cudaError_t up(int n, int smoother, int nu2, double omega, bool paper, const dou
     A.paper = paper;
     A.black = k == RB;
     A.omega = omega;
-    const size_t bytes = sizeof(double) * (k == WJ ? 3 : 2) * (A.TX + 2 * A.S) * (A.TY + 2 * A.S);
+    const size_t bytes = up_bytes(k == WJ ? 3 : 2, A.TX, A.TY, A.S);
     auto kern = k == WJ ? k_up<WJ> : k == RB ? k_up<RB> : k_up<MC>;
-    cudaError_t e = allow(kern, bytes);
+    cudaError_t e = allow(kern);
     if (e != cudaSuccess) return e;
     kern<<<dim3((n + A.TX - 1) / A.TX, (n + A.TY - 1) / A.TY), threads_of(n), bytes, s>>>(uc, u, uo, q,
                                                                                     A);

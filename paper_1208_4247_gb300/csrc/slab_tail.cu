@@ -321,16 +321,23 @@ bool slab_applies(int d, int n, int levels, int smoother, bool paper, bool fp64)
            (smoother == GMG_RBGS || smoother == GMG_LEARNED) && !paper;
 }
 
+// bytes of a launch whose top level has n intervals
+template <typename T>
+constexpr size_t slab_bytes(int n) {
+    return sizeof(T) * (slab_elems(n) + (n == 32 ? slab_elems(16) : 0) + 3 * kSmallNodes + 2 * 81);
+}
+
 template <typename T>
 cudaError_t launch_slab(const Lay& top, int levels, T* u_top, const T* q_top, int smoother,
                         int nu1, int nu2, int coarse_sweeps, cudaStream_t s, bool exact_top,
                         bool first_done) {
-    const size_t bytes = sizeof(T) * (slab_elems(top.n) + (top.n == 32 ? slab_elems(16) : 0) +
-                                      3 * kSmallNodes + 2 * 81);
+    const size_t bytes = slab_bytes<T>(top.n);
     const Cycle cy{smoother, nu1, nu2, coarse_sweeps, false, 0.0};
     auto kern = k_slab_tail<T>;
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    // the limit belongs to the kernel: the larger launch's for both, so that no
+    // thread lowers it between another's limit and launch
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)slab_bytes<T>(32));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;

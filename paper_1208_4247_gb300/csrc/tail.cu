@@ -218,9 +218,12 @@ cudaError_t launch(int d, const Lay& top, int levels, T* u_top, const T* q_top, 
     const int64_t nodes = d == 3 ? (int64_t)top.n * top.n * top.n : (int64_t)top.n * top.n;
     const int64_t slots = smoother == GMG_WJACOBI ? nodes : nodes / 2;
     const int threads = (int)std::min<int64_t>(1024, std::max<int64_t>(128, slots));
+    if (bytes > kSmemLimit) return cudaErrorInvalidValue;
     auto kern = d == 3 ? k_tail<3, T> : k_tail<2, T>;
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    // the limit belongs to the kernel: one value whatever the launch takes, so
+    // that no thread lowers it between another's limit and launch
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kSmemLimit);
     if (e != cudaSuccess) return e;
     kern<<<1, threads, bytes, s>>>(u_top, q_top, top, levels, cy, exact0,
                                   first_done ? 1 : 0);

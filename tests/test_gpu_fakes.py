@@ -1,0 +1,40 @@
+"""What the library does where a CUDA call answers in a way that no argument
+brings about (tests/cuda_fakes.cpp), each script in a process of its own."""
+import pytest
+
+import fakes
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return fakes.link(str(tmp_path_factory.mktemp("fakes") / "libgmg_fakes.so"))
+
+
+def test_shared_memory_limits_do_not_depend_on_the_size(lib):
+    """A kernel's shared-memory limit is one value for the process, so handles of
+    different sizes on different threads cannot lower it under one another's
+    launches."""
+    out = fakes.run(lib, """
+for d, n, kw in [(2, 512, {}), (2, 64, {}), (2, 32, dict(smoother="mcgs")), (2, 256, dict(smoother="wjacobi")),
+                 (2, 8, dict(smoother="wjacobi")), (3, 16, {}), (3, 32, {}), (3, 64, dict(precision="df")),
+                 (3, 16, dict(precision="df")), (3, 32, dict(precision="fp32")), (3, 16, dict(precision="fp32")),
+                 (3, 8, dict(precision="bf16")), (3, 32, dict(precision="bf16")), (3, 8, dict(smoother="wjacobi")),
+                 (3, 4, dict(smoother="wjacobi")), (3, 128, dict(precision="fp32"))]:
+    f = torch.from_numpy(inputs.rhs_uniform(d, n, 5)).cuda()
+    with gmg.Solver(d, n, **kw) as S:
+        S.cycles(f, torch.zeros_like(f), 1)
+for d, n in [(3, 128), (3, 16), (2, 512), (2, 1024)]:
+    f = torch.from_numpy(inputs.rhs_uniform(d, n, 5)).cuda()
+    with gmg.FFTSolver(d, n) as F:
+        F.solve(f, torch.zeros_like(f))
+for k in (1, 2):
+    with gmg.Batch([3, 2], [16 * k, 64 * k]) as B:
+        pass
+print(fake.fake_attribute_changes())
+""")
+    assert out == ["0"]
