@@ -117,8 +117,8 @@ gmg_status gmg_config_init(gmg_config* cfg, int d, int n);
  * bit for bit; slower on GB300, see the design notes).  GMG_TAIL_N=m sets the
  * largest level n handled by the single-CTA tail launch (1 turns the tail
  * off; default 32 in 2D and 8 in 3D, where red-black handles run the levels
- * from n = 32, FP64 16, down as one 16-CTA cluster instead); results are the
- * same bit for bit.
+ * from n = 32, FP64 16, down as one 16-CTA cluster instead if the device has
+ * room for one, asked at create); results are the same bit for bit.
  * GMG_RB_WALK=0 (read once per process) replaces the diagonal-walker FP64 3D
  * half sweeps, red-only residuals and norms (levels 128 <= n <= 512) by row
  * kernels; results are the same bit for bit.  GMG_NORM_AHEAD=0 (read once

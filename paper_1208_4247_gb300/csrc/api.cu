@@ -117,6 +117,8 @@ struct gmg_handle_s {
     // cycle's first level-0 red half sweep (norm_ahead_ok)
     bool ahead = false;
     int tail_max = 0;       // GMG_TAIL_N at create: largest tail level n (0 = default)
+    // the device places the cycles' cluster tail from n = 16, from n = 32 down
+    bool slab16 = false, slab32 = false;
     // fused leg kernels (legs_reg.cu, legs.cu) on large 3D levels of the
     // red-black inner hierarchies.  legs_mode 1 (default): FP32 levels with n
     // >= 256, where they beat the unfused kernels; 2 (GMG_FUSED_LEGS=1 at
@@ -507,13 +509,14 @@ bool leg2d_level(gmg_handle h, const std::vector<Level<T>>& lv, int l) {
 // fit in 200 KB of shared memory, below every learned level, leaving at
 // least two tail levels.
 // Red-black 3D handles start it at 33^3 or 17^3 (as the cluster of
-// slab_tail.cu) where the hierarchy has such a level and no threshold is given.
+// slab_tail.cu) where the hierarchy has such a level, no threshold is given and
+// the device has room for the cluster.
 template <typename T>
 bool slab_level(gmg_handle h, const std::vector<Level<T>>& lv, int l) {
     const gmg_config& c = h->cfg;
-    return h->tail_max == 0 && tail::slab_applies(c.d, lv[l].n, (int)lv.size() - l, c.smoother,
-                                                  c.transfer == GMG_TRANSFER_PAPER,
-                                                  std::is_same<T, double>::value);
+    return h->tail_max == 0 && (lv[l].n == 32 ? h->slab32 : h->slab16) &&
+           tail::slab_applies(c.d, lv[l].n, (int)lv.size() - l, c.smoother,
+                              c.transfer == GMG_TRANSFER_PAPER, std::is_same<T, double>::value);
 }
 template <typename T>
 int tail_level(gmg_handle h, const std::vector<Level<T>>& lv) {
@@ -1672,6 +1675,16 @@ gmg_status gmg_create(const gmg_config* cfg, void* cuda_stream, gmg_handle* out)
         if (h->gtail_blocks > 0 &&
             (st = dev_alloc(h, (char**)&h->gtail_bar, (int64_t)tail::grid_bar_bytes())) != GMG_OK)
             return fail(st);
+    }
+    if (d == 3 && cfg->n >= 16 && (cfg->smoother == GMG_RBGS || cfg->smoother == GMG_LEARNED)) {
+        auto fits = [&](int n) {
+            return cfg->precision == GMG_FP64      ? tail::slab_fits<double>(n)
+                   : cfg->precision == GMG_FP32_IR ? tail::slab_fits<float>(n)
+                   : cfg->precision == GMG_DF_IR   ? tail::slab_fits<df32>(n)
+                                                   : tail::slab_fits<bf16>(n);
+        };
+        h->slab16 = fits(16);
+        h->slab32 = cfg->precision != GMG_FP64 && cfg->n >= 32 && fits(32);
     }
     if (cfg->precision == GMG_FP64) {
         if ((st = alloc_hierarchy<double>(h, h->lv, L, false)) != GMG_OK) return fail(st);

@@ -278,6 +278,10 @@ cudaError_t launch(int d, const Lay& top, int levels, T* u_top, const T* q_top, 
 // (slab_tail.cu): red-black smoothing, full weighting, a hierarchy that
 // reaches 9^3.  first_done: as launch's.
 bool slab_applies(int d, int n, int levels, int smoother, bool paper, bool fp64);
+// Whether the current device can place that cluster from n intervals down;
+// where it cannot, the single-CTA tail runs (launch).
+template <typename T>
+bool slab_fits(int n);
 template <typename T>
 cudaError_t launch_slab(const Lay& top, int levels, T* u_top, const T* q_top, int smoother,
                         int nu1, int nu2, int coarse_sweeps, cudaStream_t s, bool exact_top,

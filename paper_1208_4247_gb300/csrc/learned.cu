@@ -489,6 +489,7 @@ struct Trainer {
     // NULL), then made
     char* base = nullptr;
     size_t used = 0;
+    bool slab16 = false;  // the device places the cluster tail from n = 16 down
 
     cudaError_t alloc(void** p, size_t bytes) {
         *p = base ? base + used : nullptr;
@@ -535,6 +536,7 @@ struct Trainer {
         pair_cycles = pc;
         s = st;
         nodes = nodes_of(d, n);
+        slab16 = d == 3 && n >= 16 && tail::slab_fits<double>(16);
         deal(extra);
         const size_t total = used;
         cudaError_t e = cudaMalloc((void**)&base, total);
@@ -550,6 +552,10 @@ struct Trainer {
         return d == 2 && l + 1 < (int)lv.size() &&
                legs2d::applies(lv[l].n, 0, GMG_RBGS, 1, 1);
     }
+    // the cluster tail takes level l of a hierarchy of L
+    bool slab_level(const std::vector<Level<double>>& lv, int l) const {
+        return slab16 && tail::slab_applies(d, lv[l].n, (int)lv.size() - l, GMG_RBGS, false, true);
+    }
     // RB-GS V(nu,nu) cycle on hierarchy lv (level-0 iterate lv[0].u[0], rhs
     // lv[0].q) with the solver's kernels: grid kernels (2D: legs) and the
     // cluster or single-CTA tail.  first_done: the first red half sweep ran.
@@ -557,7 +563,7 @@ struct Trainer {
         const int L = (int)lv.size();
         int lt = L;
         for (int l = 0; l < L && lt == L; ++l)
-            if (nu > 0 && (tail::slab_applies(d, lv[l].n, L - l, GMG_RBGS, false, true) ||
+            if (nu > 0 && (slab_level(lv, l) ||
                            (lv[l].n <= (d == 3 ? 8 : 16) && L - l >= 2)))
                 lt = l;
         std::vector<char> done(L + 1, 0);
@@ -579,7 +585,7 @@ struct Trainer {
         if (lt < L) {
             Level<double>& t = lv[lt];
             const Lay lay = dense_lay(d, t.n);
-            if (tail::slab_applies(d, t.n, L - lt, GMG_RBGS, false, true))
+            if (slab_level(lv, lt))
                 tail::launch_slab<double>(lay, L - lt, t.u[0], t.q, GMG_RBGS, nu, nu, 0, s, false,
                                           done[lt]);
             else

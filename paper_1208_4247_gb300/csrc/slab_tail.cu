@@ -327,38 +327,64 @@ constexpr size_t slab_bytes(int n) {
     return sizeof(T) * (slab_elems(n) + (n == 32 ? slab_elems(16) : 0) + 3 * kSmallNodes + 2 * 81);
 }
 
+// The launch of a cluster over a top level of n intervals: its attribute is at
+// `at`, and the kernel's limits are set.  They belong to the kernel: the larger
+// launch's for both sizes, so that no thread lowers them between another's limit
+// and launch.
 template <typename T>
-cudaError_t launch_slab(const Lay& top, int levels, T* u_top, const T* q_top, int smoother,
-                        int nu1, int nu2, int coarse_sweeps, cudaStream_t s, bool exact_top,
-                        bool first_done) {
-    const size_t bytes = slab_bytes<T>(top.n);
-    const Cycle cy{smoother, nu1, nu2, coarse_sweeps, false, 0.0};
+cudaError_t slab_config(int n, cudaStream_t s, cudaLaunchAttribute* at, cudaLaunchConfig_t* cfg) {
     auto kern = k_slab_tail<T>;
-    // the limit belongs to the kernel: the larger launch's for both, so that no
-    // thread lowers it between another's limit and launch
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)slab_bytes<T>(32));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(kRanks);
-    cfg.blockDim = dim3(kSlabThreads);
-    cfg.dynamicSmemBytes = bytes;
-    cfg.stream = s;
+    *cfg = cudaLaunchConfig_t{};
+    cfg->gridDim = dim3(kRanks);
+    cfg->blockDim = dim3(kSlabThreads);
+    cfg->dynamicSmemBytes = slab_bytes<T>(n);
+    cfg->stream = s;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = kRanks;
+    at->val.clusterDim.y = 1;
+    at->val.clusterDim.z = 1;
+    cfg->attrs = at;
+    cfg->numAttrs = 1;
+    return e;
+}
+
+// 16 CTAs are more than the portable 8: whether the current device has a place
+// for them (16 free SMs in one GPC, or in a part of the device) is its answer.
+template <typename T>
+bool slab_fits(int n) {
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kRanks;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cudaLaunchConfig_t cfg;
+    int clusters = 0;
+    cudaError_t e = slab_config<T>(n, nullptr, at, &cfg);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, k_slab_tail<T>, &cfg);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return clusters > 0;
+}
+
+template <typename T>
+cudaError_t launch_slab(const Lay& top, int levels, T* u_top, const T* q_top, int smoother,
+                        int nu1, int nu2, int coarse_sweeps, cudaStream_t s, bool exact_top,
+                        bool first_done) {
+    const Cycle cy{smoother, nu1, nu2, coarse_sweeps, false, 0.0};
+    cudaLaunchAttribute at[1];
+    cudaLaunchConfig_t cfg;
+    cudaError_t e = slab_config<T>(top.n, s, at, &cfg);
+    if (e != cudaSuccess) return e;
     const int ex = exact_top && std::is_same<T, double>::value ? 1 : 0;
-    e = cudaLaunchKernelEx(&cfg, kern, u_top, q_top, top, levels, cy, ex, first_done ? 1 : 0);
+    e = cudaLaunchKernelEx(&cfg, k_slab_tail<T>, u_top, q_top, top, levels, cy, ex,
+                           first_done ? 1 : 0);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 #define GMG_SLAB_INST(T)                                                                     \
+    template bool slab_fits<T>(int);                                                         \
     template cudaError_t launch_slab<T>(const Lay&, int, T*, const T*, int, int, int, int,   \
                                         cudaStream_t, bool, bool);
 GMG_SLAB_INST(double)

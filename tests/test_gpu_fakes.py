@@ -38,3 +38,24 @@ for k in (1, 2):
 print(fake.fake_attribute_changes())
 """)
     assert out == ["0"]
+
+
+def test_no_room_for_a_cluster(lib):
+    """Where the device cannot place a cluster of 16 CTAs the small levels run in
+    the single-CTA tail: every form solves, with the same bits."""
+    out = fakes.run(lib, """
+for kw in (dict(), dict(precision="df"), dict(precision="fp32"), dict(precision="bf16"),
+           dict(smoother="learned")):
+    f = torch.from_numpy(inputs.rhs_uniform(3, 64, 6)).cuda()
+    got = []
+    for limit in (16, 8):
+        fake.fake_cluster_limit(limit)
+        u = torch.zeros_like(f)
+        with gmg.Solver(3, 64, **kw) as S:
+            S.set_timing(True)
+            S.cycles(f, u, 2)
+            tails = sorted((r["kernel"], r["level"]) for r in S.timing_report()[0] if "tail" in r["kernel"])
+        got.append((u, tails))
+    print(torch.equal(got[0][0], got[1][0]), got[0][1] != got[1][1])
+""")
+    assert out == ["True True"] * 5
