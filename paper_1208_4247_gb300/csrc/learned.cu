@@ -490,6 +490,18 @@ struct Trainer {
     char* base = nullptr;
     size_t used = 0;
     bool slab16 = false;  // the device places the cluster tail from n = 16 down
+    // first error of a launch: the legs and tails opt in to shared memory and
+    // clusters, and report (and clear) their own errors
+    cudaError_t err = cudaSuccess;
+
+    void note(cudaError_t e) {
+        if (err == cudaSuccess) err = e;
+    }
+    // that error, or the one a plain launch left
+    cudaError_t status() {
+        note(cudaGetLastError());
+        return err;
+    }
 
     cudaError_t alloc(void** p, size_t bytes) {
         *p = base ? base + used : nullptr;
@@ -536,6 +548,7 @@ struct Trainer {
         pair_cycles = pc;
         s = st;
         nodes = nodes_of(d, n);
+        cudaGetLastError();  // an error that some other call left is not this one's
         slab16 = d == 3 && n >= 16 && tail::slab_fits<double>(16);
         deal(extra);
         const size_t total = used;
@@ -574,8 +587,8 @@ struct Trainer {
             const int init = C.n == 2 ? INIT_EXACT : nu > 0 ? INIT_RED : INIT_ZERO;
             done[l + 1] = init == INIT_RED;
             if (leg_level(lv, l) && F.u[1]) {
-                legs2d::down(F.n, GMG_RBGS, nu, done[l], 0.0, false, true, init, F.u[0], F.u[1], F.q,
-                             C.q, C.u[0], s);
+                note(legs2d::down(F.n, GMG_RBGS, nu, done[l], 0.0, false, true, init, F.u[0], F.u[1],
+                                  F.q, C.q, C.u[0], s));
                 continue;
             }
             half_sweeps(F, nu, done[l]);
@@ -586,18 +599,18 @@ struct Trainer {
             Level<double>& t = lv[lt];
             const Lay lay = dense_lay(d, t.n);
             if (slab_level(lv, lt))
-                tail::launch_slab<double>(lay, L - lt, t.u[0], t.q, GMG_RBGS, nu, nu, 0, s, false,
-                                          done[lt]);
+                note(tail::launch_slab<double>(lay, L - lt, t.u[0], t.q, GMG_RBGS, nu, nu, 0, s, false,
+                                               done[lt]));
             else
-                tail::launch<double>(d, lay, L - lt, t.u[0], t.q, GMG_RBGS, 0.8, nu, nu, 0, s, false,
-                                     false, done[lt]);
+                note(tail::launch<double>(d, lay, L - lt, t.u[0], t.q, GMG_RBGS, 0.8, nu, nu, 0, s,
+                                          false, false, done[lt]));
         } else if (L == 1) {
             half_sweeps(lv[0], nu, first_done);
         }
         for (int l = down - 1; l >= 0; --l) {
             Level<double>&F = lv[l], &C = lv[l + 1];
             if (leg_level(lv, l) && F.u[1]) {
-                legs2d::up(F.n, GMG_RBGS, nu, 0.0, false, C.u[0], F.u[1], F.u[0], F.q, s);
+                note(legs2d::up(F.n, GMG_RBGS, nu, 0.0, false, C.u[0], F.u[1], F.u[0], F.q, s));
                 continue;
             }
             lk::prolong_add<double>(d, C.n, C.u[0], F.u[0], s, nu > 0);
@@ -780,6 +793,7 @@ gmg_status gmg_learned_loss_grad(int d, int n, const float* weights, const doubl
     GMG_TRY_CUDA_RELEASE(cudaMemcpyAsync(tr.scal + 2, &one, sizeof(double), cudaMemcpyHostToDevice, s),
                          tr);
     tr.loss_grad(wd + W, 1.0, grad_out != nullptr);
+    GMG_TRY_CUDA_RELEASE(tr.status(), tr);
     double sc[2];
     GMG_TRY_CUDA_RELEASE(cudaMemcpyAsync(sc, tr.scal, sizeof(double) * 2, cudaMemcpyDeviceToHost, s),
                          tr);
@@ -829,6 +843,7 @@ gmg_status gmg_learned_train(int d, int n, int steps, int batch, int pair_cycles
             tr.loss_grad(work, (double)batch, true);
         }
         k_adam<<<(W + 255) / 256, 256, 0, s>>>(master, work, tr.grad, m1, m2, W, it + 1, lr);
+        GMG_TRY_CUDA_RELEASE(tr.status(), tr);
         if (loss_history) {
             GMG_TRY_CUDA_RELEASE(cudaMemcpyAsync(&loss_history[it], tr.scal + 1, sizeof(double),
                                                  cudaMemcpyDeviceToHost, s),

@@ -59,3 +59,24 @@ for kw in (dict(), dict(precision="df"), dict(precision="fp32"), dict(precision=
     print(torch.equal(got[0][0], got[1][0]), got[0][1] != got[1][1])
 """)
     assert out == ["True True"] * 5
+
+
+def test_training_reports_a_failed_launch(lib):
+    """A launch that fails inside the coarse solves of a loss, a gradient or a
+    training run comes back as an error, not as a number; the next call works."""
+    out = fakes.run(lib, """
+w = np.random.default_rng(0).normal(0, 0.01, (2, 8, 27)).astype(np.float32)
+e = torch.from_numpy(inputs.rhs_uniform(3, 64, 7)).cuda()
+print("ok", gmg.learned_loss_grad(w, e, 8)[0] > 0.0)
+fake.fake_cluster_fails(1)
+for call in (lambda: gmg.learned_loss_grad(w, e, 8),
+             lambda: gmg.learned_train(3, 64, 2, 1, w, coarse_cycles=8)):
+    try:
+        call()
+        print("returned")
+    except gmg.GMGError as ex:
+        print(gmg.STATUS[ex.status])
+fake.fake_cluster_fails(0)
+print("ok", gmg.learned_loss_grad(w, e, 8)[0] > 0.0)
+""")
+    assert out == ["ok True", "ERR_CUDA", "ERR_CUDA", "ok True"]
