@@ -274,6 +274,23 @@ __host__ __device__ __forceinline__ df32 sixth(df32 s) {
     const float t = rn::fma(kSixth0, s.lo, rn::fma(kSixth1, s.hi, rn::mul(kSixth2, s.hi)));
     return fast_two_sum(p, rn::add(pe, t));
 }
+// (float)(x / 6), to 2^-47 before the rounding to 24 bits.  Outside [2^-74,
+// 2^127) the parts of x or the product error could overflow or be subnormal
+// although the quotient is a float: divided 2^64 times as large or as small
+// (exact).  From 2^137 on the quotient is infinite as a float, as the cast of x
+// is; NaN stays NaN, zero keeps its sign.
+__host__ __device__ __forceinline__ float narrow_sixth(double x) {
+    const uint64_t b = cvt::d_bits(x);
+    const uint32_t ex = (uint32_t)(b >> 52) & 0x7ffu;
+    if (ex - 949u > 1149u - 949u) {
+        if ((b << 1) == 0) return cvt::bits_f((uint32_t)(b >> 32));
+        if (ex >= 1160u) return (float)x;
+        const bool small = ex < 949u;
+        const float v = sixth(df32(x * (small ? 0x1p64 : 0x1p-64))).hi;
+        return rn::mul(v, small ? 0x1p-64f : 0x1p64f);
+    }
+    return sixth(df32(x)).hi;
+}
 // s / 4, exact
 __host__ __device__ __forceinline__ df32 quarter(df32 s) {
     return df32(rn::mul(0.25f, s.hi), rn::mul(0.25f, s.lo));

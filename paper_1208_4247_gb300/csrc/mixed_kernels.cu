@@ -59,8 +59,8 @@ __device__ inline void store_value(T* __restrict__ q_in, T* __restrict__ e_init,
 // FP32 and BF16 storage in 3D: 6 sigma = 6 q + (sum - 6 u) in two fused
 // multiply-adds (the inner one cancels u with one rounding), instead of two for the
 // unbiased 1/6 and a subtraction; the division by 6 and the rounding to T go to
-// the integer and FP32 pipes (cvt::split, sixth: 2^-47 before the one rounding
-// to 24 bits).  Other types of FP32 arithmetic: rounded on the integer pipe,
+// the integer and FP32 pipes (narrow_sixth: 2^-47 before the one rounding to 24
+// bits).  Other types of FP32 arithmetic: rounded on the integer pipe,
 // because the cast takes a slot of the FP64 pipe, which bounds the kernel.  257^3, BF16:
 // 307 us with the cast and the subtraction, 281 without the cast, 248 in this form; 513^3, FP32: 2334, 2297, 1865 us.
 template <int DIM, typename T>
@@ -82,7 +82,7 @@ struct Sigma {
                                                  int64_t idx, double sig, bool red,
                                                  float* __restrict__ resid) {
         if constexpr (kSix) {
-            store_value(q_in, e_init, idx, N::st(sixth(df32(sig)).hi), red);
+            store_value(q_in, e_init, idx, N::st(dw::narrow_sixth(sig)), red);
         } else if constexpr (kF) {
             store_value(q_in, e_init, idx, N::st(cvt::narrow(sig)), red);
         } else {
