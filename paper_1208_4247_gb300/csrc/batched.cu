@@ -33,10 +33,10 @@ using lk::fastdiv_make;
 
 struct BLevel {
     int d, n;
-    int64_t u0, u1, q, r;  // element offsets into the inner pool (-1: none)
-    int64_t sy, sz;        // inner pool row / plane pitch
-    int lgG;               // log2 of the 16-byte groups per row the vector kernels take
-    FastDiv rows;          // division by n - 1 (interior nodes per row)
+    int64_t u0, u1, q;  // element offsets into the inner pool (-1: none)
+    int64_t sy, sz;     // inner pool row / plane pitch
+    int lgG;            // log2 of the 16-byte groups per row the vector kernels take
+    FastDiv rows;       // division by n - 1 (interior nodes per row)
 };
 struct BSolve {
     int d, n, levels, lev0;  // lev0: index of level 0 in the level table
@@ -1413,7 +1413,7 @@ gmg_status gmg_batch_create(int count, const int* d, const int* n, const gmg_con
         cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming) != cudaSuccess)
         return fail(GMG_ERR_CUDA, "stream/event creation failed");
-    // layout: per solve, per level: u0 [u1] q [r] in the inner pool (256-byte
+    // layout: per solve, per level: u0 [u1] q in the inner pool (256-byte
     // aligned regions); FP64 q64 per solve
     const int64_t align = 256 / b->elem;
     auto up = [&](int64_t v, int64_t a) { return (v + a - 1) / a * a; };
@@ -1452,11 +1452,6 @@ gmg_status gmg_batch_create(int count, const int* d, const int* n, const gmg_con
             }
             lv.q = poff;
             poff = up(poff + nodes, align);
-            lv.r = -1;
-            if (l + 1 < L) {
-                lv.r = poff;
-                poff = up(poff + nodes, align);
-            }
             b->hl.push_back(lv);
         }
         b->G = std::max(b->G, L - 1);
