@@ -67,13 +67,17 @@ inline int leg_rows(int n, int threads) { return 2 * (threads / std::min(n / 4, 
 inline int leg_pieces(int64_t columns, int64_t slots, int len, int unit, int extra) {
     int best = 1;
     int64_t cost = INT64_MAX;
-    for (int p = 1; p <= len; ++p) {
+    // of the counts that give pieces of seg steps only the least can win
+    for (int p = 1; p <= len;) {
+        const int seg = (len + p - 1) / p;
         const int64_t waves = (columns * p + slots - 1) / slots;
-        const int64_t c = waves * ((int64_t)unit * ((len + p - 1) / p) + extra);
+        const int64_t c = waves * ((int64_t)unit * seg + extra);
         if (c < cost) {
             best = p;
             cost = c;
         }
+        if (seg == 1) break;
+        p = (len + seg - 2) / (seg - 1);
     }
     return best;
 }

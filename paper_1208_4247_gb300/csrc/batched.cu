@@ -1125,7 +1125,7 @@ gmg_status enqueue_cycles(gmg_batch b, int d, cudaStream_t st) {
     const bool sweep_down = !rbgs && c.nu1 >= 1, sweep_up = !rbgs && c.nu2 >= 1;
     int G = 0;
     for (int g = 1; g <= b->G; ++g)
-        if (steps[g].fine.count) G = g;
+        if (steps[g].down.count) G = g;
     std::vector<int> cur(G + 1, 0);  // which u buffer holds each level step's iterate
     auto relax = [&](int g, int sweeps, int zero) {
         const Range& r = steps[g].fine;
@@ -1337,7 +1337,7 @@ gmg_status gmg_batch_destroy(gmg_batch b) {
     if (b->stream) cudaStreamSynchronize(b->stream);
     if (b->graph) cudaGraphExecDestroy(b->graph);
     b->timer.destroy();
-    for (void* p : {(void*)b->ds, (void*)b->dl, (void*)b->di, (void*)b->dt, b->pool, (void*)b->pool64,
+    for (void* p : {(void*)b->ds, (void*)b->dl, (void*)b->di, b->pool, (void*)b->pool64,
                     (void*)b->partial, (void*)b->res0_2, (void*)b->relres, (void*)b->active,
                     (void*)b->iters, (void*)b->num_active})
         if (p) cudaFree(p);
@@ -1477,75 +1477,90 @@ gmg_status gmg_batch_create(int count, const int* d, const int* n, const gmg_con
     const bool rbgs = common->smoother == GMG_RBGS;
     const cudaError_t oe = b->elem == 4 ? leg_occupancy<float>(b) : leg_occupancy<__nv_bfloat16>(b);
     if (oe != cudaSuccess) return fail(GMG_ERR_CUDA, cudaGetErrorString(oe));
+    // sweeps that no leg takes (relax)
+    const bool plain = rbgs || common->nu1 > 1 || common->nu2 > 1;
+    struct Leg {  // the tiles of a step: a solve's side by side
+        Range* r;
+        int dim, g, len, np;
+        std::vector<Rows> rows;
+        std::vector<int> cols;
+    };
+    std::vector<Leg> legs;
+    std::vector<std::vector<int>> members(2 * (b->G + 1));
+    size_t ntiles = 0;
     for (int dim = 2; dim <= 3; ++dim) {
         b->steps[dim - 2].resize(b->G + 1);
         for (int g = 1; g <= b->G; ++g) {
             Step& S = b->steps[dim - 2][g];
             const int n_g = 2 << g, nc = n_g / 2;  // the same size for every solve
-            std::vector<int> members;
+            std::vector<int>& mem = members[2 * g + dim - 2];
             for (int s = 0; s < count; ++s)
-                if (b->hs[s].d == dim && b->hs[s].levels - 1 >= g) members.push_back(s);
-            if (members.empty()) continue;
+                if (b->hs[s].d == dim && b->hs[s].levels - 1 >= g) mem.push_back(s);
+            if (mem.empty()) continue;
             b->has_d[dim - 2] = true;
             auto level_of = [&](int s) { return b->hs[s].levels - 1 - g; };
-            // plain sweeps: (interior row, 16-byte group) pairs, chunk / V groups per item
+            // (interior row, 16-byte group) pairs, chunk / V groups per item
             S.fine.off = (int)b->items.size();
             const int V = 16 / b->elem;
-            for (int s : members) {
+            for (int s : mem) {
                 const int l = level_of(s);
                 const int64_t groups = (int64_t)(dim == 3 ? (n_g - 1) * (n_g - 1) : n_g - 1)
                                        << b->hl[b->hs[s].lev0 + l].lgG;
                 const int64_t gchunk = std::max<int64_t>(1, b->chunk / V);
-                for (int64_t st = 0; st < groups; st += gchunk)
+                for (int64_t st = 0; plain && st < groups; st += gchunk)
                     b->items.push_back({s, l, st, (int)std::min<int64_t>(gchunk, groups - st)});
                 S.fine.nodes += groups * V;
             }
             S.fine.count = (int)b->items.size() - S.fine.off;
             if (rbgs || common->nu2 == 0) {
                 S.cells.off = (int)b->items.size();
-                for (int s : members) {
+                for (int s : mem) {
                     add_items(s, level_of(s), pw(nc, dim), b->items);
                     S.cells.nodes += pw(nc, dim);
                 }
                 S.cells.count = (int)b->items.size() - S.cells.off;
             }
-            // legs' tiles, a solve's side by side
             S.lanes = std::min(n_g / 4, 32);
-            const std::vector<int> cols = leg_columns(n_g / 4, kHaloLanes);
-            const int64_t nm = (int64_t)members.size();
             for (int down = 0; down < 2; ++down) {
                 if (!down && (rbgs || common->nu2 == 0)) continue;
-                Range& r = down ? S.down : S.up;
-                r.off = (int)b->tiles.size();
+                Leg L{down ? &S.down : &S.up, dim, g, 0, 0, {Rows{0, 0, 0}},
+                      leg_columns(n_g / 4, kHaloLanes)};
                 // walk: coarse planes 1..nc-1 down (2 fine planes each), fine planes 1..n-1 up
-                const int len = down ? nc - 1 : n_g - 1, unit = down ? 2 : 1, extra = down ? 4 : 2;
+                L.len = down ? nc - 1 : n_g - 1;
+                const int unit = down ? 2 : 1, extra = down ? 4 : 2;
                 int& th = down ? S.down_threads : S.up_threads;
-                std::vector<Rows> rows(1, Rows{0, 0, 0});
                 int64_t slots;
                 if (dim == 3) {
                     th = leg_threads(n_g, down);
                     const int R = leg_rows(n_g, th);
-                    rows = down ? rows_down(n_g, R) : rows_up(n_g, R);
+                    L.rows = down ? rows_down(n_g, R) : rows_up(n_g, R);
                     slots = (int64_t)b->sms * std::max(1, b->leg_warps[2 + down] / (th / 32));
                 } else {
                     slots = (int64_t)b->sms * b->leg_warps[down] * (32 / S.lanes);
                 }
-                const int np = leg_pieces(nm * (int64_t)(rows.size() * cols.size()), slots, len,
-                                          unit, extra);
-                for (int s : members)
-                    for (int pc = 0; pc < np; ++pc) {
-                        const int a = 1 + (int)((int64_t)len * pc / np),
-                                  e = 1 + (int)((int64_t)len * (pc + 1) / np);
-                        for (const Rows& rw : rows)
-                            for (int g0 : cols)
-                                b->tiles.push_back(dim == 3 ? Tile{s, level_of(s), g0, rw.y0, rw.ja,
-                                                                   rw.jb, a, e}
-                                                            : Tile{s, level_of(s), g0, 0, a, e, 0,
-                                                                   0});
-                    }
-                r.count = (int)b->tiles.size() - r.off;
-                r.nodes = nm * pw(n_g - 1, dim);
+                const int64_t columns = (int64_t)(mem.size() * L.rows.size() * L.cols.size());
+                L.np = leg_pieces(columns, slots, L.len, unit, extra);
+                L.r->off = (int)ntiles;
+                L.r->count = (int)(columns * L.np);
+                L.r->nodes = (int64_t)mem.size() * pw(n_g - 1, dim);
+                ntiles += L.r->count;
+                legs.push_back(std::move(L));
             }
+        }
+    }
+    b->tiles.reserve(ntiles);  // (grown step by step they took longer than all else here)
+    std::vector<int> cut;
+    for (const Leg& L : legs) {
+        cut.resize(L.np + 1);
+        for (int pc = 0; pc <= L.np; ++pc) cut[pc] = 1 + (int)((int64_t)L.len * pc / L.np);
+        for (int s : members[2 * L.g + L.dim - 2]) {
+            const int level = b->hs[s].levels - 1 - L.g;
+            for (int pc = 0; pc < L.np; ++pc)
+                for (const Rows& rw : L.rows)
+                    for (int g0 : L.cols)
+                        b->tiles.push_back(
+                            L.dim == 3 ? Tile{s, level, g0, rw.y0, rw.ja, rw.jb, cut[pc], cut[pc + 1]}
+                                       : Tile{s, level, g0, 0, cut[pc], cut[pc + 1], 0, 0});
         }
     }
     cudaError_t e = cudaSuccess;
@@ -1556,8 +1571,10 @@ gmg_status gmg_batch_create(int count, const int* d, const int* n, const gmg_con
     al((void**)&b->ds, sizeof(BSolve) * count);
     al((void**)&b->dl, sizeof(BLevel) * b->hl.size());
     al((void**)&b->di, sizeof(Item) * b->items.size());
-    al((void**)&b->dt, sizeof(Tile) * b->tiles.size());
-    al(&b->pool, (size_t)b->elem * poff);
+    // the tiles behind the pool (an allocation of their own took 45 us)
+    const size_t pool_bytes = ((size_t)b->elem * poff + 255) / 256 * 256;
+    al(&b->pool, pool_bytes + sizeof(Tile) * b->tiles.size());
+    b->dt = reinterpret_cast<Tile*>(static_cast<char*>(b->pool) + pool_bytes);
     al((void**)&b->pool64, sizeof(double) * off64);
     al((void**)&b->partial, sizeof(double) * b->level0.count);
     al((void**)&b->res0_2, sizeof(double) * count);

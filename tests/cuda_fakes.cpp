@@ -3,6 +3,7 @@
 //
 //   fake_attribute_changes()  how often a kernel's shared-memory limit was set to
 //                             another value than before
+//   fake_copied_bytes()       bytes copied from host memory so far
 //   fake_cluster_limit(c)     the device has no room for clusters of more than c
 //                             CTAs: the query answers 0, a launch fails
 //   fake_cluster_fails(on)    the launch of a cluster fails
@@ -14,6 +15,7 @@
 namespace {
 std::mutex lock;
 std::map<const void*, int> limit;
+size_t copied = 0;
 int changes = 0, cluster_limit = 1 << 30, cluster_fails = 0;
 
 int cluster_of(const cudaLaunchConfig_t* c) {
@@ -29,6 +31,10 @@ int fake_attribute_changes() {
     std::lock_guard<std::mutex> g(lock);
     return changes;
 }
+size_t fake_copied_bytes() {
+    std::lock_guard<std::mutex> g(lock);
+    return copied;
+}
 void fake_cluster_limit(int c) { cluster_limit = c; }
 void fake_cluster_fails(int on) { cluster_fails = on; }
 
@@ -41,6 +47,16 @@ cudaError_t __wrap_cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int 
         limit[f] = v;
     }
     return __real_cudaFuncSetAttribute(f, a, v);
+}
+
+cudaError_t __real_cudaMemcpyAsync(void*, const void*, size_t, cudaMemcpyKind, cudaStream_t);
+cudaError_t __wrap_cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind k,
+                                   cudaStream_t st) {
+    if (k == cudaMemcpyHostToDevice) {
+        std::lock_guard<std::mutex> g(lock);
+        copied += n;
+    }
+    return __real_cudaMemcpyAsync(d, s, n, k, st);
 }
 
 cudaError_t __real_cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void*, void**);

@@ -7,7 +7,8 @@ import sys
 from paper_1208_4247_gb300 import build
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-WRAPPED = ["cudaFuncSetAttribute", "cudaLaunchKernelExC", "cudaOccupancyMaxActiveClusters"]
+WRAPPED = ["cudaFuncSetAttribute", "cudaLaunchKernelExC", "cudaOccupancyMaxActiveClusters",
+           "cudaMemcpyAsync"]
 
 
 def link(path):

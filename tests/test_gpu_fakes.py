@@ -80,3 +80,21 @@ fake.fake_cluster_fails(0)
 print("ok", gmg.learned_loss_grad(w, e, 8)[0] > 0.0)
 """)
     assert out == ["ok True", "ERR_CUDA", "ERR_CUDA", "ok True"]
+
+
+def test_batch_tables_hold_what_the_cycle_takes(lib):
+    """The chunks of the plain sweeps belong to batches that sweep outside the
+    legs: V(1,1) weighted Jacobi, all of whose sweeps are the legs', is made
+    without them."""
+    out = fakes.run(lib, """
+fake.fake_copied_bytes.restype = ctypes.c_size_t
+got = []
+for nu in (1, 2):
+    a = fake.fake_copied_bytes()
+    with gmg.Batch([2, 3], [512, 64], nu1=nu, nu2=nu):
+        got.append(fake.fake_copied_bytes() - a)
+# the finest levels: 511 rows of 128 groups of 4 nodes, 63 * 63 rows of 16, in items
+# (24 bytes) of 256 groups
+print(got[0] > 0, got[1] - got[0] >= (511 * 128 + 63 * 63 * 16) // 256 * 24)
+""")
+    assert out == ["True True"]
