@@ -305,7 +305,9 @@ gmg_status gmg_learned_train(int d, int n, int steps, int batch, int pair_cycles
 typedef struct gmg_fft_s* gmg_fft;
 
 /* d = 2 or 3, n a power of two (2D up to 8192, 3D up to 1024); allocates
- * about 1.5 n^d doubles: work space and the eliminations' coefficients. */
+ * about 1.5 n^d doubles: work space and the eliminations' coefficients, which
+ * are computed here (3D: 0.7 ms at n = 256, 2.8 ms at 512), so a program that
+ * solves several times on one grid keeps the handle. */
 gmg_status gmg_fft_create(int d, int n, void* cuda_stream, gmg_fft* out);
 /* Section 2.3: u = A'^-1 h^2 f on the interior, 0 on the boundary (f, u
  * device pointers, layout above).  Synchronises the handle's stream.

@@ -633,10 +633,15 @@ gmg_status gmg_fft_create(int d, int n, void* cuda_stream, gmg_fft* out) {
         return fail(GMG_ERR_ALLOC, "cudaMalloc failed");
     if (h->plan.threads > 256 && allow_smem() != cudaSuccess)
         return fail(GMG_ERR_CUDA, "cudaFuncSetAttribute failed");
-    std::vector<double> t(4 * (size_t)n);
+    // cos and sin of the first octant (long double: every entry correctly rounded up
+    // to the rounding of a small argument), the other octants from it
+    std::vector<double> t(4 * (size_t)n), oct_c(n / 4 + 1), oct_s(n / 4 + 1);
+    for (int r = 0; r <= n / 4; ++r) {
+        const long double a = 3.14159265358979323846264338327950288L * r / n;
+        oct_c[r] = (double)cosl(a);
+        oct_s[r] = (double)sinl(a);
+    }
     for (int k = 0; k < 2 * n; ++k) {
-        // from the first octant, so that every entry is correctly rounded up to
-        // the rounding of a small argument
         const int oct = (int)((int64_t)4 * k / n), r = k - (int)((int64_t)oct * n / 4);
         double c, s;
         if (n < 4) {  // k multiples of pi/2
@@ -645,8 +650,7 @@ gmg_status gmg_fft_create(int d, int n, void* cuda_stream, gmg_fft* out) {
             s = sn[(k * (2 / n)) & 3];
         } else {
             const bool odd = oct & 1;  // measured back from the octant's end
-            const long double a = 3.14159265358979323846264338327950288L * (odd ? n / 4 - r : r) / n;
-            const double ca = (double)cosl(a), sa = (double)sinl(a);
+            const double ca = oct_c[odd ? n / 4 - r : r], sa = oct_s[odd ? n / 4 - r : r];
             const int quad = ((oct + 1) / 2) & 3;  // nearest multiple of pi/2, angle = quad pi/2 +- a
             const double sg = odd ? -1.0 : 1.0;
             const double cc[4] = {ca, -sg * sa, -ca, sg * sa}, ss[4] = {sg * sa, ca, -sg * sa, -ca};

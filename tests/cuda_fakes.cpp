@@ -1,9 +1,10 @@
-// Fakes of CUDA runtime calls, linked in front of the library's objects with
+// Fakes of CUDA runtime (and libm) calls, linked in front of the library's objects with
 // --wrap, for failures that no argument of the public entry points brings about:
 //
 //   fake_attribute_changes()  how often a kernel's shared-memory limit was set to
 //                             another value than before
 //   fake_copied_bytes()       bytes copied from host memory so far
+//   fake_long_sines()         calls of the long double sine, cosine (or both) so far
 //   fake_cluster_limit(c)     the device has no room for clusters of more than c
 //                             CTAs: the query answers 0, a launch fails
 //   fake_cluster_fails(on)    the launch of a cluster fails
@@ -15,7 +16,7 @@
 namespace {
 std::mutex lock;
 std::map<const void*, int> limit;
-size_t copied = 0;
+size_t copied = 0, long_sines = 0;
 int changes = 0, cluster_limit = 1 << 30, cluster_fails = 0;
 
 int cluster_of(const cudaLaunchConfig_t* c) {
@@ -35,6 +36,7 @@ size_t fake_copied_bytes() {
     std::lock_guard<std::mutex> g(lock);
     return copied;
 }
+size_t fake_long_sines() { return long_sines; }
 void fake_cluster_limit(int c) { cluster_limit = c; }
 void fake_cluster_fails(int on) { cluster_fails = on; }
 
@@ -47,6 +49,22 @@ cudaError_t __wrap_cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int 
         limit[f] = v;
     }
     return __real_cudaFuncSetAttribute(f, a, v);
+}
+
+long double __real_sinl(long double);
+long double __real_cosl(long double);
+void __real_sincosl(long double, long double*, long double*);
+long double __wrap_sinl(long double x) {
+    ++long_sines;
+    return __real_sinl(x);
+}
+long double __wrap_cosl(long double x) {
+    ++long_sines;
+    return __real_cosl(x);
+}
+void __wrap_sincosl(long double x, long double* s, long double* c) {
+    ++long_sines;
+    __real_sincosl(x, s, c);
 }
 
 cudaError_t __real_cudaMemcpyAsync(void*, const void*, size_t, cudaMemcpyKind, cudaStream_t);

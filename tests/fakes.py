@@ -8,7 +8,7 @@ from paper_1208_4247_gb300 import build
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 WRAPPED = ["cudaFuncSetAttribute", "cudaLaunchKernelExC", "cudaOccupancyMaxActiveClusters",
-           "cudaMemcpyAsync"]
+           "cudaMemcpyAsync", "sinl", "cosl", "sincosl"]
 
 
 def link(path):
@@ -19,7 +19,7 @@ def link(path):
     if not all(os.path.exists(o) for o in objs):
         build.build(force=True)
     r = subprocess.run([build.nvcc(), "-shared", *build.ARCH, "-Xcompiler", "-fPIC", "-o", path,
-                        os.path.join(HERE, "cuda_fakes.cpp"), *objs, "-lcudart",
+                        os.path.join(HERE, "cuda_fakes.cpp"), *objs, "-lcudart", "-lm",
                         *[x for w in WRAPPED for x in ("-Xlinker", f"--wrap={w}")]],
                        capture_output=True, text=True)
     assert r.returncode == 0, r.stdout + r.stderr

@@ -98,3 +98,16 @@ for nu in (1, 2):
 print(got[0] > 0, got[1] - got[0] >= (511 * 128 + 63 * 63 * 16) // 256 * 24)
 """)
     assert out == ["True True"]
+
+
+def test_direct_solver_takes_one_octant_of_sines(lib):
+    """The angles of a plan's table are those of one octant, n/4 + 1 of them (a
+    sine and a cosine each, in software on Arm)."""
+    out = fakes.run(lib, """
+fake.fake_long_sines.restype = ctypes.c_size_t
+for d, n in [(2, 4096), (3, 64), (2, 4), (2, 2)]:
+    a = fake.fake_long_sines()
+    with gmg.FFTSolver(d, n):
+        print(0 < fake.fake_long_sines() - a <= 2 * (n // 4 + 1))
+""")
+    assert out == ["True"] * 4
