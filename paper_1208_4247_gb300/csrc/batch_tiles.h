@@ -39,6 +39,9 @@ inline std::vector<Rows> rows_up(int n, int R) {
     return v;
 }
 
+// What the 3D legs are compiled for (launch bounds, shared memory).
+constexpr int kLegThreads = 512;
+
 // Threads of a 3D leg's CTA: n / 4 lanes per row (at most 32) times the pairs
 // of rows.  Levels up to n = 64 are one tile; above, the number of warps (one
 // pair of rows each) that holds the fewest rows in all, the halo rows of the
@@ -47,10 +50,10 @@ inline std::vector<Rows> rows_up(int n, int R) {
 inline int leg_threads(int n, bool down) {
     if (n <= 16) return 32;
     if (n <= 32) return 128;
-    if (n <= 64) return 512;
+    if (n <= 64) return kLegThreads;
     int best = 0;
     int64_t cost = 0;
-    for (int w = 16; w >= 12; --w) {
+    for (int w = kLegThreads / 32; w >= 12; --w) {
         const int64_t c = (int64_t)2 * w * (down ? rows_down(n, 2 * w) : rows_up(n, 2 * w)).size();
         if (!best || c < cost) {
             best = w;

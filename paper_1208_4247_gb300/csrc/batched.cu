@@ -329,7 +329,7 @@ __device__ inline void fw_row(float* acc, float l, const float* r, float w) {
 // level / on its coarser levels and is not read.  clear: write u_c = 0 (the
 // coarse level reads it); the one unknown of an n = 2 grid gets u_c = q_c.
 template <typename T, bool SWEEP>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(kLegThreads, 1)
     k_down3(const Tile* __restrict__ tiles, int ntiles, const BSolve* __restrict__ sv,
             const BLevel* __restrict__ lv, const T* __restrict__ pool_in, T* __restrict__ pool_out,
             const int* __restrict__ active, int src, int dst, int zero, int clear, float omega) {
@@ -578,7 +578,7 @@ __device__ inline void widen3(float2 a, int lanes, bool last, float* c) {
 // ccur).  The corners a fine node lies between are added in k_prolong's order
 // (x, then y, then z), so the plane above is added value by value.
 template <typename T>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(kLegThreads, 1)
     k_up3(const Tile* __restrict__ tiles, int ntiles, const BSolve* __restrict__ sv,
           const BLevel* __restrict__ lv, const T* __restrict__ pool_in, T* __restrict__ pool_out,
           const int* __restrict__ active, int src, int dst, int ccur, float omega) {
@@ -1312,7 +1312,7 @@ cudaError_t leg_occupancy(gmg_batch b) {
     const bool sweep = !rbgs && b->cfg.nu1 >= 1;
     auto d3 = sweep ? k_down3<T, true> : k_down3<T, false>;
     auto d2 = sweep ? k_down2<T, true> : k_down2<T, false>;
-    cudaError_t e = cudaFuncSetAttribute(d3, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 512);
+    cudaError_t e = cudaFuncSetAttribute(d3, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * kLegThreads);
     auto occ = [&](auto k, int threads, int smem, int& warps) {
         int n = 0;
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem);
