@@ -18,11 +18,11 @@
 // (about 14 instructions per value at n = 256; a complex FFT of the odd
 // extension, length 2n, takes about 35, the real one of length 2n that a
 // library offers the same again in gathers and scatters).  The elimination
-// along the last axis takes 3 where the two transforms and the division by
+// along the last axis takes 4 where the two transforms and the division by
 // the eigenvalues would take about 30.
 // 3D 257^3: 14.94 ms with length-2n library transforms of the odd extension
-// on all three axes, 2.16 ms with these kernels (0.50 ms a
-// transform of one axis at 84% of the FP64 pipe, 0.13 ms the eliminations).
+// on all three axes, 2.19 ms with these kernels (0.50 ms a
+// transform of one axis at 84% of the FP64 pipe, 0.15 ms the eliminations).
 #include <algorithm>
 #include <cmath>
 #include <string>
@@ -341,15 +341,19 @@ __global__ void __launch_bounds__(THREADS) k_dst_y(double* __restrict__ w, int64
 // coefficients): c_1 = 1/(2+lambda), c_k = 1/(2+lambda - c_{k-1}) serve both
 // halves, v'_k = (s d_k + v'_{k-1}) c_k, the middle value takes 1/(2+lambda -
 // 2 c_{n/2-1}), and each half substitutes back v_k = v'_k + c_k v_{k+1}.
-// The coefficients are a table of the plan (one row per k = 1..n/2, the last
-// one the middle's), in closed form: with r + 1/r = 2 + lambda, r < 1,
+// With r + 1/r = 2 + lambda, r < 1, in closed form
 //     c_k = 1 - e_k,  e_k = (1-r)(1 + r^{2k+1}) / (1 - r^{2k+2}),
 //     1 - r = sqrt(lambda + lambda^2/4) - lambda/2.
-// r and its powers are double-double.  An error that all c_k of a line share
-// enters the solution 1/(1-r) times over, so they have to be as good as
-// correctly rounded: the recurrence in double (c_k = 1/(2 + lambda - c_{k-1}),
-// or e_k = t/(1+t), t = lambda + e_{k-1}, free of cancellation) cost 2D 4097^2
-// a relative 1e-14, these 5e-15 like the transforms.
+// A table of the plan holds e_k (one row per k = 1..n/2, the last one the middle's
+// coefficient), formed with r and its powers in double-double.  The steps take
+// c_k v as v - e_k v: an error that the c_k of a line share enters its solution
+// 2/(1-r) times over, and where r^{2k} is below the last bit all of them share
+// the rounding of r to double; e_k, of the size of 1 - r, brings none that counts.
+// Error against the exact solution of the system, smooth f (uniform f): 2D 257^2
+// 2.9e-16 (4.3e-16), with a table of c_k 6.7e-16 (5.2e-16), by transforms of both
+// axes 4.1e-16 (4.2e-16); 2049^2 4.6e-16 (7.0e-16), 11.6e-16 (18.4e-16), 6.0e-16
+// (9.6e-16); 3D 257^3 3.7e-16 (5.0e-16), 3.9e-16 (5.2e-16), 5.8e-16 (5.5e-16).  The
+// recurrence of c_k or e_k in double is worse still (4097^2: 1e-14).
 struct DD {
     double h, l;
 };
@@ -402,17 +406,20 @@ __global__ void __launch_bounds__(128) k_coeffs(double* __restrict__ c, int d, i
         return e1.h * num.h / den.h;
     };
     if (power.h == 0.0) {
-        const double ck = r.h;
-        for (int k = k0; k < k1; ++k) c[(int64_t)k * lines + l] = ck;
+        for (int k = k0; k < k1; ++k) c[(int64_t)k * lines + l] = e1.h;
     } else {
         for (int k = k0; k < k1; ++k) {
             power = dd_mul(power, r2);  // r^(2k+1)
-            c[(int64_t)k * lines + l] = 1.0 - e_of(power);
+            c[(int64_t)k * lines + l] = e_of(power);
         }
     }
     // the middle: 2 + lambda - 2 c = lambda + 2 e, k = n/2 - 1
     if (k1 == n / 2) c[(int64_t)k1 * lines + l] = 1.0 / (lambda + 2.0 * e_of(power));
 }
+
+// c v and c v + d with c = 1 - e
+__device__ inline double times_c(double v, double e) { return fma(-e, v, v); }
+__device__ inline double times_c_plus(double v, double e, double d) { return v + fma(-e, v, d); }
 
 // `count` steps v[k dv] -> f(v[k dv], c[k dc]), k = 0.. ; the operands of kB
 // steps are loaded together.  STORE: f's value replaces v[k dv].
@@ -439,8 +446,9 @@ __device__ inline void chain(double* __restrict__ v, int64_t dv, const double* _
 
 // 3D: one thread per half line; x along the lanes, threadIdx.y the half (0:
 // from k = 1 up, 1: from k = n-1 down), threadIdx.z one of the CTA's rows.
-// 3 FP64 instructions and (with the coefficients, read twice) 40 bytes per
-// node: 126 us at 257^3, 76% of the FP64 pipe.
+// 4 FP64 instructions and (with the coefficients, read twice) 40 bytes per
+// node: 151 us at 257^3, 87% of the FP64 pipe (a table of c_k: 3 instructions,
+// 125 us).
 __global__ void __launch_bounds__(256) k_lines(double* __restrict__ w, const double* __restrict__ c,
                                                int n, int64_t step, double scale) {
     __shared__ double tip[4][2][32];
@@ -456,7 +464,7 @@ __global__ void __launch_bounds__(256) k_lines(double* __restrict__ w, const dou
     double prev = 0.0, dm = 0.0;
     if (in) {
         chain<true>(v + dir, dir, cl + step, step, m - 1,
-                    [&](double d, double ck) { return prev = fma(scale, d, prev) * ck; });
+                    [&](double d, double e) { return prev = times_c(fma(scale, d, prev), e); });
         tip[threadIdx.z][half][threadIdx.x] = prev;
         dm = v[m * dir];  // the same entry for both halves, read before it is replaced
     }
@@ -467,7 +475,7 @@ __global__ void __launch_bounds__(256) k_lines(double* __restrict__ w, const dou
            cl[m * step];
     if (half == 0) v[m * dir] = prev;
     chain<true>(v + (m - 1) * dir, -dir, cl + (m - 1) * step, -step, m - 1,
-                [&](double d, double ck) { return prev = fma(ck, prev, d); });
+                [&](double d, double e) { return prev = times_c_plus(prev, e, d); });
 }
 
 // 2D has only n - 1 lines, too few for their chains (192 cycles of dependent
@@ -475,8 +483,9 @@ __global__ void __launch_bounds__(256) k_lines(double* __restrict__ w, const dou
 // thread each.  Both recurrences are linear in what flows into a piece, so a
 // first pass over the piece with inflow 0 gives its outflow t and the factor
 // p = prod c_k of its inflow, the inflows follow from those, and a second
-// pass stores the values.  7 instructions per node instead of 3, a chain 1/16
-// as long: 4097^2 578 -> 318 us, 257^2 33 -> 12 us.
+// pass stores the values.  9 instructions per node instead of 4, a chain 1/16
+// as long: 356 us at 4097^2, 12.7 at 257^2 (with a table of c_k 319 and 12.0, one
+// piece a line 578 and 33).
 // X columns to a CTA: 16 (128-byte rows) where that makes enough CTAs, else 8.
 constexpr int kC = 16;
 template <int X>
@@ -495,9 +504,9 @@ __global__ void __launch_bounds__(2 * X * kC) k_lines_2d(double* __restrict__ w,
     const double* cl = c + x;
     double t = 0.0, p = 1.0, dm = 0.0;
     if (in) {
-        chain<false>(v + k0 * dir, dir, cl + k0 * step, step, count, [&](double d, double ck) {
-            p *= ck;
-            return t = fma(scale, d, t) * ck;
+        chain<false>(v + k0 * dir, dir, cl + k0 * step, step, count, [&](double d, double e) {
+            p = times_c(p, e);
+            return t = times_c(fma(scale, d, t), e);
         });
         dm = v[m * dir];  // read before it is replaced
     }
@@ -516,11 +525,11 @@ __global__ void __launch_bounds__(2 * X * kC) k_lines_2d(double* __restrict__ w,
     if (in) {
         mid = (fma(scale, dm, tip[0]) + tip[1]) * cl[m * step];
         chain<true>(v + k0 * dir, dir, cl + k0 * step, step, count,
-                    [&](double d, double ck) { return prev = fma(scale, d, prev) * ck; });
+                    [&](double d, double e) { return prev = times_c(fma(scale, d, prev), e); });
         // back substitution from the piece's far end
         t = 0.0;
         chain<false>(v + (k0 + count - 1) * dir, -dir, cl + (k0 + count - 1) * step, -step, count,
-                     [&](double d, double ck) { return t = fma(ck, t, d); });
+                     [&](double d, double e) { return t = times_c_plus(t, e, d); });
     }
     __syncthreads();
     out[half][piece][tx] = t;
@@ -530,7 +539,7 @@ __global__ void __launch_bounds__(2 * X * kC) k_lines_2d(double* __restrict__ w,
     for (int i = kC - 1; i > piece; --i) prev = fma(fac[half][i][tx], prev, out[half][i][tx]);
     if (half == 0 && piece == 0) v[m * dir] = mid;
     chain<true>(v + (k0 + count - 1) * dir, -dir, cl + (k0 + count - 1) * step, -step, count,
-                [&](double d, double ck) { return prev = fma(ck, prev, d); });
+                [&](double d, double e) { return prev = times_c_plus(prev, e, d); });
 }
 
 }  // namespace
