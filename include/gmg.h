@@ -116,13 +116,14 @@ gmg_status gmg_config_init(gmg_config* cfg, int d, int n);
  * layout instead of two half sweeps on the colour-split one (same results
  * bit for bit; slower on GB300, see the design notes).  GMG_TAIL_N=m sets the
  * largest level n handled by the single-CTA tail launch (1 turns the tail
- * off; default 32 in 2D and 8 in 3D, where red-black handles run the levels
- * from n = 32, FP64 16, down as one 16-CTA cluster instead if the device has
- * room for one, asked at create); results are the same bit for bit.
+ * off; default 32 in 2D, or 16 under levels with leg kernels, and 8 in 3D,
+ * where red-black handles run the levels from n = 32, FP64 16, down as one
+ * 16-CTA cluster instead if the device has room for one, asked at create);
+ * results are the same bit for bit.
  * GMG_RB_WALK=0 (read once per process) replaces the diagonal-walker FP64 3D
- * half sweeps, red-only residuals and norms (levels 128 <= n <= 512) by row
- * kernels; results are the same bit for bit.  GMG_NORM_AHEAD=0 (read once
- * per process) keeps the stopping-test norm of the plain red-black form a
+ * half sweeps, residuals and norms (levels 128 <= n <= 512) by row kernels; u is
+ * the same bit for bit, the norms agree to rounding (another order of the sum).
+ * GMG_NORM_AHEAD=0 (read once per process) keeps the stopping-test norm of the plain red-black form a
  * separate kernel instead of fusing it with the next cycle's first red half
  * sweep (3D levels 128 <= n <= 512; a solve that stops undoes that sweep);
  * u and the cycle count are the same bit for bit, the norms agree to
@@ -145,8 +146,9 @@ gmg_status gmg_config_init(gmg_config* cfg, int d, int n);
  * GMG_FUSED_LEGS=0/1 turns the fused leg kernels off / on for every FP32
  * and double-float level that takes them, and those of the 2D FP64 levels up to
  * 512 (default: FP32 levels n >= 256, 2D FP64 levels);
- * GMG_LEG_NMIN / GMG_LEG_NMAX bound the level sizes; results are the same bit
- * for bit.  GMG_GRID_TAIL_N=m runs the levels with n <= m (red-black) and
+ * GMG_LEG_NMIN (3D) / GMG_LEG_NMAX bound the level sizes, and GMG_LEG_SEGS=k
+ * (read when a handle's cycle is captured) has the 3D legs walk the z range in k
+ * pieces; results are the same bit for bit.  GMG_GRID_TAIL_N=m runs the levels with n <= m (red-black) and
  * all smaller ones as one cooperative launch with grid barriers between the
  * steps, the levels with n <= GMG_GRID_TAIL_CTA_N (default 8) in one CTA of
  * it (default off: slower than the per-level kernels on GB300);

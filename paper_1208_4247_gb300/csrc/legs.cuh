@@ -1,5 +1,7 @@
 // Fused leg kernels of the V-cycle (Algorithm 1) for the 3D red-black
-// inner hierarchies (FP32 and double-float storage, colour-split layout):
+// inner hierarchies (colour-split layout; the library runs them for double-float
+// storage, FP32 levels take legs_reg.cu and the float form here is compiled by
+// the CTA algorithm's host check only):
 //
 //   down leg  S half sweeps (alternating colours, the last one black), the
 //             red-only residual and the full-weighting restriction of it:

@@ -109,7 +109,7 @@ __device__ int smooth(const Box& B, double* u, double* u2, const double* q, int 
 }
 
 // Load the box's nodes of arrays a (and b) of a dense level n; zero outside the
-// grid.  Eight nodes per thread in flight.
+// grid.  Four nodes per thread in flight.
 __device__ inline void load_box(const Box& B, int n, const double* __restrict__ a, double* sa,
                                 const double* __restrict__ b, double* sb) {
     constexpr int U = 4;
