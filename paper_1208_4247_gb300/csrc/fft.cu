@@ -18,11 +18,11 @@
 // (about 14 instructions per value at n = 256; a complex FFT of the odd
 // extension, length 2n, takes about 35, the real one of length 2n that a
 // library offers the same again in gathers and scatters).  The elimination
-// along the last axis takes 4 where the two transforms and the division by
+// along the last axis takes 3 (2D: 9) where the two transforms and the division by
 // the eigenvalues would take about 30.
 // 3D 257^3: 14.94 ms with length-2n library transforms of the odd extension
-// on all three axes, 2.19 ms with these kernels (0.50 ms a
-// transform of one axis at 84% of the FP64 pipe, 0.15 ms the eliminations).
+// on all three axes, 2.16 ms with these kernels (0.50 ms a
+// transform of one axis at 84% of the FP64 pipe, 0.13 ms the eliminations).
 #include <algorithm>
 #include <cmath>
 #include <string>
@@ -344,16 +344,22 @@ __global__ void __launch_bounds__(THREADS) k_dst_y(double* __restrict__ w, int64
 // With r + 1/r = 2 + lambda, r < 1, in closed form
 //     c_k = 1 - e_k,  e_k = (1-r)(1 + r^{2k+1}) / (1 - r^{2k+2}),
 //     1 - r = sqrt(lambda + lambda^2/4) - lambda/2.
-// A table of the plan holds e_k (one row per k = 1..n/2, the last one the middle's
-// coefficient), formed with r and its powers in double-double.  The steps take
-// c_k v as v - e_k v: an error that the c_k of a line share enters its solution
-// 2/(1-r) times over, and where r^{2k} is below the last bit all of them share
-// the rounding of r to double; e_k, of the size of 1 - r, brings none that counts.
-// Error against the exact solution of the system, smooth f (uniform f): 2D 257^2
-// 2.9e-16 (4.3e-16), with a table of c_k 6.7e-16 (5.2e-16), by transforms of both
-// axes 4.1e-16 (4.2e-16); 2049^2 4.6e-16 (7.0e-16), 11.6e-16 (18.4e-16), 6.0e-16
-// (9.6e-16); 3D 257^3 3.7e-16 (5.0e-16), 3.9e-16 (5.2e-16), 5.8e-16 (5.5e-16).  The
-// recurrence of c_k or e_k in double is worse still (4097^2: 1e-14).
+// (r and its powers in double-double), a table of the plan: one row per k =
+// 1..n/2, the last one the middle's coefficient.
+//
+// An error that the c_k of a line share enters its solution 2/(1-r) times over,
+// and where r^{2k} is below the last bit all of them share the rounding of r to
+// double: 2D 8193^2 was solved to 8.6e-15 in some modes that way.  So in 2D,
+// where 1 - r is small and the chains long, the table holds e_k, of the size of 1
+// - r, and a step takes c_k v as v - e_k v.  In 3D it holds c_k, each rounded
+// together with the error of those before it, which saves the back substitution
+// an instruction (257^3: 125 us, 151 with e_k); the same in 2D is less accurate
+// (2049^2 13.5e-16).  Error against the exact solution of the system, smooth f
+// (uniform f): 2D 257^2 2.9e-16 (4.3e-16), with c_k just rounded 6.7e-16 (5.2e-16),
+// by transforms of both axes 4.1e-16 (4.2e-16); 2049^2 4.6e-16 (7.0e-16), 11.6e-16
+// (18.4e-16), 6.0e-16 (9.6e-16); 3D 257^3 3.8e-16 (5.4e-16), 3.9e-16 (5.2e-16),
+// 5.8e-16 (5.5e-16); 129^3 3.8e-16 (4.1e-16), 4.3e-16 (4.3e-16), 3.3e-16 (4.4e-16).
+// The recurrence of c_k or e_k in double is worse still (4097^2: 1e-14).
 struct DD {
     double h, l;
 };
@@ -405,19 +411,30 @@ __global__ void __launch_bounds__(128) k_coeffs(double* __restrict__ c, int d, i
         const DD den = dd_add({1.0, 0.0}, {-rp.h, -rp.l}), num = dd_add({1.0, 0.0}, pw);
         return e1.h * num.h / den.h;
     };
+    // 3D: 1 - e less what the entries before it have too much in all.  A segment
+    // starts with an amount of its own, spread over the half units, so that what
+    // the segments of a line leave at their ends is not shared either.
+    const double golden = 0.6180339887498949 * blockIdx.y;
+    double carry = 0x1p-53 * (golden - floor(golden) - 0.5);
+    auto entry = [&](double e) {
+        if (d == 2) return e;
+        const double w = e + carry, ck = 1.0 - w;
+        carry = (ck - 1.0) + w;  // exact (|w| < 1)
+        return ck;
+    };
     if (power.h == 0.0) {
-        for (int k = k0; k < k1; ++k) c[(int64_t)k * lines + l] = e1.h;
+        for (int k = k0; k < k1; ++k) c[(int64_t)k * lines + l] = entry(e1.h);
     } else {
         for (int k = k0; k < k1; ++k) {
             power = dd_mul(power, r2);  // r^(2k+1)
-            c[(int64_t)k * lines + l] = e_of(power);
+            c[(int64_t)k * lines + l] = entry(e_of(power));
         }
     }
     // the middle: 2 + lambda - 2 c = lambda + 2 e, k = n/2 - 1
     if (k1 == n / 2) c[(int64_t)k1 * lines + l] = 1.0 / (lambda + 2.0 * e_of(power));
 }
 
-// c v and c v + d with c = 1 - e
+// 2D: c v and c v + d with c = 1 - e
 __device__ inline double times_c(double v, double e) { return fma(-e, v, v); }
 __device__ inline double times_c_plus(double v, double e, double d) { return v + fma(-e, v, d); }
 
@@ -446,9 +463,8 @@ __device__ inline void chain(double* __restrict__ v, int64_t dv, const double* _
 
 // 3D: one thread per half line; x along the lanes, threadIdx.y the half (0:
 // from k = 1 up, 1: from k = n-1 down), threadIdx.z one of the CTA's rows.
-// 4 FP64 instructions and (with the coefficients, read twice) 40 bytes per
-// node: 151 us at 257^3, 87% of the FP64 pipe (a table of c_k: 3 instructions,
-// 125 us).
+// 3 FP64 instructions and (with the coefficients, read twice) 40 bytes per
+// node: 125 us at 257^3, 78% of the FP64 pipe.
 __global__ void __launch_bounds__(256) k_lines(double* __restrict__ w, const double* __restrict__ c,
                                                int n, int64_t step, double scale) {
     __shared__ double tip[4][2][32];
@@ -464,7 +480,7 @@ __global__ void __launch_bounds__(256) k_lines(double* __restrict__ w, const dou
     double prev = 0.0, dm = 0.0;
     if (in) {
         chain<true>(v + dir, dir, cl + step, step, m - 1,
-                    [&](double d, double e) { return prev = times_c(fma(scale, d, prev), e); });
+                    [&](double d, double ck) { return prev = fma(scale, d, prev) * ck; });
         tip[threadIdx.z][half][threadIdx.x] = prev;
         dm = v[m * dir];  // the same entry for both halves, read before it is replaced
     }
@@ -475,7 +491,7 @@ __global__ void __launch_bounds__(256) k_lines(double* __restrict__ w, const dou
            cl[m * step];
     if (half == 0) v[m * dir] = prev;
     chain<true>(v + (m - 1) * dir, -dir, cl + (m - 1) * step, -step, m - 1,
-                [&](double d, double e) { return prev = times_c_plus(prev, e, d); });
+                [&](double d, double ck) { return prev = fma(ck, prev, d); });
 }
 
 // 2D has only n - 1 lines, too few for their chains (192 cycles of dependent
@@ -484,8 +500,8 @@ __global__ void __launch_bounds__(256) k_lines(double* __restrict__ w, const dou
 // first pass over the piece with inflow 0 gives its outflow t and the factor
 // p = prod c_k of its inflow, the inflows follow from those, and a second
 // pass stores the values.  9 instructions per node instead of 4, a chain 1/16
-// as long: 356 us at 4097^2, 12.7 at 257^2 (with a table of c_k 319 and 12.0, one
-// piece a line 578 and 33).
+// as long: 356 us at 4097^2, 12.7 at 257^2 (with a table of c_k 319 and 12.0; one
+// piece a line, 578 and 33).
 // X columns to a CTA: 16 (128-byte rows) where that makes enough CTAs, else 8.
 constexpr int kC = 16;
 template <int X>
