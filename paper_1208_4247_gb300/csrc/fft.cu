@@ -349,13 +349,14 @@ __global__ void __launch_bounds__(THREADS) k_dst_y(double* __restrict__ w, int64
 //
 // An error that the c_k of a line share enters its solution 2/(1-r) times over,
 // and where r^{2k} is below the last bit all of them share the rounding of r to
-// double: 2D 8193^2 was solved to 8.6e-15 in some modes that way.  So in 2D,
-// where 1 - r is small and the chains long, the table holds e_k, of the size of 1
-// - r, and a step takes c_k v as v - e_k v.  In 3D it holds c_k, each rounded
-// together with the error of those before it, which saves the back substitution
-// an instruction (257^3: 125 us, 151 with e_k); the same in 2D is less accurate
-// (2049^2 13.5e-16).  Error against the exact solution of the system, smooth f
-// (uniform f): 2D 257^2 2.9e-16 (4.3e-16), with c_k just rounded 6.7e-16 (5.2e-16),
+// double: 2D 8193^2 was solved to 8.6e-15 in some modes that way.  So in 2D from n =
+// 512 up, where 1 - r is small and the chains long, the table holds e_k, of the
+// size of 1 - r, and a step takes c_k v as v - e_k v.  Else it holds c_k, each
+// rounded together with the error of those before it, which saves the back
+// substitution an instruction (257^3: 125 us, 151 with e_k; 2D 257^2 12.0, 12.7)
+// and is as accurate up to there, but not above (2D 513^2 5.5e-16 against 4.5,
+// 2049^2 13.5e-16 against 7.0).  Error against the exact solution of the system, smooth f
+// (uniform f): 2D 257^2 3.6e-16 (3.3e-16), with c_k just rounded 6.7e-16 (5.2e-16),
 // by transforms of both axes 4.1e-16 (4.2e-16); 2049^2 4.6e-16 (7.0e-16), 11.6e-16
 // (18.4e-16), 6.0e-16 (9.6e-16); 3D 257^3 3.8e-16 (5.4e-16), 3.9e-16 (5.2e-16),
 // 5.8e-16 (5.5e-16); 129^3 3.8e-16 (4.1e-16), 4.3e-16 (4.3e-16), 3.3e-16 (4.4e-16).
@@ -375,6 +376,8 @@ __device__ inline DD dd_mul(DD a, DD b) {
     const double p = a.h * b.h;
     return dd_sum(p, fma(a.h, b.h, -p) + fma(a.h, b.l, a.l * b.h));
 }
+// The table holds e_k (2D, long chains), else c_k.
+__host__ __device__ inline bool table_of_e(int d, int n) { return d == 2 && n > 256; }
 // One thread per line and kSeg coefficients.
 constexpr int kSeg = 16;
 __global__ void __launch_bounds__(128) k_coeffs(double* __restrict__ c, int d, int n) {
@@ -411,13 +414,13 @@ __global__ void __launch_bounds__(128) k_coeffs(double* __restrict__ c, int d, i
         const DD den = dd_add({1.0, 0.0}, {-rp.h, -rp.l}), num = dd_add({1.0, 0.0}, pw);
         return e1.h * num.h / den.h;
     };
-    // 3D: 1 - e less what the entries before it have too much in all.  A segment
+    // c_k tables: 1 - e less what the entries before it have too much in all.  A segment
     // starts with an amount of its own, spread over the half units, so that what
     // the segments of a line leave at their ends is not shared either.
     const double golden = 0.6180339887498949 * blockIdx.y;
     double carry = 0x1p-53 * (golden - floor(golden) - 0.5);
     auto entry = [&](double e) {
-        if (d == 2) return e;
+        if (table_of_e(d, n)) return e;
         const double w = e + carry, ck = 1.0 - w;
         carry = (ck - 1.0) + w;  // exact (|w| < 1)
         return ck;
@@ -434,9 +437,15 @@ __global__ void __launch_bounds__(128) k_coeffs(double* __restrict__ c, int d, i
     if (k1 == n / 2) c[(int64_t)k1 * lines + l] = 1.0 / (lambda + 2.0 * e_of(power));
 }
 
-// 2D: c v and c v + d with c = 1 - e
-__device__ inline double times_c(double v, double e) { return fma(-e, v, v); }
-__device__ inline double times_c_plus(double v, double e, double d) { return v + fma(-e, v, d); }
+// c v and c v + d from the table's entry x: c = x, or (E) c = 1 - x
+template <bool E>
+__device__ inline double times_c(double v, double x) {
+    return E ? fma(-x, v, v) : v * x;
+}
+template <bool E>
+__device__ inline double times_c_plus(double v, double x, double d) {
+    return E ? v + fma(-x, v, d) : fma(x, v, d);
+}
 
 // `count` steps v[k dv] -> f(v[k dv], c[k dc]), k = 0.. ; the operands of kB
 // steps are loaded together.  STORE: f's value replaces v[k dv].
@@ -499,12 +508,13 @@ __global__ void __launch_bounds__(256) k_lines(double* __restrict__ w, const dou
 // thread each.  Both recurrences are linear in what flows into a piece, so a
 // first pass over the piece with inflow 0 gives its outflow t and the factor
 // p = prod c_k of its inflow, the inflows follow from those, and a second
-// pass stores the values.  9 instructions per node instead of 4, a chain 1/16
-// as long: 356 us at 4097^2, 12.7 at 257^2 (with a table of c_k 319 and 12.0; one
-// piece a line, 578 and 33).
+// pass stores the values.  9 instructions per node instead of 4 (c_k: 7 of 3), a
+// chain 1/16 as long: 356 us at 4097^2, 12.0 at 257^2 (one piece a line: 578 and
+// 33 with a table of c_k, which would take 319 in pieces).
 // X columns to a CTA: 16 (128-byte rows) where that makes enough CTAs, else 8.
 constexpr int kC = 16;
-template <int X>
+// E: the table holds e_k (table_of_e)
+template <int X, bool E>
 __global__ void __launch_bounds__(2 * X * kC) k_lines_2d(double* __restrict__ w,
                                                       const double* __restrict__ c, int n,
                                                       double scale) {
@@ -521,8 +531,8 @@ __global__ void __launch_bounds__(2 * X * kC) k_lines_2d(double* __restrict__ w,
     double t = 0.0, p = 1.0, dm = 0.0;
     if (in) {
         chain<false>(v + k0 * dir, dir, cl + k0 * step, step, count, [&](double d, double e) {
-            p = times_c(p, e);
-            return t = times_c(fma(scale, d, t), e);
+            p = times_c<E>(p, e);
+            return t = times_c<E>(fma(scale, d, t), e);
         });
         dm = v[m * dir];  // read before it is replaced
     }
@@ -541,11 +551,11 @@ __global__ void __launch_bounds__(2 * X * kC) k_lines_2d(double* __restrict__ w,
     if (in) {
         mid = (fma(scale, dm, tip[0]) + tip[1]) * cl[m * step];
         chain<true>(v + k0 * dir, dir, cl + k0 * step, step, count,
-                    [&](double d, double e) { return prev = times_c(fma(scale, d, prev), e); });
+                    [&](double d, double e) { return prev = times_c<E>(fma(scale, d, prev), e); });
         // back substitution from the piece's far end
         t = 0.0;
         chain<false>(v + (k0 + count - 1) * dir, -dir, cl + (k0 + count - 1) * step, -step, count,
-                     [&](double d, double e) { return t = times_c_plus(t, e, d); });
+                     [&](double d, double e) { return t = times_c_plus<E>(t, e, d); });
     }
     __syncthreads();
     out[half][piece][tx] = t;
@@ -555,7 +565,7 @@ __global__ void __launch_bounds__(2 * X * kC) k_lines_2d(double* __restrict__ w,
     for (int i = kC - 1; i > piece; --i) prev = fma(fac[half][i][tx], prev, out[half][i][tx]);
     if (half == 0 && piece == 0) v[m * dir] = mid;
     chain<true>(v + (k0 + count - 1) * dir, -dir, cl + (k0 + count - 1) * step, -step, count,
-                [&](double d, double e) { return prev = times_c_plus(prev, e, d); });
+                [&](double d, double e) { return prev = times_c_plus<E>(prev, e, d); });
 }
 
 }  // namespace
@@ -717,9 +727,11 @@ gmg_status gmg_fft_solve(gmg_fft h, const double* f, double* u) {
         k_lines<<<dim3((n + 31) / 32, (n + 3) / 4), dim3(32, 2, 4), 0, s>>>(h->work, h->coeffs, n,
                                                                             wz, scale);
     else if (n >= 2048)
-        k_lines_2d<16><<<n / 16, dim3(16, 2 * kC), 0, s>>>(h->work, h->coeffs, n, scale);
+        k_lines_2d<16, true><<<n / 16, dim3(16, 2 * kC), 0, s>>>(h->work, h->coeffs, n, scale);
+    else if (table_of_e(d, n))
+        k_lines_2d<8, true><<<(n + 7) / 8, dim3(8, 2 * kC), 0, s>>>(h->work, h->coeffs, n, scale);
     else
-        k_lines_2d<8><<<(n + 7) / 8, dim3(8, 2 * kC), 0, s>>>(h->work, h->coeffs, n, scale);
+        k_lines_2d<8, false><<<(n + 7) / 8, dim3(8, 2 * kC), 0, s>>>(h->work, h->coeffs, n, scale);
     if (d == 3) dst_y(h);
     dst_x(h, h->work, wy, wz, u, m, mz, 1);
     GMG_CUDA_TRY(cudaGetLastError());
